@@ -344,7 +344,7 @@ static pv_status add_receptor(pv_context* ctx, pv_grid_set* set, const pv_recept
     Layout L;
     const size_t o_xyz = L.take<float>(3 * (size_t)n), o_el = L.take<uint8_t>(n), o_don = L.take<uint8_t>(n),
                  o_acc = L.take<uint8_t>(n), o_sorted = L.take<float4>(n),
-                 o_cof = L.take<int>(n), o_rank = L.take<int>(n), o_cnt = L.take<int>(n_cells),
+                 o_cof = L.take<int>(n), o_next = L.take<int>(n), o_head = L.take<int>(n_cells),
                  o_start = L.take<int>(n_cells + 1), o_tiles = L.take<int2>(tiles.size());
     char* w = (char*)dalloc(ctx, L.off);
     if (!w) return fail(ctx, PV_ERR_OOM, "grid scratch allocation failed");
@@ -371,14 +371,9 @@ static pv_status add_receptor(pv_context* ctx, pv_grid_set* set, const pv_recept
         e = cudaMemcpyAsync(w + o_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, ctx->stream);
     }
     if (e == cudaSuccess) {
-        stage = "receptor typing";
-        e = launch_receptor_type(xyz, el, don, acc, n, typed, ctx->stream);
-    }
-    if (e == cudaSuccess) {
-        stage = "receptor binning";
-        e = launch_receptor_bin(typed, n, flo, kCellEdge, cd, (int*)(w + o_cof),
-                                (int*)(w + o_rank), (int*)(w + o_cnt), (int*)(w + o_start),
-                                (float4*)(w + o_sorted), ctx->stream);
+        stage = "receptor typing and binning";
+        e = launch_receptor_prep(xyz, el, don, acc, n, flo, kCellEdge, cd, typed, (int*)(w + o_cof), (int*)(w + o_next),
+                                 (int*)(w + o_head), (int*)(w + o_start), (float4*)(w + o_sorted), ctx->stream);
     }
     if (e == cudaSuccess) {
         stage = "map build";

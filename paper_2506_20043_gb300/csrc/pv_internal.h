@@ -31,14 +31,14 @@ constexpr int kMaxTopK = 32;
 constexpr int kMaxMergeEntries = 8192;
 
 // ---- grid cache (pv_grid.cu) ----
-// XS typing of receptor atoms: typed[i] = (x, y, z, type as int bits).
-cudaError_t launch_receptor_type(const float* xyz, const uint8_t* el, const uint8_t* don,
-                                 const uint8_t* acc, int n, float4* typed, cudaStream_t s);
-// Binning into cubic cells of edge `cell` over the region lo + [0, cdims * cell) as CSR:
-// cell_start[n_cells + 1], sorted atoms by (cell, input index); atoms outside are dropped.
-cudaError_t launch_receptor_bin(const float4* typed, int n, const float lo[3], float cell,
-                                const int cdims[3], int* cell_of, int* rank, int* cell_count,
-                                int* cell_start, float4* sorted, cudaStream_t s);
+// XS typing of receptor atoms, typed[i] = (x, y, z, type as int bits), and their binning into cubic
+// cells of edge `cell` over the region lo + [0, cdims * cell): sorted holds them by cell, in input order
+// within a cell, cells consecutive along x (cell_start[c] .. cell_start[c + 1] for every cell but the
+// last of a row); atoms outside the region are typed but not binned. cell_of, next: [n], head: [cells],
+// cell_start: [cells + 1].
+cudaError_t launch_receptor_prep(const float* xyz, const uint8_t* el, const uint8_t* don, const uint8_t* acc, int n,
+                                 const float lo[3], float cell, const int cdims[3], float4* typed, int* cell_of,
+                                 int* next, int* head, int* cell_start, float4* sorted, cudaStream_t s);
 // Map build over a tile list (pocket, tile index); one CTA per 8 x 8 x 8 node tile.
 cudaError_t launch_grid_tiles(const float4* sorted, const int* cell_start, const float lo[3],
                               float cell, const int cdims[3], const PvPocket* pockets_dev,

@@ -34,9 +34,9 @@ constexpr size_t kOffAcc = align256(kOffDon + kMaxAtoms);
 constexpr size_t kOffTyped = align256(kOffAcc + kMaxAtoms);
 constexpr size_t kOffSorted = align256(kOffTyped + sizeof(float4) * kMaxAtoms);
 constexpr size_t kOffCellOf = align256(kOffSorted + sizeof(float4) * kMaxAtoms);
-constexpr size_t kOffRank = align256(kOffCellOf + sizeof(int) * kMaxAtoms);
-constexpr size_t kOffCount = align256(kOffRank + sizeof(int) * kMaxAtoms);
-constexpr size_t kOffStart = align256(kOffCount + sizeof(int) * kMaxCells);
+constexpr size_t kOffNext = align256(kOffCellOf + sizeof(int) * kMaxAtoms);
+constexpr size_t kOffHead = align256(kOffNext + sizeof(int) * kMaxAtoms);
+constexpr size_t kOffStart = align256(kOffHead + sizeof(int) * kMaxCells);
 constexpr size_t kOffTiles = align256(kOffStart + sizeof(int) * (kMaxCells + 1));
 constexpr size_t kOffPocket = align256(kOffTiles + sizeof(int2) * kMaxTiles);
 constexpr size_t kScratchBytes = align256(kOffPocket + sizeof(PvPocket));
@@ -175,13 +175,13 @@ extern "C" pv_status pv_build_grid_noalloc(pv_context* ctx, const pv_receptor* r
             fill_tiles_kernel<<<(int)((n_tiles + 255) / 256), 256, 0, stream>>>((int2*)(scratch + kOffTiles), (int)n_tiles);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = launch_receptor_type(xyz, el, don, acc, n, (float4*)(scratch + kOffTyped), stream);
-        // the cell counts are zeroed inside the binning step; every other array is fully
+        // the cell lists are emptied inside the binning step; every other array is fully
         // written before it is read, so what an earlier call left behind is never used
         if (e == cudaSuccess)
-            e = launch_receptor_bin((const float4*)(scratch + kOffTyped), n, flo, kCell, cd, (int*)(scratch + kOffCellOf),
-                                    (int*)(scratch + kOffRank), (int*)(scratch + kOffCount),
-                                    (int*)(scratch + kOffStart), (float4*)(scratch + kOffSorted), stream);
+            e = launch_receptor_prep(xyz, el, don, acc, n, flo, kCell, cd, (float4*)(scratch + kOffTyped),
+                                     (int*)(scratch + kOffCellOf), (int*)(scratch + kOffNext),
+                                     (int*)(scratch + kOffHead), (int*)(scratch + kOffStart),
+                                     (float4*)(scratch + kOffSorted), stream);
         uint64_t s_lo = 0, s_hi = 0;
         for (int t = 0; t < 8; ++t) s_lo |= (uint64_t)(uint8_t)slot[t] << (8 * t);
         for (int t = 0; t < 8; ++t) s_hi |= (uint64_t)(uint8_t)slot[8 + t] << (8 * t);

@@ -1,0 +1,49 @@
+"""Edges of the receptor binning of the grid cache, against the FP64 oracle's direct sums at sampled
+nodes (the grid tolerance of tests/_gpu.py): atom counts around a block's, boxes whose rows of binning
+cells are longer than a warp, receptors mostly outside every box, dense and far-away ones."""
+import numpy as np
+import pytest
+
+import oracle as O
+import pvsynth as S
+from tests import _gpu as G
+
+pytestmark = pytest.mark.gpu
+
+
+def _receptor(n, density, seed, shift=0.0):
+    r = S.make_receptor(n, seed, density=density)
+    return G.receptor32(S.Receptor(r.xyz + shift, r.element, r.donor, r.acceptor))
+
+
+def _box(center, size, spacing=0.375):
+    return G.box32(S.Box(np.asarray(center, float), np.asarray(size, float), spacing))
+
+
+CASES = {
+    "one atom": (_receptor(1, 0.05, 1), [_box((0.5, 0, 0), (4, 4, 4))]),
+    "127 atoms": (_receptor(127, 0.05, 2), [_box((0, 0, 0), (5, 7, 6))]),
+    "129 atoms, all types in one cell's reach": (_receptor(129, 0.8, 3), [_box((0, 0, 0), (3, 3, 3))]),
+    "dense": (_receptor(6000, 1.5, 4), [_box((0, 0, 0), (4.2, 4.9, 3.4))]),
+    "long rows": (_receptor(4000, 0.05, 5), [_box((-18, 0, 0), (6, 6, 6)), _box((80, 1, -60), (6, 6, 6)),
+                                             _box((10, 5, 5), (9, 3, 3))]),
+    "mostly outside": (_receptor(8000, 0.05, 6), [_box((24, 24, 24), (3, 3, 3))]),
+    "far away": (_receptor(1000, 0.05, 7, shift=1000.0), [_box((1000, 1002, 999), (6, 6, 6))]),
+    "coarse": (_receptor(3000, 0.05, 8), [_box((0, 0, 0), (40, 30, 22), 4.0)]),
+}
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_binned_receptor_gives_the_direct_sums(name):
+    rec, boxes = CASES[name]
+    types = [0, 1, 4, 9, 10]
+    gs = G.context().build_grids(rec, boxes, types)
+    rt = O.xs_type_receptor(rec)
+    rng = np.random.default_rng(11)
+    for p, b in enumerate(boxes):
+        _, dims = O.grid_geometry(b)
+        idx = np.concatenate([rng.integers(0, dims, size=(60, 3)), [dims - 1, np.zeros(3, int)]])
+        for t in types:
+            ref = np.array([O.grid_node_value(rec, rt, b, t, *i) for i in idx])
+            got = gs.read_map(p, t)[idx[:, 2], idx[:, 1], idx[:, 0]]
+            assert G.close(got, ref).all(), (p, t, np.abs(got - ref).max())

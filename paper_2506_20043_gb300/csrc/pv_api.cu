@@ -299,13 +299,7 @@ static pv_status add_receptor(pv_context* ctx, pv_grid_set* set, const pv_recept
     }
     const long long n_cells = (long long)cd[0] * cd[1] * cd[2];
     if (n_cells > (1 << 24)) return fail(ctx, PV_ERR_ARG, "pocket boxes span too large a region");
-    // tiles
-    std::vector<int2> tiles;
     const int first = (int)set->pockets.size();
-    for (int p = 0; p < n_pockets; ++p) {
-        const int tx = (pk[p].dims[0] + 7) / 8, ty = (pk[p].dims[1] + 7) / 8, tz = (pk[p].dims[2] + 7) / 8;
-        for (int t = 0; t < tx * ty * tz; ++t) tiles.push_back(make_int2(first + p, t));
-    }
     // maps arena, and the typed receptor kept for direct rescoring of poses
     float* arena = (float*)dalloc(ctx, map_floats * sizeof(float));
     if (!arena) return fail(ctx, PV_ERR_OOM, "map allocation failed");
@@ -345,7 +339,7 @@ static pv_status add_receptor(pv_context* ctx, pv_grid_set* set, const pv_recept
     const size_t o_xyz = L.take<float>(3 * (size_t)n), o_el = L.take<uint8_t>(n), o_don = L.take<uint8_t>(n),
                  o_acc = L.take<uint8_t>(n), o_sorted = L.take<float4>(n),
                  o_cof = L.take<int>(n), o_next = L.take<int>(n), o_head = L.take<int>(n_cells),
-                 o_start = L.take<int>(n_cells + 1), o_tiles = L.take<int2>(tiles.size());
+                 o_start = L.take<int>(n_cells + 1);
     char* w = (char*)dalloc(ctx, L.off);
     if (!w) return fail(ctx, PV_ERR_OOM, "grid scratch allocation failed");
     const float* xyz = (const float*)r->xyz;
@@ -367,10 +361,6 @@ static pv_status add_receptor(pv_context* ctx, pv_grid_set* set, const pv_recept
         acc = (const uint8_t*)(w + o_acc);
     }
     if (e == cudaSuccess) {
-        stage = "tile table upload";
-        e = cudaMemcpyAsync(w + o_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, ctx->stream);
-    }
-    if (e == cudaSuccess) {
         stage = "receptor typing and binning";
         e = launch_receptor_prep(xyz, el, don, acc, n, flo, kCellEdge, cd, typed, (int*)(w + o_cof), (int*)(w + o_next),
                                  (int*)(w + o_head), (int*)(w + o_start), (float4*)(w + o_sorted), ctx->stream);
@@ -383,9 +373,9 @@ static pv_status add_receptor(pv_context* ctx, pv_grid_set* set, const pv_recept
         if (e == cudaSuccess) set->map_events.push_back({e0, e1});
         if (e == cudaSuccess) e = cudaEventRecord(e0, ctx->stream);
         if (e == cudaSuccess)
-            e = launch_grid_tiles((const float4*)(w + o_sorted), (const int*)(w + o_start), flo, kCellEdge, cd, d_p,
-                                  (const int2*)(w + o_tiles), (int)tiles.size(), pack_slots(set->slot, 0),
-                                  pack_slots(set->slot, 1), set->type_mask, ctx->stream);
+            e = launch_grid_maps((const float4*)(w + o_sorted), (const int*)(w + o_start), flo, kCellEdge, cd, d_p + first,
+                                 pk.data(), n_pockets, pack_slots(set->slot, 0), pack_slots(set->slot, 1),
+                                 set->type_mask, ctx->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e1, ctx->stream);
     }
     if (e == cudaSuccess && set->packed) {

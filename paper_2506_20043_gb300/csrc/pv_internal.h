@@ -39,11 +39,10 @@ constexpr int kMaxMergeEntries = 8192;
 cudaError_t launch_receptor_prep(const float* xyz, const uint8_t* el, const uint8_t* don, const uint8_t* acc, int n,
                                  const float lo[3], float cell, const int cdims[3], float4* typed, int* cell_of,
                                  int* next, int* head, int* cell_start, float4* sorted, cudaStream_t s);
-// Map build over a tile list (pocket, tile index); one CTA per 8 x 8 x 8 node tile.
-cudaError_t launch_grid_tiles(const float4* sorted, const int* cell_start, const float lo[3],
-                              float cell, const int cdims[3], const PvPocket* pockets_dev,
-                              const int2* tiles_dev, int n_tiles, uint64_t slots_lo, uint64_t slots_hi,
-                              int type_mask, cudaStream_t s);
+// Map build of n_pockets pockets (their device records and the same records on the host).
+cudaError_t launch_grid_maps(const float4* sorted, const int* cell_start, const float lo[3], float cell,
+                             const int cdims[3], const PvPocket* pockets_dev, const PvPocket* pockets_host, int n_pockets,
+                             uint64_t slots_lo, uint64_t slots_hi, int type_mask, cudaStream_t s);
 
 // Cell-packed copies of the maps of pockets [first, first + n) of a device pocket table: for every
 // map slot and cell, its eight corner values as two float4 at P.cells.

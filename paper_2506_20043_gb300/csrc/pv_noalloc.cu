@@ -5,7 +5,7 @@
 // or plugin that is handed device buffers but is not allowed to call cudaMalloc (or a caching
 // allocator) itself. pv_build_grid_noalloc serves them: the caller passes the receptor and the
 // output buffer for the maps, and every intermediate array of the build (typed and binned
-// receptor atoms, the cell index, the tile list, the pocket record) lives in one fixed array
+// receptor atoms, the cell index, the pocket record) lives in one fixed array
 // in this library's device memory, declared below. Each GPU that loads the library holds that
 // array until the process exits.
 #include <cmath>
@@ -37,9 +37,9 @@ constexpr size_t kOffCellOf = align256(kOffSorted + sizeof(float4) * kMaxAtoms);
 constexpr size_t kOffNext = align256(kOffCellOf + sizeof(int) * kMaxAtoms);
 constexpr size_t kOffHead = align256(kOffNext + sizeof(int) * kMaxAtoms);
 constexpr size_t kOffStart = align256(kOffHead + sizeof(int) * kMaxCells);
-constexpr size_t kOffTiles = align256(kOffStart + sizeof(int) * (kMaxCells + 1));
-constexpr size_t kOffPocket = align256(kOffTiles + sizeof(int2) * kMaxTiles);
-constexpr size_t kScratchBytes = align256(kOffPocket + sizeof(PvPocket));
+constexpr size_t kOffPocket = align256(kOffStart + sizeof(int) * (kMaxCells + 1));
+// 8 bytes per tile at the end are unused: the array keeps the size that the header states
+constexpr size_t kScratchBytes = align256(align256(kOffPocket + sizeof(PvPocket)) + 8 * kMaxTiles);
 static_assert(kScratchBytes == PV_NOALLOC_SCRATCH_BYTES, "scratch size must match the header");
 
 }  // namespace
@@ -52,11 +52,6 @@ namespace {
 
 std::mutex g_setup_mutex;
 void* g_scratch_addr[64];   // device address of the array, per device, after set-up
-
-__global__ void fill_tiles_kernel(int2* tiles, int n) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) tiles[t] = make_int2(0, t);
-}
 
 pv_status fail(pv_context* ctx, pv_status s, const std::string& msg) {
     context_set_error(ctx, msg.c_str());
@@ -171,10 +166,6 @@ extern "C" pv_status pv_build_grid_noalloc(pv_context* ctx, const pv_receptor* r
         // may free or reuse its arrays once this call returns
         if (e == cudaSuccess && r->mem == PV_MEM_HOST && host_pinned(r->xyz, r->element, r->donor, r->acceptor))
             e = cudaStreamSynchronize(stream);
-        if (e == cudaSuccess) {
-            fill_tiles_kernel<<<(int)((n_tiles + 255) / 256), 256, 0, stream>>>((int2*)(scratch + kOffTiles), (int)n_tiles);
-            e = cudaGetLastError();
-        }
         // the cell lists are emptied inside the binning step; every other array is fully
         // written before it is read, so what an earlier call left behind is never used
         if (e == cudaSuccess)
@@ -186,9 +177,8 @@ extern "C" pv_status pv_build_grid_noalloc(pv_context* ctx, const pv_receptor* r
         for (int t = 0; t < 8; ++t) s_lo |= (uint64_t)(uint8_t)slot[t] << (8 * t);
         for (int t = 0; t < 8; ++t) s_hi |= (uint64_t)(uint8_t)slot[8 + t] << (8 * t);
         if (e == cudaSuccess)
-            e = launch_grid_tiles((const float4*)(scratch + kOffSorted), (const int*)(scratch + kOffStart), flo, kCell,
-                                  cd, (const PvPocket*)(scratch + kOffPocket), (const int2*)(scratch + kOffTiles),
-                                  (int)n_tiles, s_lo, s_hi, mask, stream);
+            e = launch_grid_maps((const float4*)(scratch + kOffSorted), (const int*)(scratch + kOffStart), flo, kCell,
+                                 cd, (const PvPocket*)(scratch + kOffPocket), &P, 1, s_lo, s_hi, mask, stream);
         if (e != cudaSuccess) {
             status = e == cudaErrorMemoryAllocation ? PV_ERR_OOM : PV_ERR_CUDA;
             msg = std::string("pv_build_grid_noalloc: ") + cudaGetErrorString(e);

@@ -47,3 +47,14 @@ def test_binned_receptor_gives_the_direct_sums(name):
             ref = np.array([O.grid_node_value(rec, rt, b, t, *i) for i in idx])
             got = gs.read_map(p, t)[idx[:, 2], idx[:, 1], idx[:, 0]]
             assert G.close(got, ref).all(), (p, t, np.abs(got - ref).max())
+
+
+@pytest.mark.parametrize("types", [[10], [0], [1], [2, 5], [3, 7], [0, 10], [1, 4, 8], [6, 9, 10], [0, 1, 6], [2, 10]])
+def test_maps_do_not_depend_on_the_other_types_asked_for(types):
+    """Each set of element classes has its own map kernel: a type's map has the same bits in all."""
+    rec, boxes = _receptor(1500, 0.3, 9), [_box((0, 0, 0), (6.4, 4.9, 7.2)), _box((2, 1, 0), (3.0, 3.1, 2.6))]
+    every = G.context().build_grids(rec, boxes, list(range(11)))
+    some = G.context().build_grids(rec, boxes, types)
+    for p in range(len(boxes)):
+        for t in types:
+            np.testing.assert_array_equal(some.read_map(p, t), every.read_map(p, t))

@@ -457,27 +457,57 @@ __global__ void __launch_bounds__(kGridThreads, 7) grid_kernel(GridArgs A) {
     }
 }
 
-// Cell-packed copy of one pocket's maps: thread per (map slot, cell), the cell's eight corners
-// (x fastest) read from the plain map and written as two float4.
-__global__ void __launch_bounds__(256) pack_cells_kernel(const PvPocket* __restrict__ pockets, int pocket, int n_maps) {
-    const PvPocket& P = pockets[pocket];
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (long long)n_maps * P.ncells) return;
-    const int slot = (int)(k / P.ncells), cell = (int)(k - (long long)slot * P.ncells);
-    const int cx = P.dims[0] - 1, cy = P.dims[1] - 1;
-    const int ix = cell % cx, iy = (cell / cx) % cy, iz = cell / (cx * cy);
-    const float* m = P.maps + (long long)slot * P.nxyz + ((long long)iz * P.nxy + (long long)iy * P.dims[0] + ix);
-    float4* out = const_cast<float4*>(P.cells) + 2 * k;
-    out[0] = make_float4(m[0], m[1], m[P.dims[0]], m[P.dims[0] + 1]);
-    out[1] = make_float4(m[P.nxy], m[P.nxy + 1], m[P.nxy + P.dims[0]], m[P.nxy + P.dims[0] + 1]);
+// Cell-packed copies of pockets' maps: a thread takes a column of kPackZ cells of one map, whose
+// upper corners become the next cell's lower ones, so a cell costs four loads (three of them
+// L1 hits of its neighbours' lines) and one 32-byte store; a warp stores 1 KB without a gap. Bound by
+// the stores: 671 MB written and 88 MB read for ten 24 A boxes of 8 types in 214 us as a launch per
+// pocket of one cell per thread, its two 16-byte stores 32 bytes apart and its index divided out of a
+// 64-bit cell number; 113 us for the one launch, 6.7 TB/s.
+constexpr int kPackZ = 8;
+__global__ void __launch_bounds__(128) pack_cells_kernel(const PvPocket* __restrict__ pockets, int n_chunks) {
+    const PvPocket& P = pockets[blockIdx.z];
+    const int cx = P.dims[0] - 1, cy = P.dims[1] - 1, cz = P.dims[2] - 1;
+    const int slot = blockIdx.y / n_chunks, iz0 = (blockIdx.y - slot * n_chunks) * kPackZ;
+    const int col = blockIdx.x * blockDim.x + threadIdx.x;
+    if (col >= cx * cy || iz0 >= cz) return;
+    const int iy = col / cx, ix = col - iy * cx;
+    const int nx = P.dims[0], nxy = P.nxy, n = min(kPackZ, cz - iz0);
+    const float* m = P.maps + (long long)slot * P.nxyz + ((long long)iz0 * nxy + iy * nx + ix);
+    float* out = reinterpret_cast<float*>(const_cast<float4*>(P.cells)) +
+                 8 * ((long long)slot * P.ncells + (long long)iz0 * (cx * cy) + col);
+    const bool wide = (reinterpret_cast<uintptr_t>(P.cells) & 31) == 0;   // a caller's allocator may align to 16 bytes
+    float4 lo = make_float4(__ldg(m), __ldg(m + 1), __ldg(m + nx), __ldg(m + nx + 1));
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) {
+        m += nxy;
+        const float4 hi = make_float4(__ldg(m), __ldg(m + 1), __ldg(m + nx), __ldg(m + nx + 1));
+        if (wide) {
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(out), "f"(lo.x), "f"(lo.y),
+                         "f"(lo.z), "f"(lo.w), "f"(hi.x), "f"(hi.y), "f"(hi.z), "f"(hi.w)
+                         : "memory");
+        } else {
+            reinterpret_cast<float4*>(out)[0] = lo;
+            reinterpret_cast<float4*>(out)[1] = hi;
+        }
+        lo = hi;
+        out += 8LL * cx * cy;
+    }
 }
 
 cudaError_t launch_pack_cells(const PvPocket* pockets_dev, const PvPocket* pockets_host, int first, int n,
                               int n_maps, cudaStream_t s) {
-    for (int p = first; p < first + n; ++p) {
-        const long long work = (long long)n_maps * pockets_host[p].ncells;
-        if (work <= 0) continue;
-        pack_cells_kernel<<<(unsigned)((work + 255) / 256), 256, 0, s>>>(pockets_dev, p, n_maps);
+    // blockIdx: columns of a map, (map slot, chunk of z), pocket; sized for the largest pocket of the
+    // launch, at most 65,535 pockets each
+    for (int p0 = first; p0 < first + n; p0 += 65535) {
+        const int np = first + n - p0 < 65535 ? first + n - p0 : 65535;
+        int cols = 0, chunks = 0;
+        for (int p = p0; p < p0 + np; ++p) {
+            const int* d = pockets_host[p].dims;
+            const int c = (d[0] - 1) * (d[1] - 1), z = (d[2] - 1 + kPackZ - 1) / kPackZ;
+            cols = c > cols ? c : cols;
+            chunks = z > chunks ? z : chunks;
+        }
+        pack_cells_kernel<<<dim3((cols + 127) / 128, chunks * n_maps, np), 128, 0, s>>>(pockets_dev + p0, chunks);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

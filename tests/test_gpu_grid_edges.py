@@ -58,3 +58,38 @@ def test_maps_do_not_depend_on_the_other_types_asked_for(types):
     for p in range(len(boxes)):
         for t in types:
             np.testing.assert_array_equal(some.read_map(p, t), every.read_map(p, t))
+
+
+def _offset_context(shift):
+    """A context whose device memory starts `shift` bytes past the torch allocator's blocks."""
+    import torch
+    from paper_2506_20043_gb300 import _capi as A
+    from paper_2506_20043_gb300 import api
+    ctx = api.Context(0, torch_allocator=False)
+    alloc = A.ALLOC_FN(lambda n, stream, _: torch.cuda.caching_allocator_alloc(int(n) + shift, 0, stream) + shift)
+    free = A.FREE_FN(lambda p, _s, _u: torch.cuda.caching_allocator_delete(p - shift))
+    ctx._keep += [alloc, free]
+    ctx._check(ctx.lib.pv_context_set_allocator(ctx.h, alloc, free, None), "pv_context_set_allocator")
+    return ctx
+
+
+@pytest.mark.parametrize("shift", [0, 16])
+def test_packed_cells_of_ragged_boxes_hold_the_plain_corners(shift):
+    """Boxes of 1 to 27 cells per axis packed in one launch, in 32-byte and in 16-byte aligned memory:
+    a lookup in the packed cells gives the bits of one in the plain maps, over the whole box and beyond."""
+    import torch
+    ctx = _offset_context(shift)
+    sizes = [(0.3, 0.3, 0.3), (3.0, 3.0, 3.0), (0.375, 4.0, 10.0), (10.0, 0.5, 3.1), (5.2, 6.1, 3.4)]
+    boxes = [_box((0.3 * i, -0.2 * i, 0.1), s) for i, s in enumerate(sizes)]
+    lig = ctx.ligand(S.Ligand(np.zeros((1, 3)), np.zeros(1, np.uint8), np.zeros(1, np.uint8), np.zeros(1, np.uint8),
+                              np.zeros((0, 2), np.int32), np.zeros(0, np.uint8)))
+    rec = _receptor(800, 0.05, 10)
+    plain, packed = ctx.build_grids(rec, boxes, [0, 3, 10]), ctx.build_grids(rec, boxes, [0, 3, 10]).pack()
+    rng = np.random.default_rng(0)
+    for p, s in enumerate(sizes):
+        at = np.zeros((4096, 7), np.float32)
+        at[:, :3] = np.asarray(boxes[p].center) + (rng.random((4096, 3)) - 0.5) * (np.asarray(s) + 0.4)
+        at[:, 3] = 1.0
+        x = torch.tensor(at, device="cuda")
+        for a, b in zip(ctx.score(plain, lig, p, x)[:2], ctx.score(packed, lig, p, x)[:2]):
+            assert torch.equal(a, b)

@@ -314,8 +314,10 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
         float ge;
         const float fe = obj.eval(xt, ge);
         ++evals;
-        float f = Q.f, gd = Q.gd, lam = Q.lam, lo = Q.lo, hi = Q.hi, flo = Q.flo;
-        int it = Q.it, tr = Q.tr, stored = Q.stored, head = Q.head, have_lo = Q.have_lo;
+        const float4 q0 = *reinterpret_cast<const float4*>(&Q.f);
+        const int4 q1 = *reinterpret_cast<const int4*>(&Q.hi), q2 = *reinterpret_cast<const int4*>(&Q.stored);
+        float f = q0.x, gd = q0.y, lam = q0.z, lo = q0.w, hi = __int_as_float(q1.x), flo = __int_as_float(q1.y);
+        int it = q1.z, tr = q1.w, stored = q2.x, head = q2.y, have_lo = q2.z;
         bool next_iter = false, stop = false, retry = false, at_xt = false;
         if (start) {
             start = false;
@@ -397,8 +399,9 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
         }
         (void)retry;
         Tm::sync();                       // every lane has read this iteration's scalars
-        Q.f = f; Q.gd = gd; Q.lam = lam; Q.lo = lo; Q.hi = hi; Q.flo = flo;
-        Q.it = it; Q.tr = tr; Q.stored = stored; Q.head = head; Q.have_lo = have_lo;
+        *reinterpret_cast<float4*>(&Q.f) = make_float4(f, gd, lam, lo);
+        *reinterpret_cast<int4*>(&Q.hi) = make_int4(__float_as_int(hi), __float_as_int(flo), it, tr);
+        *reinterpret_cast<int4*>(&Q.stored) = make_int4(stored, head, have_lo, 0);
     }
 }
 template <bool FOCC, int LAYOUT>
@@ -554,7 +557,7 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) search_round_kernel(SearchA
     PvLigBlob& L = *reinterpret_cast<PvLigBlob*>(smem);
     WarpScratch* scratch = reinterpret_cast<WarpScratch*>(smem + ((A.lig_smem_bytes + 127) & ~127));
     __shared__ int s_item, s_lig, s_skip;
-    __shared__ PvPocket s_pocket;
+    __shared__ __align__(16) PvPocket s_pocket;
     constexpr int TPW = 32 / LANES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int team = warp * TPW + Team<LANES>::index();

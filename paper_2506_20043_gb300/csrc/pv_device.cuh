@@ -237,19 +237,22 @@ struct GridCell {
 };
 
 __device__ __forceinline__ GridCell grid_locate(const PvPocket& P, float3 p) {
-    const float g[3] = {(p.x - P.origin[0]) * P.inv_spacing, (p.y - P.origin[1]) * P.inv_spacing,
-                        (p.z - P.origin[2]) * P.inv_spacing};
+    const float4 o = *reinterpret_cast<const float4*>(P.origin);         // origin, 1 / spacing
+    const int4 n = *reinterpret_cast<const int4*>(P.dims);               // node counts, spacing
+    const float g[3] = {(p.x - o.x) * o.w, (p.y - o.y) * o.w, (p.z - o.z) * o.w};
+    const int dims[3] = {n.x, n.y, n.z};
+    const float spacing = __int_as_float(n.w);
     GridCell c;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const float hi = (float)(P.dims[k] - 1);
+        const float hi = (float)(dims[k] - 1);
         c.cl[k] = (g[k] < 0.0f) || (g[k] > hi);
         const float gc = fminf(fmaxf(g[k], 0.0f), hi);
         int ii = (int)floorf(gc);
-        ii = min(ii, P.dims[k] - 2);
+        ii = min(ii, dims[k] - 2);
         c.i[k] = ii;
         c.f[k] = gc - (float)ii;
-        c.out[k] = c.cl[k] ? (g[k] - gc) * P.spacing : 0.0f;
+        c.out[k] = c.cl[k] ? (g[k] - gc) * spacing : 0.0f;
     }
     return c;
 }

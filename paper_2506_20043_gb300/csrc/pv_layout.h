@@ -61,20 +61,21 @@ struct PvLigBlob {
     (PV_LIG_FIXED_BYTES + ((lanes) == 32 ? (n_rounds) * 32 : (n_rounds16) * 16) * (int)sizeof(PvPairSlot))
 
 // One pocket box of a grid set.
-struct PvPocket {
+// What a grid lookup reads comes first, in 16-byte words.
+struct __attribute__((aligned(16))) PvPocket {
     float origin[3];
-    float spacing;
     float inv_spacing;
     int32_t dims[3];
-    float center[3];
-    float size[3];
+    float spacing;
     float* maps;                // this pocket's maps, slot-major, each [z][y][x]
     int32_t nxy, nxyz;
     const float4* cells;        // the same maps cell-packed (slot-major, each cell's 8 corners as two
                                 // float4), or null when the grid set holds the plain layout only
-    const float4* rec_atoms;    // the pocket's receptor: xyz and XS type (int bits), for rescoring
-    int32_t rec_n;
     int32_t ncells;             // cells per map: (dims - 1) per axis
+    int32_t rec_n;
+    const float4* rec_atoms;    // the pocket's receptor: xyz and XS type (int bits), for rescoring
+    float center[3];
+    float size[3];
 };
 
 // XS type -> map slot of a grid set (-1: no map)

@@ -23,9 +23,13 @@ namespace pv {
 // Team-uniform scalars of a chain's MC step and of its line search, kept in shared memory rather
 // than registers: they are used between evaluations only, and every evaluation ends with a team
 // barrier, so registers holding them across it would only lower the kernel's occupancy.
-struct ChainScalars {
-    float e_cur, e_best, u, f, gd, lam, lo, hi, flo;
-    int s, stage, flags, nb_n, nb_head, it, tr, stored, head, have_lo;
+struct __align__(16) ChainScalars {
+    float f, gd, lam, lo;                     // of the line search: three 16-byte words
+    float hi, flo;
+    int it, tr;
+    int stored, head, have_lo, pad;
+    float e_cur, e_best, u;
+    int s, stage, flags, nb_n, nb_head;
     uint32_t evals_before;
 };
 
@@ -63,21 +67,29 @@ struct Team {
         for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask(), v, o, LANES);
         return v;
     }
-    static __device__ __forceinline__ float3 sum3(float3 v) {
-#pragma unroll
-        for (int o = LANES / 2; o > 0; o >>= 1) {
-            v.x += __shfl_xor_sync(mask(), v.x, o, LANES);
-            v.y += __shfl_xor_sync(mask(), v.y, o, LANES);
-            v.z += __shfl_xor_sync(mask(), v.z, o, LANES);
-        }
-        return v;
-    }
     static __device__ __forceinline__ float3 shfl3(float3 v, int src) {
         return make_float3(shfl(v.x, src), shfl(v.y, src), shfl(v.z, src));
     }
     static __device__ __forceinline__ float3 xor3(float3 v, int o) {
         return make_float3(__shfl_xor_sync(mask(), v.x, o, LANES), __shfl_xor_sync(mask(), v.y, o, LANES),
                            __shfl_xor_sync(mask(), v.z, o, LANES));
+    }
+    // Butterfly sums of eight values at once: while more than one value is left, a lane keeps half of
+    // them and sends the other half, so 8 values cost 7 + 1 + 1 shuffles (of a whole warp) instead of 5
+    // each. Every value is added over the same pairs of lanes in the same order as by sum(), so it has
+    // the same bits. Value k ends up in the lanes that agree with sum8_lane(k) in the top three lane bits.
+    static __device__ __forceinline__ float halve(float a, float b, int o) {
+        const bool hi = lane() & o;
+        return (hi ? b : a) + __shfl_xor_sync(mask(), hi ? a : b, o, LANES);
+    }
+    static __device__ __forceinline__ float finish8(float w0, float w1, float w2, float w3) {
+        float v = halve(halve(w0, w1, LANES / 4), halve(w2, w3, LANES / 4), LANES / 8);
+#pragma unroll
+        for (int o = LANES / 16; o > 0; o >>= 1) v += __shfl_xor_sync(mask(), v, o, LANES);
+        return v;
+    }
+    static __device__ __forceinline__ int sum8_lane(int k) {
+        return (k & 1) * (LANES / 2) + ((k >> 1) & 1) * (LANES / 4) + ((k >> 2) & 1) * (LANES / 8);
     }
     static __device__ __forceinline__ void sync() { __syncwarp(mask()); }
 };
@@ -105,15 +117,16 @@ __device__ __forceinline__ void init_scratch(WarpScratch& S) {
     __syncwarp();
 }
 
-// Pair slots of the team width's schedule.
+// Staged pair slots of the team width's schedule (stage_ligand).
 template <int LANES>
-__device__ __forceinline__ const PvPairSlot* pair_rounds(const PvLigBlob& L, int& rounds) {
-    if (LANES == 32) {
-        rounds = L.h.n_rounds;
-        return L.pairs;
-    }
-    rounds = L.h.n_rounds16;
-    return L.pairs + L.h.pairs16_at;
+__device__ __forceinline__ const float4* pair_rounds(const PvLigBlob& L, int& rounds) {
+    rounds = LANES == 32 ? L.h.n_rounds : L.h.n_rounds16;
+    return reinterpret_cast<const float4*>(L.pairs + (LANES == 32 ? 0 : L.h.pairs16_at));
+}
+
+// Position of a staged slot's partner.
+__device__ __forceinline__ float4 partner(const WarpScratch& S, int meta) {
+    return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(S.x) + ((unsigned)meta >> 16));
 }
 
 // Forward kinematics (Eq. 1: position, orientation, torsions -> atom coordinates). Writes S.x.
@@ -189,16 +202,16 @@ __device__ __forceinline__ void team_fk(const PvLigBlob& L, WarpScratch& S, cons
     axw = mat_vec(M, axis);   // the hinge axis in the world frame (rotating about it keeps it)
 }
 
-// The lane's pairs of two rounds (slots pa, pb; source atoms xia, xib; partners xa, xb), their
+// The lane's pairs of two rounds (staged slots p0, p1; source atoms xia, xib; partners xa, xb), their
 // arithmetic two pairs per instruction (packed FP32x2 adds, multiplies and FMAs; the reciprocal
 // square roots and exponentials one pair at a time): adds both energies to e_intra and returns the
 // forces on the sources in fa, fb. Per pair the same terms as pair_force.
-__device__ __forceinline__ void pair_force2(const PvPairSlot& pa, const PvPairSlot& pb, const float4& xia,
+__device__ __forceinline__ void pair_force2(const float4& p0, const float4& p1, const float4& xia,
                                             const float4& xib, const float4& xa, const float4& xb, float& e_intra,
                                             float3& fa, float3& fb) {
-    const float2 dx = __fadd2_rn(make_float2(xia.x, xib.x), make_float2(-xa.x, -xb.x));
-    const float2 dy = __fadd2_rn(make_float2(xia.y, xib.y), make_float2(-xa.y, -xb.y));
-    const float2 dz = __fadd2_rn(make_float2(xia.z, xib.z), make_float2(-xa.z, -xb.z));
+    const float2 dx = make_float2(xia.x - xa.x, xib.x - xb.x);
+    const float2 dy = make_float2(xia.y - xa.y, xib.y - xb.y);
+    const float2 dz = make_float2(xia.z - xa.z, xib.z - xb.z);
     const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
     const float2 rinv = make_float2(rsqrtf(fmaxf(r2.x, 1e-12f)), rsqrtf(fmaxf(r2.y, 1e-12f)));
     const float2 r = __fmul2_rn(r2, rinv);
@@ -209,8 +222,8 @@ __device__ __forceinline__ void pair_force2(const PvPairSlot& pa, const PvPairSl
     const float2 g1 = make_float2(exp2_approx(a1.x), exp2_approx(a1.y));   // exp(-(d / 0.5)^2)
     const float2 g2 = make_float2(exp2_approx(a2.x), exp2_approx(a2.y));   // exp(-((d - 3) / 2)^2)
     const float2 rep = make_float2(fminf(d.x, 0.f), fminf(d.y, 0.f));
-    const float2 c1 = make_float2(pa.c1, pb.c1), w = make_float2(pa.w, pb.w);
-    const float2 t = __ffma2_rn(c1, d, make_float2(pa.c0, pb.c0));        // the ramp w sat(c0 + c1 d)
+    const float2 c1 = make_float2(p0.z, p0.w), w = make_float2(p1.x, p1.y);
+    const float2 t = __ffma2_rn(c1, d, make_float2(p0.x, p0.y));        // the ramp w sat(c0 + c1 d)
     const float2 v = make_float2(__saturatef(t.x), __saturatef(t.y));
     const float2 dv = make_float2((t.x > 0.0f && t.x <= 1.0f) ? c1.x : 0.0f, (t.y > 0.0f && t.y <= 1.0f) ? c1.y : 0.0f);
     float2 e = __fmul2_rn(make_float2(kWGauss1, kWGauss1), g1);
@@ -232,13 +245,13 @@ __device__ __forceinline__ void pair_force2(const PvPairSlot& pa, const PvPairSl
 // The lane's pair of one round (source atom xi, partner position xj, the slot's ramp constants):
 // its energy and the force on the source, which the target's lane receives with the opposite
 // sign. An empty slot's partner is the far dummy atom: beyond the cutoff, it adds nothing.
-__device__ __forceinline__ float3 pair_force(const PvPairSlot& ps, const float4& xi, const float4& xj,
+__device__ __forceinline__ float3 pair_force(const float4& ps, const float4& xi, const float4& xj,
                                              float& e_intra) {
     const float3 d = make_float3(xi.x - xj.x, xi.y - xj.y, xi.z - xj.z);
     const float r2 = dot3(d, d);
     const bool live = r2 < kCutoff2;
     float c;
-    const float e = vina_pair_ramp(r2, xi.w + xj.w, ps.c0, ps.c1, ps.w, c);
+    const float e = vina_pair_ramp(r2, xi.w + xj.w, ps.y, ps.z, ps.w, c);
     e_intra += live ? e : 0.f;
     c = live ? c : 0.f;
     return c * d;
@@ -283,61 +296,65 @@ __device__ __forceinline__ float team_eval(const PvLigBlob& L, WarpScratch& S, c
     // atom is the source) and takes the opposite force of the pair it receives from the sending lane
     // by a shuffle, so forces stay in registers and rounds need no barrier.
     int rounds;
-    const PvPairSlot* pr = pair_rounds<LANES>(L, rounds);
+    const float4* pr = pair_rounds<LANES>(L, rounds) + tl;
     if (n <= LANES) {                         // every atom of a pair is its lane's first
         int r = 0;
-        for (; r + 1 < rounds; r += 2) {
-            const PvPairSlot pa = pr[r * LANES + tl], pb = pr[(r + 1) * LANES + tl];
-            const float4 xa = S.x[pa.meta & 127], xb = S.x[pb.meta & 127];
+        for (; r + 1 < rounds; r += 2, pr += 2 * LANES) {
+            const float4 p0 = pr[0], p1 = pr[LANES];
+            const int ma = __float_as_int(p1.z), mb = __float_as_int(p1.w);
+            const float4 xa = partner(S, ma), xb = partner(S, mb);
             float3 fa, fb;
-            pair_force2(pa, pb, own[0], own[0], xa, xb, e_intra, fa, fb);
-            const float3 fia = Tm::shfl3(fa, (pa.meta >> 8) & (LANES - 1));
-            const float3 fib = Tm::shfl3(fb, (pb.meta >> 8) & (LANES - 1));
+            pair_force2(p0, p1, own[0], own[0], xa, xb, e_intra, fa, fb);
+            const float3 fia = Tm::shfl3(fa, ma);
+            const float3 fib = Tm::shfl3(fb, mb);
             acc[0] = acc[0] + fa + fb;
-            if ((pa.meta >> 13) & 1) acc[0] = acc[0] - fia;
-            if ((pb.meta >> 13) & 1) acc[0] = acc[0] - fib;
+            if (ma & 32) acc[0] = acc[0] - fia;
+            if (mb & 32) acc[0] = acc[0] - fib;
         }
         if (r < rounds) {
-            const PvPairSlot pa = pr[r * LANES + tl];
-            const float3 fa = pair_force(pa, own[0], S.x[pa.meta & 127], e_intra);
-            const float3 fia = Tm::shfl3(fa, (pa.meta >> 8) & (LANES - 1));
+            const float4 pa = pr[0];
+            const int ma = __float_as_int(pa.x);
+            const float3 fa = pair_force(pa, own[0], partner(S, ma), e_intra);
+            const float3 fia = Tm::shfl3(fa, ma);
             acc[0] = acc[0] + fa;
-            if ((pa.meta >> 13) & 1) acc[0] = acc[0] - fia;
+            if (ma & 32) acc[0] = acc[0] - fia;
         }
     } else {
-        // two atoms per lane: meta bit 7 says the pair's own atom is the lane's second, bit 14 that
+        // two atoms per lane: meta bit 7 says the pair's own atom is the lane's second, bit 6 that
         // the received pair's atom is
         int r = 0;
-        for (; r + 1 < rounds; r += 2) {
-            const PvPairSlot pa = pr[r * LANES + tl], pb = pr[(r + 1) * LANES + tl];
-            const float4 xa = S.x[pa.meta & 127], xb = S.x[pb.meta & 127];
-            const bool sa = (pa.meta >> 7) & 1, sb = (pb.meta >> 7) & 1;
+        for (; r + 1 < rounds; r += 2, pr += 2 * LANES) {
+            const float4 p0 = pr[0], p1 = pr[LANES];
+            const int ma = __float_as_int(p1.z), mb = __float_as_int(p1.w);
+            const float4 xa = partner(S, ma), xb = partner(S, mb);
+            const bool sa = ma & 128, sb = mb & 128;
             float3 fa, fb;
-            pair_force2(pa, pb, sa ? own[1] : own[0], sb ? own[1] : own[0], xa, xb, e_intra, fa, fb);
-            const float3 fia = Tm::shfl3(fa, (pa.meta >> 8) & (LANES - 1));
-            const float3 fib = Tm::shfl3(fb, (pb.meta >> 8) & (LANES - 1));
+            pair_force2(p0, p1, sa ? own[1] : own[0], sb ? own[1] : own[0], xa, xb, e_intra, fa, fb);
+            const float3 fia = Tm::shfl3(fa, ma);
+            const float3 fib = Tm::shfl3(fb, mb);
             if (sa) acc[1] = acc[1] + fa;
             else acc[0] = acc[0] + fa;
             if (sb) acc[1] = acc[1] + fb;
             else acc[0] = acc[0] + fb;
-            if ((pa.meta >> 13) & 1) {
-                if ((pa.meta >> 14) & 1) acc[1] = acc[1] - fia;
+            if (ma & 32) {
+                if (ma & 64) acc[1] = acc[1] - fia;
                 else acc[0] = acc[0] - fia;
             }
-            if ((pb.meta >> 13) & 1) {
-                if ((pb.meta >> 14) & 1) acc[1] = acc[1] - fib;
+            if (mb & 32) {
+                if (mb & 64) acc[1] = acc[1] - fib;
                 else acc[0] = acc[0] - fib;
             }
         }
         if (r < rounds) {
-            const PvPairSlot pa = pr[r * LANES + tl];
-            const bool sa = (pa.meta >> 7) & 1;
-            const float3 fa = pair_force(pa, sa ? own[1] : own[0], S.x[pa.meta & 127], e_intra);
-            const float3 fia = Tm::shfl3(fa, (pa.meta >> 8) & (LANES - 1));
+            const float4 pa = pr[0];
+            const int ma = __float_as_int(pa.x);
+            const bool sa = ma & 128;
+            const float3 fa = pair_force(pa, sa ? own[1] : own[0], partner(S, ma), e_intra);
+            const float3 fia = Tm::shfl3(fa, ma);
             if (sa) acc[1] = acc[1] + fa;
             else acc[0] = acc[0] + fa;
-            if ((pa.meta >> 13) & 1) {
-                if ((pa.meta >> 14) & 1) acc[1] = acc[1] - fia;
+            if (ma & 32) {
+                if (ma & 64) acc[1] = acc[1] - fia;
                 else acc[0] = acc[0] - fia;
             }
         }
@@ -348,15 +365,14 @@ __device__ __forceinline__ float team_eval(const PvLigBlob& L, WarpScratch& S, c
         const int a = tl + LANES * h;
         if (a < n) S.g[a] = make_float4(acc[h].x, acc[h].y, acc[h].z, 0.f);
     }
-    float ei, ej;
-    if (parts) {
-        ei = Tm::sum(e_inter);
-        ej = Tm::sum(e_intra);
-        parts[0] = ei;
-        parts[1] = ej;
-    } else {
-        ei = Tm::sum(e_inter + e_intra);
-        ej = 0.f;
+    float ei, ej = 0.f;
+    if (!want_grad) {
+        if (parts) {
+            ei = Tm::sum(e_inter);
+            ej = Tm::sum(e_intra);
+        } else {
+            ei = Tm::sum(e_inter + e_intra);
+        }
     }
     if (want_grad) {
         Tm::sync();
@@ -370,8 +386,15 @@ __device__ __forceinline__ float team_eval(const PvLigBlob& L, WarpScratch& S, c
                 tau = tau + cross3(f3(own[h]) - x.T, acc[h]);
             }
         }
-        F = Tm::sum3(F);
-        tau = Tm::sum3(tau);
+        // force, torque and energy (its parts when asked for) in one butterfly; lane k < 6 then fetches
+        // component k, and every lane the energy
+        float w3 = parts ? Tm::halve(e_inter, e_intra, LANES / 2) : e_inter + e_intra;
+        if (!parts) w3 += __shfl_xor_sync(Tm::mask(), w3, LANES / 2, LANES);
+        const float v8 = Tm::finish8(Tm::halve(F.x, F.y, LANES / 2), Tm::halve(F.z, tau.x, LANES / 2),
+                                     Tm::halve(tau.y, tau.z, LANES / 2), w3);
+        const float rt = Tm::shfl(v8, Tm::sum8_lane(tl));
+        ei = Tm::shfl(v8, Tm::sum8_lane(6));
+        if (parts) ej = Tm::shfl(v8, Tm::sum8_lane(7));
         // torsions: the torque of each fragment's subtree (a contiguous atom range) about its
         // anchor, on its world hinge axis. k lanes share a fragment (k the largest power of two
         // with k * n_frag <= LANES), each summing every k-th atom of the range, then a butterfly
@@ -391,9 +414,11 @@ __device__ __forceinline__ float team_eval(const PvLigBlob& L, WarpScratch& S, c
         const int nt = 6 + L.h.n_rot;
         const int src = (tl >= 6 && tl < nt) ? L.tor_frag[tl - 6] * k : tl;
         float gp = Tm::shfl(gpsi, src);
-        // lane k takes component k (a select chain: an array indexed by the lane would live in local memory)
-        const float rt = tl == 0 ? F.x : (tl == 1 ? F.y : (tl == 2 ? F.z : (tl == 3 ? tau.x : (tl == 4 ? tau.y : tau.z))));
         grad = tl < 6 ? rt : (tl < nt ? gp : 0.f);
+    }
+    if (parts) {
+        parts[0] = ei;
+        parts[1] = ej;
     }
     Tm::sync();
     return ei + ej;

@@ -6,13 +6,18 @@
 // Layout. Receptor atoms are binned into cubic cells of kCell A over their bounding box (CSR,
 // input order kept within a cell, so every sum below runs in a fixed order). The SAS kernel runs
 // one warp per atom: the warp gathers the atoms whose expanded spheres can reach its sphere into
-// a shared-memory list (ballot compaction) and each lane tests the lattice points
-// lane + 32 m against it, keeping one burial bit per point in a register. The feature kernel runs
-// one warp per 32 consecutive points: the atoms of the cells within reach of the warp's bounding
-// box are staged 32 at a time in shared memory with one chunk of their property columns, and every
-// lane accumulates its point's sums in registers. Clustering hashes points into link-sized cells,
-// joins neighbours with a lock-free union-find that always hooks the larger root under the smaller
-// (so a component's root is its lowest index), and reduces per root in float64.
+// a shared-memory list, near ones first; each lane tests the lattice points lane + 32 m against the
+// near ones, keeping one burial bit per point in a register, and the warp takes the few points left
+// one by one against the rest. The feature kernel runs one CTA per 32 points: the atoms of the cells
+// within reach of the group's bounding box are staged 32 at a time in shared memory with one chunk of
+// their property columns, and every lane accumulates its point's sums in registers. Clustering hashes
+// points into link-sized cells, joins neighbours with a lock-free union-find that always hooks the
+// larger root under the smaller (so a component's root is its lowest index), and reduces per root in
+// float64.
+//
+// Every step but the features runs once for all receptors or point sets of a call: blockIdx.y picks the
+// item's record (SurfaceItem, ClusterItem) from a table uploaded with the inputs, so a call costs a dozen
+// launches whatever the number of receptors.
 //
 // Device memory comes from a library-owned stream-ordered pool per device (allocated and freed on
 // the context's stream); freed blocks stay in the pool for the next call.
@@ -65,37 +70,123 @@ __device__ __forceinline__ float3 sphere_point(const float4& A, float a, const f
 
 // ------------------------------------------------------------------------------ binning ---
 
-// Atoms in input order as (x, y, z, index bits), expanded radius a_i = R_i + probe, cell key.
-__global__ void prep_atoms_kernel(const float* __restrict__ xyz, const uint8_t* __restrict__ element,
-                                  const float* __restrict__ radius, float probe, int n, AtomGrid G,
-                                  float4* __restrict__ atoms, float* __restrict__ arad,
-                                  int* __restrict__ key, int* __restrict__ count, int* __restrict__ err) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
-    float r;
-    if (radius) {
-        r = radius[i];
-        if (!(r > 0.f && r <= 10.f)) atomicOr(err, kErrRadius);
-    } else {
-        const int e = element[i];
-        if (e > 3) atomicOr(err, kErrElement);
-        r = c_bondi[e & 3];
+// One receptor of a surface call (device pointers).
+struct SurfaceItem {
+    const float* xyz;        // [n][3]
+    const uint8_t* element;
+    const float* radius;     // or null: Bondi radii by element
+    int n, n_cells;
+    AtomGrid G;
+    float reach_max;         // largest a_j plus a margin
+    float4* atoms;           // input order: (x, y, z, index bits)
+    float* arad;             // a_i = R_i + probe, input order
+    int* key;                // cell of an atom
+    int* count;              // [n_cells] atoms of a cell
+    int* head;               // [n_cells] 1 + the last atom linked into the cell's list, 0: none
+    int* next;               // [n] likewise
+    int* cell_start;         // [n_cells + 1]
+    float4* sorted;          // cell order, input order within a cell
+    float* srad;             // a_i, cell order
+    int* order;              // input index of the sorted atoms
+    uint32_t* kept;          // [n][32]: bit m of lane's word = point lane + 32 m kept
+    int* n_kept;             // [n]
+    int* offset;             // [n + 1] first kept point of an atom, atoms in input order
+    int* offset_sorted;      // [n + 1] the same with atoms in cell order
+    float* pts;              // [n_points][3]
+    int* src;                // [n_points]
+    int* perm;               // [n_points] points grouped by the cell order of their atoms
+    int* status;             // [0] error bits, [1] kept points
+};
+
+// Bounding box and validity of device-resident receptors, one CTA each: out[8 j ..] = lo, hi (x, y, z),
+// the largest radius, error bits (kErrCoord: a coordinate beyond 1e6 A or not finite; kErrRadius).
+struct BoundsItem {
+    const float* xyz;
+    const float* radius;
+    int n;
+};
+__global__ void __launch_bounds__(1024) bounds_kernel(const BoundsItem* __restrict__ items, float* __restrict__ out) {
+    __shared__ float s_v[8][32];
+    const BoundsItem it = items[blockIdx.x];
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { v[k] = INFINITY; v[3 + k] = -INFINITY; }
+    v[6] = 0.f;
+    int err = 0;
+    for (int i = threadIdx.x; i < it.n; i += 1024) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float x = it.xyz[3 * (size_t)i + k];
+            if (!(fabsf(x) <= 1e6f)) err |= kErrCoord;
+            v[k] = fminf(v[k], x);
+            v[3 + k] = fmaxf(v[3 + k], x);
+        }
+        if (it.radius) {
+            const float r = it.radius[i];
+            if (!(r > 0.f && r <= 10.f)) err |= kErrRadius;
+            v[6] = fmaxf(v[6], r);
+        }
     }
-    if (!(isfinite(x) && isfinite(y) && isfinite(z))) atomicOr(err, kErrCoord);
-    atoms[i] = make_float4(x, y, z, __int_as_float(i));
-    arad[i] = r + probe;
-    const int c = (cell_coord(z, G.lo[2], G.inv_cell, G.cd[2]) * G.cd[1] +
-                   cell_coord(y, G.lo[1], G.inv_cell, G.cd[1])) * G.cd[0] +
-                  cell_coord(x, G.lo[0], G.inv_cell, G.cd[0]);
-    key[i] = c;
-    atomicAdd(&count[c], 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    err = __reduce_or_sync(0xffffffffu, err);
+    auto fold = [&]() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 7; ++k) {
+                const float u = __shfl_xor_sync(0xffffffffu, v[k], o);
+                v[k] = k < 3 ? fminf(v[k], u) : fmaxf(v[k], u);
+            }
+    };
+    fold();
+    if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < 7; ++k) s_v[k][warp] = v[k];
+        s_v[7][warp] = __int_as_float(err);
+    }
+    __syncthreads();
+    if (warp != 0) return;
+#pragma unroll
+    for (int k = 0; k < 7; ++k) v[k] = s_v[k][lane];
+    err = __reduce_or_sync(0xffffffffu, __float_as_int(s_v[7][lane]));
+    fold();
+    if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < 7; ++k) out[8 * blockIdx.x + k] = v[k];
+        out[8 * blockIdx.x + 7] = __int_as_float(err);
+    }
 }
 
-// Exclusive scan of count[0 .. n) into start[0 .. n] by one CTA of 1024 threads, over tiles of
-// 4096 elements (four consecutive elements per thread, coalesced loads), carrying the running total.
-__global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ count, int n,
-                                                    int* __restrict__ start) {
+// Atoms in input order, expanded radii, and each atom linked into its cell's list.
+__global__ void __launch_bounds__(256) prep_atoms_kernel(const SurfaceItem* __restrict__ items, float probe) {
+    const SurfaceItem& g = items[blockIdx.y];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.n) return;
+    const float x = g.xyz[3 * i], y = g.xyz[3 * i + 1], z = g.xyz[3 * i + 2];
+    float r;
+    if (g.radius) {
+        r = g.radius[i];
+        if (!(r > 0.f && r <= 10.f)) atomicOr(g.status, kErrRadius);
+    } else {
+        const int e = g.element[i];
+        if (e > 3) atomicOr(g.status, kErrElement);
+        r = c_bondi[e & 3];
+    }
+    if (!(isfinite(x) && isfinite(y) && isfinite(z))) atomicOr(g.status, kErrCoord);
+    g.atoms[i] = make_float4(x, y, z, __int_as_float(i));
+    g.arad[i] = r + probe;
+    const int c = (cell_coord(z, g.G.lo[2], g.G.inv_cell, g.G.cd[2]) * g.G.cd[1] +
+                   cell_coord(y, g.G.lo[1], g.G.inv_cell, g.G.cd[1])) * g.G.cd[0] +
+                  cell_coord(x, g.G.lo[0], g.G.inv_cell, g.G.cd[0]);
+    g.key[i] = c;
+    atomicAdd(&g.count[c], 1);
+    g.next[i] = atomicExch(&g.head[c], i + 1);
+}
+
+// Exclusive scan of count(0 .. n) into start[0 .. n] by one CTA of 1024 threads, over tiles of
+// 4096 elements (four consecutive elements per thread), carrying the running total, which is returned.
+template <typename F>
+__device__ __forceinline__ int block_scan(F&& count, int n, int* __restrict__ start) {
     __shared__ int s_warp[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int carry = 0;
@@ -103,7 +194,7 @@ __global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ coun
         const int i0 = base + 4 * (int)threadIdx.x;
         int v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = i0 + k < n ? count[i0 + k] : 0;
+        for (int k = 0; k < 4; ++k) v[k] = i0 + k < n ? count(i0 + k) : 0;
         const int sum = v[0] + v[1] + v[2] + v[3];
         int x = sum;
 #pragma unroll
@@ -133,160 +224,201 @@ __global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ coun
         carry += s_warp[31];
     }
     if (threadIdx.x == 0) start[n] = carry;
+    return carry;
 }
 
-// Unstable placement: each element with key >= 0 takes a slot of its key's segment.
-__global__ void scatter_kernel(const int* __restrict__ key, int n, const int* __restrict__ start,
-                               int* __restrict__ cursor, int* __restrict__ slot_elem) {
+__global__ void __launch_bounds__(1024) cell_scan_kernel(const SurfaceItem* __restrict__ items) {
+    const SurfaceItem& g = items[blockIdx.y];
+    const int* count = g.count;
+    block_scan([&](int i) { return count[i]; }, g.n_cells, g.cell_start);
+}
+
+// Every atom to its place: its cell's first slot plus the number of the cell's atoms of lower index.
+__global__ void __launch_bounds__(256) sort_atoms_kernel(const SurfaceItem* __restrict__ items) {
+    const SurfaceItem& g = items[blockIdx.y];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int k = key[i];
-    if (k < 0) return;
-    slot_elem[start[k] + atomicAdd(&cursor[k], 1)] = i;
-}
-
-// Stable order: within a segment, an element's rank is the number of lower indices in it.
-// Only the start[n_keys] placed slots are read.
-__global__ void stable_kernel(const int* __restrict__ key, const int* __restrict__ slot_elem, int n,
-                              const int* __restrict__ start, int n_keys, int* __restrict__ order) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n || s >= start[n_keys]) return;
-    const int i = slot_elem[s];
-    const int k = key[i], b = start[k], e = start[k + 1];
-    int r = 0;
-    for (int t = b; t < e; ++t) r += slot_elem[t] < i;
-    order[b + r] = i;
-}
-
-__global__ void gather_atoms_kernel(const int* __restrict__ order, int n, const float4* __restrict__ atoms,
-                                    float4* __restrict__ sorted) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n) sorted[s] = atoms[order[s]];
-}
-
-// Stable CSR of n keys in [0, n_keys) (key < 0: left out): start[n_keys + 1], order[count].
-cudaError_t bin_keys(const int* key, int n, int n_keys, const int* count, int* start, int* cursor,
-                     int* slot_elem, int* order, cudaStream_t s) {
-    scan_kernel<<<1, 1024, 0, s>>>(count, n_keys, start);
-    cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(int) * n_keys, s);
-    if (e != cudaSuccess) return e;
-    const int b = (n + 255) / 256;
-    if (b > 0) {
-        scatter_kernel<<<b, 256, 0, s>>>(key, n, start, cursor, slot_elem);
-        stable_kernel<<<b, 256, 0, s>>>(key, slot_elem, n, start, n_keys, order);
-    }
-    return cudaGetLastError();
+    if (i >= g.n) return;
+    const int c = g.key[i];
+    int r = g.cell_start[c];
+    for (int a = g.head[c]; a; a = g.next[a - 1]) r += a - 1 < i;
+    g.sorted[r] = g.atoms[i];
+    g.srad[r] = g.arad[i];
+    g.order[r] = i;
 }
 
 // ---------------------------------------------------------------------- Step 1: SAS ---
 
-struct SasArgs {
-    const float4* atoms;     // input order
-    const float4* sorted;    // cell order
-    const float* arad;       // a_i, input order
-    const int* cell_start;
-    AtomGrid G;
-    const float* dirs;       // [n_sphere][3]
-    int n_atoms, n_sphere;
-    float reach_max;         // largest a_j plus a margin
-    uint32_t* kept;          // [n_atoms][32]: bit m of lane's word = point lane + 32 m kept
-    int* n_kept;             // [n_atoms]
-};
-
-__device__ __forceinline__ uint32_t bury(const float4* nb, int cnt, const float4& A, float a,
+// The points of atom A not yet buried, against the spheres of the list: the n_near near ones at its
+// front (each buries about a third of the sphere) lane by lane, every lane its points lane + 32 m; then
+// the points left (about one in ten) four at a time, eight lanes each, against the n_far others at the
+// list's end. Whether a point is buried does not depend on the order of the tests.
+__device__ __forceinline__ uint32_t bury(const float4* nb, int n_near, int n_far, const float4& A, float a,
                                          const float* dirs, int n_sphere, int lane, uint32_t buried) {
     const int M = (n_sphere + 31) >> 5;
+    auto inside = [](const float3& p, const float4& q) {
+        const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
+        return dx * dx + dy * dy + dz * dz < q.w;
+    };
+    const int group = lane >> 3, sub = lane & 7;
     for (int m = 0; m < M; ++m) {
         const int k = lane + 32 * m;
-        if (k >= n_sphere || ((buried >> m) & 1u)) continue;
-        const float3 p = sphere_point(A, a, dirs, k);
-        for (int t = 0; t < cnt; ++t) {
-            const float4 q = nb[t];
-            const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
-            if (dx * dx + dy * dy + dz * dz < q.w) {
-                buried |= 1u << m;
-                break;
+        bool open = k < n_sphere && !((buried >> m) & 1u);
+        if (open) {
+            const float3 p = sphere_point(A, a, dirs, k);
+            for (int t = 0; t < n_near; ++t)
+                if (inside(p, nb[t])) {
+                    buried |= 1u << m;
+                    open = false;
+                    break;
+                }
+        }
+        for (unsigned left = __ballot_sync(0xffffffffu, open); left;) {
+            int b = -1;                                  // this group's point: the group-th one left
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (group == q && left) b = __ffs(left) - 1;
+                left &= left - 1;                        // stays 0 once it is
             }
+            bool hit = false;
+            if (b >= 0) {
+                const float3 p = sphere_point(A, a, dirs, b + 32 * m);
+                for (int t = sub; t < n_far && !hit; t += 8) hit = inside(p, nb[kNb - 1 - t]);
+            }
+            // the points found inside, as bits of the lanes that own them
+            const unsigned hits = __ballot_sync(0xffffffffu, hit);
+            const bool found = b >= 0 && ((hits >> (8 * group)) & 0xffu);
+            const unsigned mine = __reduce_or_sync(0xffffffffu, found ? 1u << b : 0u);
+            if ((mine >> lane) & 1u) buried |= 1u << m;
         }
     }
     return buried;
 }
 
-__global__ void __launch_bounds__(kSasWarps * 32) sas_kernel(SasArgs g) {
+// Issue-bound: 100 lattice points per atom against the 57 spheres that can reach them. A warp that
+// tested the spheres in cell order, lanes waiting for the slowest, took 36 us for 8,000 atoms (22 of 32
+// lanes active) and 195 us for seven receptors of 36,700 atoms in all, one after another; these take 75 us in
+// one launch, 16 instead of 23 us for 1,500 atoms. Near spheres: closer than 1.1 a, about a dozen.
+__global__ void __launch_bounds__(kSasWarps * 32) sas_kernel(const SurfaceItem* __restrict__ items,
+                                                             const float* __restrict__ dirs, int n_sphere) {
     __shared__ float4 s_nb[kSasWarps][kNb];
+    const SurfaceItem& g = items[blockIdx.y];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int s = blockIdx.x * kSasWarps + wib;
-    if (s >= g.n_atoms) return;                         // warp-uniform
+    if (s >= g.n) return;                               // warp-uniform
     float4* nb = s_nb[wib];
-    const float4 A = g.sorted[s];
-    const int i = __float_as_int(A.w);
-    const float a = g.arad[i];
+    const float4* sorted = g.sorted;
+    const float* srad = g.srad;
+    const float4 A = sorted[s];
+    const float a = srad[s];
     const float reach = a + g.reach_max;
+    const AtomGrid G = g.G;
     int c0[3], c1[3];
     const float pa[3] = {A.x, A.y, A.z};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        c0[k] = cell_coord(pa[k] - reach, g.G.lo[k], g.G.inv_cell, g.G.cd[k]);
-        c1[k] = cell_coord(pa[k] + reach, g.G.lo[k], g.G.inv_cell, g.G.cd[k]);
+        c0[k] = cell_coord(pa[k] - reach, G.lo[k], G.inv_cell, G.cd[k]);
+        c1[k] = cell_coord(pa[k] + reach, G.lo[k], G.inv_cell, G.cd[k]);
     }
+    const float near2 = 1.2f * a * a;
+    const float slack = 1e-2f + 1e-6f * (fabsf(A.x) + fabsf(A.y) + fabsf(A.z));
     uint32_t buried = 0;
-    int cnt = 0;
-    for (int cz = c0[2]; cz <= c1[2]; ++cz)
-        for (int cy = c0[1]; cy <= c1[1]; ++cy) {
-            const int row = (cz * g.G.cd[1] + cy) * g.G.cd[0];
-            const int b = g.cell_start[row + c0[0]], e = g.cell_start[row + c1[0] + 1];
-            for (int base = b; base < e; base += 32) {
-                const int j = base + lane;
-                bool take = false;
-                float4 B = make_float4(0.f, 0.f, 0.f, 0.f);
-                float aj = 0.f;
-                if (j < e) {
-                    B = g.sorted[j];
-                    const int idx = __float_as_int(B.w);
-                    aj = g.arad[idx];
-                    const float dx = B.x - A.x, dy = B.y - A.y, dz = B.z - A.z;
-                    const float lim = a + aj + 1e-3f;   // spheres that can overlap, with slack
-                    take = idx != i && dx * dx + dy * dy + dz * dz < lim * lim;
-                }
-                const unsigned bal = __ballot_sync(0xffffffffu, take);
-                if (take) nb[cnt + __popc(bal & ((1u << lane) - 1u))] = make_float4(B.x, B.y, B.z, aj * aj);
-                cnt += __popc(bal);
-                if (cnt > kNb - 32) {
-                    __syncwarp();
-                    buried = bury(nb, cnt, A, a, g.dirs, g.n_sphere, lane, buried);
-                    __syncwarp();
-                    cnt = 0;
-                }
+    int n_near = 0, n_far = 0;
+    // the rows of cells in reach, a lane each, 32 at a time; their atoms as one list
+    const int ny = c1[1] - c0[1] + 1, n_rows = ny * (c1[2] - c0[2] + 1);
+    for (int r0 = 0; r0 < n_rows; r0 += 32) {
+        int b = 0, n = 0;
+        if (r0 + lane < n_rows) {
+            // the row's cells within reach of the atom (a little more than reach: cell borders are rounded)
+            const int cz = c0[2] + (r0 + lane) / ny, cy = c0[1] + (r0 + lane) % ny;
+            const float ylo = G.lo[1] + cy * kCell, zlo = G.lo[2] + cz * kCell;
+            const float dy = fmaxf(0.f, fmaxf(ylo - A.y, A.y - (ylo + kCell)) - slack);
+            const float dz = fmaxf(0.f, fmaxf(zlo - A.z, A.z - (zlo + kCell)) - slack);
+            const float left = reach * reach - dy * dy - dz * dz;
+            if (left > 0.f) {
+                const float half = sqrtf(left) + slack;
+                const int row = (cz * G.cd[1] + cy) * G.cd[0];
+                b = g.cell_start[row + cell_coord(A.x - half, G.lo[0], G.inv_cell, G.cd[0])];
+                n = g.cell_start[row + cell_coord(A.x + half, G.lo[0], G.inv_cell, G.cd[0]) + 1] - b;
             }
         }
+        int end = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += y;
+        }
+        const int total = __shfl_sync(0xffffffffu, end, 31), shift = b - (end - n);
+        for (int base = 0; base < total; base += 32) {
+            const int p = base + lane;
+            int row = 0;                                 // the rows that end at or before position p
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xffffffffu, end, row + o - 1) <= p) row += o;
+            const int j = __shfl_sync(0xffffffffu, shift, row & 31) + p;
+            bool take = false, near = false;
+            float4 B = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (p < total && j != s) {
+                B = sorted[j];
+                const float aj = srad[j];
+                const float dx = B.x - A.x, dy = B.y - A.y, dz = B.z - A.z;
+                const float lim = a + aj + 1e-3f;       // spheres that can overlap, with slack
+                const float d2 = dx * dx + dy * dy + dz * dz;
+                take = d2 < lim * lim;
+                near = take && d2 < near2;
+                B.w = aj * aj;
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, take), baln = __ballot_sync(0xffffffffu, near);
+            const unsigned below = (1u << lane) - 1u;
+            if (near) nb[n_near + __popc(baln & below)] = B;
+            else if (take) nb[kNb - 1 - (n_far + __popc(bal & ~baln & below))] = B;
+            n_near += __popc(baln);
+            n_far += __popc(bal & ~baln);
+            if (n_near + n_far > kNb - 32) {
+                __syncwarp();
+                buried = bury(nb, n_near, n_far, A, a, dirs, n_sphere, lane, buried);
+                __syncwarp();
+                n_near = n_far = 0;
+            }
+        }
+    }
     __syncwarp();
-    buried = bury(nb, cnt, A, a, g.dirs, g.n_sphere, lane, buried);
-    const int M = (g.n_sphere + 31) >> 5;
+    buried = bury(nb, n_near, n_far, A, a, dirs, n_sphere, lane, buried);
+    const int M = (n_sphere + 31) >> 5;
     uint32_t valid = 0;
     for (int m = 0; m < M; ++m)
-        if (lane + 32 * m < g.n_sphere) valid |= 1u << m;
+        if (lane + 32 * m < n_sphere) valid |= 1u << m;
     const uint32_t keep = valid & ~buried;
+    const int i = __float_as_int(A.w);
     g.kept[(size_t)i * 32 + lane] = keep;
-    int c = __popc(keep);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    const int c = __reduce_add_sync(0xffffffffu, __popc(keep));
     if (lane == 0) g.n_kept[i] = c;
 }
 
-// Kept points in (atom, k) order.
-__global__ void __launch_bounds__(128) sas_write_kernel(const float4* __restrict__ atoms,
-                                                        const float* __restrict__ arad,
-                                                        const float* __restrict__ dirs, int n_atoms,
-                                                        int n_sphere, const uint32_t* __restrict__ kept,
-                                                        const int* __restrict__ offset, float* __restrict__ pts,
-                                                        int* __restrict__ src) {
+// First points of the atoms, in input order (blockIdx.x 0) and in cell order (1).
+__global__ void __launch_bounds__(1024) point_scan_kernel(const SurfaceItem* __restrict__ items) {
+    const SurfaceItem& g = items[blockIdx.y];
+    const int *n_kept = g.n_kept, *order = g.order;
+    if (blockIdx.x == 0) {
+        const int total = block_scan([&](int i) { return n_kept[i]; }, g.n, g.offset);
+        if (threadIdx.x == 0) g.status[1] = total;
+    } else {
+        block_scan([&](int i) { return n_kept[order[i]]; }, g.n, g.offset_sorted);
+    }
+}
+
+// Kept points in (atom, k) order, a warp per atom, and their grouping by the cell order of the atoms.
+__global__ void __launch_bounds__(128) sas_write_kernel(const SurfaceItem* __restrict__ items,
+                                                        const float* __restrict__ dirs, int n_sphere) {
+    const SurfaceItem& g = items[blockIdx.y];
     const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (i >= n_atoms) return;
-    const float4 A = atoms[i];
-    const float a = arad[i];
-    const uint32_t word = kept[(size_t)i * 32 + lane];
-    int base = offset[i];
+    const int s = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (s >= g.n) return;
+    const int i = g.order[s];
+    const float4 A = g.atoms[i];
+    const float a = g.arad[i];
+    const uint32_t word = g.kept[(size_t)i * 32 + lane];
+    int base = g.offset[i];
+    const int shift = g.offset_sorted[s] - base;
     const int M = (n_sphere + 31) >> 5;
     for (int m = 0; m < M; ++m) {
         const bool on = (word >> m) & 1u;
@@ -295,10 +427,11 @@ __global__ void __launch_bounds__(128) sas_write_kernel(const float4* __restrict
             const int k = lane + 32 * m;
             const int pos = base + __popc(bal & ((1u << lane) - 1u));
             const float3 p = sphere_point(A, a, dirs, k);
-            pts[3 * (size_t)pos] = p.x;
-            pts[3 * (size_t)pos + 1] = p.y;
-            pts[3 * (size_t)pos + 2] = p.z;
-            src[pos] = i * n_sphere + k;
+            g.pts[3 * (size_t)pos] = p.x;
+            g.pts[3 * (size_t)pos + 1] = p.y;
+            g.pts[3 * (size_t)pos + 2] = p.z;
+            g.src[pos] = i * n_sphere + k;
+            g.perm[pos + shift] = pos;
         }
         base += __popc(bal);
     }
@@ -478,23 +611,6 @@ __global__ void __launch_bounds__(kFeatSplit * 32) feature_kernel(FeatArgs g) {
     if (g.prot && blockIdx.y == 0) g.prot[pi] = fin ? total : 0;
 }
 
-// Points grouped by the cell order of their atoms: perm[base_sorted[s] + t] = offset[i] + t for
-// the t-th point of atom i = order[s].
-__global__ void sorted_counts_kernel(const int* __restrict__ order, const int* __restrict__ n_kept, int n,
-                                     int* __restrict__ cnt) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n) cnt[s] = n_kept[order[s]];
-}
-
-__global__ void perm_kernel(const int* __restrict__ order, const int* __restrict__ n_kept,
-                            const int* __restrict__ offset, const int* __restrict__ base_sorted, int n,
-                            int* __restrict__ perm) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    const int i = order[s], m = n_kept[i], o = offset[i], b = base_sorted[s];
-    for (int t = 0; t < m; ++t) perm[b + t] = o + t;
-}
-
 // ------------------------------------------------------------ Steps 4-5: clusters ---
 
 // Spatial hash of a link-sized cell (Teschner et al., "Optimized Spatial Hashing for Collision
@@ -503,23 +619,36 @@ __device__ __forceinline__ int cell_hash(int x, int y, int z, uint32_t mask) {
     return (int)((((uint32_t)x * 73856093u) ^ ((uint32_t)y * 19349663u) ^ ((uint32_t)z * 83492791u)) & mask);
 }
 
-struct ClusterArgs {
+// One point set of a clustering call (device pointers).
+struct ClusterItem {
     const float* pts;
     const float* score;
-    int n;
+    int n, n_buckets;
     float theta, link2, inv_cell;
     uint32_t hmask;
     int* key;                // [n] bucket of a clustered point, -1 otherwise
-    int* count;              // [buckets]
+    int* count;              // [buckets] points of a bucket; counted down as they are placed
+    int* start;              // [buckets + 1]
+    float4* spts;            // clustered points in bucket order: (x, y, z, index bits)
     int* parent;             // [n]
-    int* err;
+    int* root;               // [n]
+    int* cid;                // [n] cluster id of a root (order of discovery)
+    double* s2;              // [n] per root
+    double* sx;              // [n][3] per root
+    int* size;               // [n] per root
+    int* c_first;            // [n] root of a cluster id
+    int* rank;               // [n] rank of a cluster id
+    int* status;             // [0] error bits, [1] clusters
+    int* cluster;            // [n] per point: its cluster's rank
+    float* out;              // K clusters by rank: score [K], center [K][3], size [K], first [K]
 };
 
 __device__ __forceinline__ int3 link_cell(const float* p, float inv) {
     return make_int3(__float2int_rd(p[0] * inv), __float2int_rd(p[1] * inv), __float2int_rd(p[2] * inv));
 }
 
-__global__ void cl_init_kernel(ClusterArgs g) {
+__global__ void __launch_bounds__(256) cl_init_kernel(const ClusterItem* __restrict__ items) {
+    const ClusterItem& g = items[blockIdx.y];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.n) return;
     g.parent[i] = i;
@@ -532,7 +661,7 @@ __global__ void cl_init_kernel(ClusterArgs g) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) ok = ok && isfinite(p[c]) && fabsf(p[c] * g.inv_cell) < lim;
         if (!ok) {
-            atomicOr(g.err, kErrCoord);
+            atomicOr(g.status, kErrCoord);
         } else {
             const int3 c = link_cell(p, g.inv_cell);
             k = cell_hash(c.x, c.y, c.z, g.hmask);
@@ -540,6 +669,25 @@ __global__ void cl_init_kernel(ClusterArgs g) {
         }
     }
     g.key[i] = k;
+}
+
+__global__ void __launch_bounds__(1024) cl_scan_kernel(const ClusterItem* __restrict__ items) {
+    const ClusterItem& g = items[blockIdx.y];
+    const int* count = g.count;
+    block_scan([&](int i) { return count[i]; }, g.n_buckets, g.start);
+}
+
+// Clustered points into their buckets (in any order within one: nothing below depends on it): a
+// neighbour scan reads each candidate with one contiguous load, and consecutive warps take
+// neighbouring points.
+__global__ void __launch_bounds__(256) cl_place_kernel(const ClusterItem* __restrict__ items) {
+    const ClusterItem& g = items[blockIdx.y];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.n) return;
+    const int k = g.key[i];
+    if (k < 0) return;
+    const float* p = g.pts + 3 * (size_t)i;
+    g.spts[g.start[k] + atomicSub(&g.count[k], 1) - 1] = make_float4(p[0], p[1], p[2], __int_as_float(i));
 }
 
 // Root of v: parents only ever point to lower indices, so the walk ends.
@@ -571,32 +719,22 @@ __device__ __forceinline__ bool uf_unite(int* par, int a, int b) {
     return a == b;
 }
 
-// Clustered points in bucket order as (x, y, z, index bits): a neighbour scan reads each candidate
-// with one contiguous load, and consecutive threads take neighbouring points.
-__global__ void cl_gather_kernel(const int* __restrict__ order, const float* __restrict__ pts,
-                                 const int* __restrict__ total, float4* __restrict__ spts) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= *total) return;
-    const int i = order[t];
-    spts[t] = make_float4(pts[3 * (size_t)i], pts[3 * (size_t)i + 1], pts[3 * (size_t)i + 2], __int_as_float(i));
-}
-
 // One warp per clustered point: lane l < 27 scans link cell l of the 27 around q's cell and calls
 // f(j) for every clustered point j within the link of q there (q included; two cells that share a
 // hash bucket are scanned twice, which changes nothing below).
 template <typename F>
-__device__ __forceinline__ void for_linked_lane(const ClusterArgs& g, const int* __restrict__ start,
-                                                const float4* __restrict__ spts, const float4& q, int lane,
-                                                F&& f) {
+__device__ __forceinline__ void for_linked_lane(const ClusterItem& g, const float4& q, int lane, F&& f) {
     if (lane >= 27) return;
     const float p3[3] = {q.x, q.y, q.z};
     const int3 c = link_cell(p3, g.inv_cell);
     const int h = cell_hash(c.x + lane % 3 - 1, c.y + (lane / 3) % 3 - 1, c.z + lane / 9 - 1, g.hmask);
-    const int e = start[h + 1];
-    for (int u = start[h]; u < e; ++u) {
+    const float4* spts = g.spts;
+    const float link2 = g.link2;
+    const int e = g.start[h + 1];
+    for (int u = g.start[h]; u < e; ++u) {
         const float4 o = spts[u];
         const float ex = o.x - q.x, ey = o.y - q.y, ez = o.z - q.z;
-        if (ex * ex + ey * ey + ez * ez <= g.link2) f(__float_as_int(o.w));
+        if (ex * ex + ey * ey + ez * ez <= link2) f(__float_as_int(o.w));
     }
 }
 
@@ -606,71 +744,61 @@ __device__ __forceinline__ void for_linked_lane(const ClusterArgs& g, const int*
 // builds a shallow forest (each point under its lowest-index linked point); after a flattening
 // pass each further round joins neighbouring trees, so their number falls quickly and the
 // lock-free unions that follow have little left to do.
-__global__ void cl_hook_kernel(ClusterArgs g, const int* __restrict__ start, const float4* __restrict__ spts,
-                               int n_buckets) {
+__global__ void __launch_bounds__(256) cl_hook_kernel(const ClusterItem* __restrict__ items) {
+    const ClusterItem& g = items[blockIdx.y];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (w >= start[n_buckets]) return;                  // warp-uniform
-    const float4 q = spts[w];
-    const int ri = __ldcg(g.parent + __float_as_int(q.w));
+    if (w >= g.start[g.n_buckets]) return;              // warp-uniform
+    const float4 q = g.spts[w];
+    int* parent = g.parent;
+    const int ri = __ldcg(parent + __float_as_int(q.w));
     int m = ri;
-    for_linked_lane(g, start, spts, q, lane, [&](int j) { m = min(m, __ldcg(g.parent + j)); });
+    for_linked_lane(g, q, lane, [&](int j) { m = min(m, __ldcg(parent + j)); });
     m = __reduce_min_sync(0xffffffffu, m);
-    if (lane == 0 && m < ri) atomicMin(g.parent + ri, m);
+    if (lane == 0 && m < ri) atomicMin(parent + ri, m);
 }
 
 // Points every clustered point at the root of its tree (each thread writes only its own entry;
 // a concurrent write elsewhere only shortens the walk), so that most linked pairs are seen to
 // share a tree by one comparison.
-__global__ void cl_flatten_kernel(ClusterArgs g, const int* __restrict__ start, const float4* __restrict__ spts,
-                                  int n_buckets) {
+__global__ void __launch_bounds__(256) cl_flatten_kernel(const ClusterItem* __restrict__ items) {
+    const ClusterItem& g = items[blockIdx.y];
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= start[n_buckets]) return;
-    const int i = __float_as_int(spts[t].w);
-    int r = __ldcg(g.parent + i);
-    for (int next; (next = __ldcg(g.parent + r)) < r;) r = next;
-    g.parent[i] = r;
+    if (t >= g.start[g.n_buckets]) return;
+    const int i = __float_as_int(g.spts[t].w);
+    int* parent = g.parent;
+    int r = __ldcg(parent + i);
+    for (int next; (next = __ldcg(parent + r)) < r;) r = next;
+    parent[i] = r;
 }
 
-__global__ void cl_union_kernel(ClusterArgs g, const int* __restrict__ start, const float4* __restrict__ spts,
-                                int n_buckets) {
+__global__ void __launch_bounds__(256) cl_union_kernel(const ClusterItem* __restrict__ items) {
+    const ClusterItem& g = items[blockIdx.y];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (w >= start[n_buckets]) return;                  // warp-uniform
-    const float4 q = spts[w];
+    if (w >= g.start[g.n_buckets]) return;              // warp-uniform
+    const float4 q = g.spts[w];
     const int i = __float_as_int(q.w);
+    int* parent = g.parent;
     bool ok = true;
-    for_linked_lane(g, start, spts, q, lane, [&](int j) {
+    for_linked_lane(g, q, lane, [&](int j) {
         // components only ever merge, so equal parents mean the pair is already joined
-        if (j > i && __ldcg(g.parent + i) != __ldcg(g.parent + j)) ok = uf_unite(g.parent, i, j) && ok;
+        if (j > i && __ldcg(parent + i) != __ldcg(parent + j)) ok = uf_unite(parent, i, j) && ok;
     });
-    if (!ok) atomicOr(g.err, kErrUnion);
+    if (!ok) atomicOr(g.status, kErrUnion);
 }
 
-struct StatsArgs {
-    const float* pts;
-    const float* score;
-    const int* key;
-    int* parent;
-    int n;
-    int* root;               // [n]
-    int* cid;                // [n] cluster id of a root (order of discovery)
-    int* n_clusters;         // counter
-    double* s2;              // [n] per root
-    double* sx;              // [n][3] per root
-    int* size;               // [n] per root
-};
-
-__global__ void cl_root_kernel(StatsArgs g) {
+// Roots, cluster ids (from a counter, so in any order: everything below depends only on the ranking,
+// which is unique) and the sums of each cluster in float64.
+__global__ void __launch_bounds__(256) cl_stats_kernel(const ClusterItem* __restrict__ items) {
+    const ClusterItem& g = items[blockIdx.y];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.n) return;
     const int r = g.key[i] < 0 ? -1 : uf_find(g.parent, i);
     g.root[i] = r;
-    if (r == i) g.cid[i] = atomicAdd(g.n_clusters, 1);
-}
-
-__global__ void cl_stats_kernel(StatsArgs g) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.n) return;
-    const int r = g.root[i];
+    if (r == i) {
+        const int c = atomicAdd(g.status + 1, 1);
+        g.cid[i] = c;
+        g.c_first[c] = i;
+    }
     if (r < 0) return;
     const double s = g.score[i];
     atomicAdd(g.s2 + r, s * s);
@@ -678,50 +806,24 @@ __global__ void cl_stats_kernel(StatsArgs g) {
     atomicAdd(g.size + r, 1);
 }
 
-// Cluster ids come from a counter, so their order is arbitrary; everything below depends on the
-// ranking (score, then lowest index) only, which is unique.
-struct RankArgs {
-    const int* cid;
-    const int* n_clusters;
-    const double* s2;
-    const double* sx;
-    const int* size;
-    int n;
-    double* c_s2;            // [n] by cluster id
-    int* c_first;            // [n]
-    int* rank;               // [n] rank of cluster id
-    float* out_score;        // [n] by rank
-    float* out_center;       // [n][3]
-    int* out_size;
-    int* out_first;
-    const int* root;
-    int* cluster;            // [n] per point
-};
-
-__global__ void cl_compact_kernel(RankArgs g) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.n || g.root[i] != i) return;
-    const int c = g.cid[i];
-    g.c_s2[c] = g.s2[i];
-    g.c_first[c] = i;
-}
-
 // rank of cluster c = the number of clusters sorting before it (score desc, first index asc)
-__global__ void __launch_bounds__(256) cl_rank_kernel(RankArgs g) {
+__global__ void __launch_bounds__(256) cl_rank_kernel(const ClusterItem* __restrict__ items) {
     __shared__ double s_s[256];
     __shared__ int s_f[256];
-    const int K = *g.n_clusters;
+    const ClusterItem& g = items[blockIdx.y];
+    const int K = g.status[1];
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (blockIdx.x * blockDim.x >= K) return;           // block-uniform
-    const double sc = c < K ? g.c_s2[c] : 0.0;
+    if ((int)(blockIdx.x * blockDim.x) >= K) return;    // block-uniform
     const int fc = c < K ? g.c_first[c] : 0;
+    const double sc = c < K ? g.s2[fc] : 0.0;
     int r = 0;
     for (int base = 0; base < K; base += 256) {
         __syncthreads();
         const int t = base + threadIdx.x;
         if (t < K) {
-            s_s[threadIdx.x] = g.c_s2[t];
-            s_f[threadIdx.x] = g.c_first[t];
+            const int f = g.c_first[t];
+            s_f[threadIdx.x] = f;
+            s_s[threadIdx.x] = g.s2[f];
         }
         __syncthreads();
         const int m = min(256, K - base);
@@ -730,18 +832,19 @@ __global__ void __launch_bounds__(256) cl_rank_kernel(RankArgs g) {
     if (c < K) g.rank[c] = r;
 }
 
-__global__ void cl_output_kernel(RankArgs g) {
+__global__ void __launch_bounds__(256) cl_output_kernel(const ClusterItem* __restrict__ items) {
+    const ClusterItem& g = items[blockIdx.y];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.n) return;
     const int r = g.root[i];
     g.cluster[i] = r < 0 ? -1 : g.rank[g.cid[r]];
     if (r != i) return;
-    const int k = g.rank[g.cid[i]];
-    const int m = g.size[i];
-    g.out_score[k] = (float)g.s2[i];
-    for (int c = 0; c < 3; ++c) g.out_center[3 * (size_t)k + c] = (float)(g.sx[3 * (size_t)i + c] / m);
-    g.out_size[k] = m;
-    g.out_first[k] = i;
+    const int k = g.rank[g.cid[i]], m = g.size[i];
+    const size_t K = (size_t)g.status[1];
+    g.out[k] = (float)g.s2[i];
+    for (int c = 0; c < 3; ++c) g.out[K + 3 * (size_t)k + c] = (float)(g.sx[3 * (size_t)i + c] / m);
+    reinterpret_cast<int*>(g.out)[4 * K + k] = m;
+    reinterpret_cast<int*>(g.out)[5 * K + k] = i;
 }
 
 // ------------------------------------------------------------------------- host side ---
@@ -860,11 +963,7 @@ struct pv_clusters {
     int device = 0;
     Pool pool;
     int n = 0, K = 0;
-    int* cluster = nullptr;
-    float* score = nullptr;
-    float* center = nullptr;
-    int* size = nullptr;
-    int* first = nullptr;
+    int* data = nullptr;      // cluster [n], then score [K], center [K][3], size [K], first [K]
 };
 
 extern "C" pv_status pv_pocket_params_default(pv_pocket_params* p) {
@@ -880,8 +979,35 @@ extern "C" pv_status pv_pocket_params_default(pv_pocket_params* p) {
 
 namespace {
 
-// One receptor of a surface call, through its three phases: prepare (host checks, binning grid),
-// issue (everything up to the point count, asynchronous) and finish (the points, once counted).
+// Host and device memory laid out alike, filled on the host and uploaded by one copy.
+struct Staging {
+    std::vector<char> host;
+    size_t take(size_t bytes) {
+        const size_t at = (host.size() + 15) & ~(size_t)15;
+        host.resize(at + bytes);
+        return at;
+    }
+    size_t put(const void* p, size_t bytes) {
+        const size_t at = take(bytes);
+        std::memcpy(host.data() + at, p, bytes);
+        return at;
+    }
+};
+
+// Offsets of arrays in one allocation (256-byte aligned).
+struct Carve {
+    size_t bytes = 0;
+    template <typename T>
+    size_t take(size_t count) {
+        const size_t at = (bytes + 255) & ~(size_t)255;
+        bytes = at + count * sizeof(T);
+        return at;
+    }
+};
+
+constexpr int kMaxGridY = 65535;   // items per launch
+
+// One receptor of a surface call on the host.
 struct SurfaceJob {
     const pv_receptor* r = nullptr;
     const float* radius = nullptr;
@@ -890,71 +1016,18 @@ struct SurfaceJob {
     AtomGrid G{};
     long long n_cells = 0;
     pv_surface* S = nullptr;
-    Pool scratch;
-    float4* atoms = nullptr;
-    float* arad = nullptr;
-    int* key = nullptr;
-    int* slot_elem = nullptr;
-    int* order = nullptr;
-    float* d_dirs = nullptr;
-    uint32_t* kept = nullptr;
-    int* n_kept = nullptr;
-    int* offset = nullptr;
 };
 
-void release_jobs(std::vector<SurfaceJob>& jobs) {
-    for (SurfaceJob& J : jobs) {
-        J.scratch.release();
-        if (J.S) {
-            J.S->pool.release();
-            delete J.S;
-            J.S = nullptr;
-        }
-    }
-}
-
-// Host checks and the binning grid of one receptor; device-resident coordinates (and radii) are
-// read back for the bounding box.
-pv_status surface_prepare(pv_context* ctx, cudaStream_t st, SurfaceJob& J) {
+pv_status surface_check(pv_context* ctx, const SurfaceJob& J) {
     const pv_receptor* r = J.r;
     if (!r || r->n_atoms < 1 || r->n_atoms > kMaxAtoms) return fail(ctx, PV_ERR_ARG, "receptor atom count must be in [1, 200000]");
     if (!r->xyz || (!J.radius && !r->element)) return fail(ctx, PV_ERR_ARG, "receptor xyz and element (or radii) required");
     if (r->mem != PV_MEM_HOST && r->mem != PV_MEM_DEVICE) return fail(ctx, PV_ERR_ARG, "receptor mem kind");
-    const int n = J.n = r->n_atoms;
-    std::vector<float> hx;
-    const float* xyz_h = r->xyz;
-    if (r->mem == PV_MEM_DEVICE) {
-        hx.resize(3 * (size_t)n);
-        cudaError_t e = cudaMemcpyAsync(hx.data(), r->xyz, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "receptor read");
-        xyz_h = hx.data();
-    }
-    // the largest vdW radius bounds how far a neighbouring sphere can reach
-    if (J.radius) {
-        std::vector<float> hr;
-        const float* rad_h = J.radius;
-        if (r->mem == PV_MEM_DEVICE) {
-            hr.resize(n);
-            cudaError_t e = cudaMemcpyAsync(hr.data(), J.radius, sizeof(float) * n, cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "radius read");
-            rad_h = hr.data();
-        }
-        J.r_max = 0.f;
-        for (int i = 0; i < n; ++i) {
-            if (!(rad_h[i] > 0.f && rad_h[i] <= 10.f)) return fail(ctx, PV_ERR_ARG, "atom radius must be in (0, 10] A");
-            J.r_max = std::max(J.r_max, rad_h[i]);
-        }
-    }
-    double lo[3] = {1e30, 1e30, 1e30}, hi[3] = {-1e30, -1e30, -1e30};
-    for (int i = 0; i < n; ++i)
-        for (int k = 0; k < 3; ++k) {
-            const double v = xyz_h[3 * i + k];
-            if (!std::isfinite(v) || std::fabs(v) > 1e6) return fail(ctx, PV_ERR_ARG, "receptor coordinates must be finite (|x| <= 1e6 A)");
-            lo[k] = std::min(lo[k], v);
-            hi[k] = std::max(hi[k], v);
-        }
+    return PV_OK;
+}
+
+// The binning grid of a receptor from its bounding box.
+pv_status surface_grid(pv_context* ctx, SurfaceJob& J, const double lo[3], const double hi[3]) {
     J.n_cells = 1;
     for (int k = 0; k < 3; ++k) {
         J.G.lo[k] = (float)(lo[k] - 0.5);
@@ -966,99 +1039,219 @@ pv_status surface_prepare(pv_context* ctx, cudaStream_t st, SurfaceJob& J) {
     return PV_OK;
 }
 
-// Everything up to the point count, issued on the stream; the receptor's error word and point
-// count are copied to status[0] and status[1] (device memory).
-cudaError_t surface_issue(pv_context* ctx, cudaStream_t st, int dev, const pv_pocket_params* p,
-                          const std::vector<float>& dirs, SurfaceJob& J, int* status, const char** stage) {
-    const pv_receptor* r = J.r;
-    const int n = J.n, ns = p->n_sphere;
-    pv_surface* S = J.S = new (std::nothrow) pv_surface();
-    if (!S) return cudaErrorMemoryAllocation;
-    S->ctx = ctx;
-    S->device = dev;
-    S->pool.init(st, dev);
-    S->n_atoms = n;
-    S->n_sphere = ns;
-    S->G = J.G;
-    J.scratch.init(st, dev);
-    Pool& sc = J.scratch;
-    const float* d_xyz = r->xyz;
-    const uint8_t* d_el = r->element;
-    const float* d_rad = J.radius;
-    if (r->mem == PV_MEM_HOST) {
-        d_xyz = sc.take<float>(3 * (size_t)n);
-        d_el = r->element ? sc.take<uint8_t>(n) : nullptr;
-        d_rad = J.radius ? sc.take<float>(n) : nullptr;
+// Validity and bounding box of every receptor: host arrays are read here, device-resident ones by one
+// launch for all of them and one readback.
+pv_status surface_prepare(pv_context* ctx, cudaStream_t st, int dev, std::vector<SurfaceJob>& jobs) {
+    std::vector<BoundsItem> items;
+    for (SurfaceJob& J : jobs) {
+        const pv_status s = surface_check(ctx, J);
+        if (s != PV_OK) return s;
+        J.n = J.r->n_atoms;
+        if (J.r->mem == PV_MEM_DEVICE) items.push_back(BoundsItem{J.r->xyz, J.radius, J.n});
     }
-    J.atoms = sc.take<float4>(n);
-    J.arad = sc.take<float>(n);
-    J.key = sc.take<int>(n + 1);   // n + 1: reused for a scan when the points are ordered
-    int* count = sc.take<int>(J.n_cells);
-    int* cursor = sc.take<int>(J.n_cells);
-    J.slot_elem = sc.take<int>(n);
-    J.order = sc.take<int>(n);
-    int* err = sc.take<int>(1);
-    J.d_dirs = sc.take<float>(3 * (size_t)ns);
-    J.kept = sc.take<uint32_t>(32 * (size_t)n);
-    J.n_kept = sc.take<int>(n);
-    J.offset = sc.take<int>(n + 1);
-    S->sorted = S->pool.take<float4>(n);
-    S->cell_start = S->pool.take<int>(J.n_cells + 1);
-    cudaError_t e = sc.err != cudaSuccess ? sc.err : S->pool.err;
-    *stage = "allocation";
-    auto step = [&](cudaError_t x, const char* what) {
-        if (e == cudaSuccess && x != cudaSuccess) { e = x; *stage = what; }
-    };
-    if (e == cudaSuccess && r->mem == PV_MEM_HOST) {
-        step(cudaMemcpyAsync((void*)d_xyz, r->xyz, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, st), "receptor upload");
-        if (d_el) step(cudaMemcpyAsync((void*)d_el, r->element, n, cudaMemcpyHostToDevice, st), "receptor upload");
-        if (d_rad) step(cudaMemcpyAsync((void*)d_rad, J.radius, sizeof(float) * n, cudaMemcpyHostToDevice, st), "radius upload");
+    std::vector<float> found(8 * items.size());
+    if (!items.empty()) {
+        Pool pool(st, dev);
+        Carve c;
+        const size_t o_items = c.take<BoundsItem>(items.size()), o_out = c.take<float>(found.size());
+        char* d = pool.take<char>(c.bytes);
+        cudaError_t e = pool.err;
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(d + o_items, items.data(), sizeof(BoundsItem) * items.size(), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) {
+            bounds_kernel<<<(unsigned)items.size(), 1024, 0, st>>>((const BoundsItem*)(d + o_items), (float*)(d + o_out));
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(found.data(), d + o_out, sizeof(float) * found.size(), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        pool.release();
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "receptor read");
     }
-    if (e == cudaSuccess) {
-        step(cudaMemcpyAsync(J.d_dirs, dirs.data(), sizeof(float) * dirs.size(), cudaMemcpyHostToDevice, st), "lattice upload");
-        step(cudaMemsetAsync(count, 0, sizeof(int) * J.n_cells, st), "memset");
-        step(cudaMemsetAsync(err, 0, sizeof(int), st), "memset");
+    const float* f = found.data();
+    for (SurfaceJob& J : jobs) {
+        double lo[3] = {1e30, 1e30, 1e30}, hi[3] = {-1e30, -1e30, -1e30};
+        bool bad_radius = false, bad_xyz = false;
+        float r_max = 0.f;
+        if (J.r->mem == PV_MEM_DEVICE) {
+            int err;
+            std::memcpy(&err, f + 7, sizeof(int));
+            bad_radius = (err & kErrRadius) != 0;
+            bad_xyz = (err & kErrCoord) != 0;
+            for (int k = 0; k < 3; ++k) {
+                lo[k] = f[k];
+                hi[k] = f[3 + k];
+            }
+            r_max = f[6];
+            f += 8;
+        } else {
+            const float* x = J.r->xyz;
+            for (int i = 0; i < J.n; ++i)
+                for (int k = 0; k < 3; ++k) {
+                    const double v = x[3 * (size_t)i + k];
+                    bad_xyz = bad_xyz || !(std::fabs(v) <= 1e6);
+                    lo[k] = std::min(lo[k], v);
+                    hi[k] = std::max(hi[k], v);
+                }
+            if (J.radius)
+                for (int i = 0; i < J.n; ++i) {
+                    bad_radius = bad_radius || !(J.radius[i] > 0.f && J.radius[i] <= 10.f);
+                    r_max = std::max(r_max, J.radius[i]);
+                }
+        }
+        if (bad_radius) return fail(ctx, PV_ERR_ARG, "atom radius must be in (0, 10] A");
+        if (bad_xyz) return fail(ctx, PV_ERR_ARG, "receptor coordinates must be finite (|x| <= 1e6 A)");
+        if (J.radius) J.r_max = r_max;   // bounds how far a neighbouring sphere can reach
+        const pv_status s = surface_grid(ctx, J, lo, hi);
+        if (s != PV_OK) return s;
     }
-    if (e == cudaSuccess) {
-        prep_atoms_kernel<<<(n + 255) / 256, 256, 0, st>>>(d_xyz, d_el, d_rad, p->probe, n, J.G, J.atoms, J.arad, J.key,
-                                                            count, err);
-        step(cudaGetLastError(), "atom preparation");
-        step(bin_keys(J.key, n, (int)J.n_cells, count, S->cell_start, cursor, J.slot_elem, J.order, st), "atom binning");
-        gather_atoms_kernel<<<(n + 255) / 256, 256, 0, st>>>(J.order, n, J.atoms, S->sorted);
-        step(cudaGetLastError(), "atom binning");
-    }
-    if (e == cudaSuccess) {
-        SasArgs a{J.atoms, S->sorted, J.arad, S->cell_start, J.G, J.d_dirs, n, ns, J.r_max + p->probe + 1e-3f,
-                  J.kept, J.n_kept};
-        sas_kernel<<<(n + kSasWarps - 1) / kSasWarps, kSasWarps * 32, 0, st>>>(a);
-        step(cudaGetLastError(), "surface points");
-        scan_kernel<<<1, 1024, 0, st>>>(J.n_kept, n, J.offset);
-        step(cudaGetLastError(), "surface points");
-        step(cudaMemcpyAsync(status, err, sizeof(int), cudaMemcpyDeviceToDevice, st), "readback");
-        step(cudaMemcpyAsync(status + 1, J.offset + n, sizeof(int), cudaMemcpyDeviceToDevice, st), "readback");
-    }
-    return e;
+    return PV_OK;
 }
 
-// Once the point count is known: the points in (atom, k) order, their sources, and the order in
-// which the feature kernel groups them; the scratch goes back to the pool in stream order.
-cudaError_t surface_finish(cudaStream_t st, const pv_pocket_params* p, SurfaceJob& J, int total, const char** stage) {
-    pv_surface* S = J.S;
-    const int n = J.n, ns = p->n_sphere;
-    S->n_points = total;
-    S->points = S->pool.take<float>(3 * (size_t)(total > 0 ? total : 1));
-    S->src = S->pool.take<int>(total > 0 ? total : 1);
-    S->perm = S->pool.take<int>(total > 0 ? total : 1);
+// All receptors from their atoms to their points. The working memory of the call is one allocation;
+// each surface keeps two (binned atoms; points). *bad: error bits found on the device.
+cudaError_t surface_build(pv_context* ctx, cudaStream_t st, int dev, const pv_pocket_params* p,
+                          std::vector<SurfaceJob>& jobs, Pool& scratch, int* bad, const char** stage) {
+    const int k = (int)jobs.size(), ns = p->n_sphere;
+    // lattice directions (spherical Fibonacci lattice, evaluated in double)
+    std::vector<float> dirs(3 * (size_t)ns);
+    const double golden_angle = kPi * (3.0 - std::sqrt(5.0));
+    for (int j = 0; j < ns; ++j) {
+        const double z = 1.0 - (2.0 * j + 1.0) / ns, rho = std::sqrt(std::max(0.0, 1.0 - z * z));
+        dirs[3 * j] = (float)(rho * std::cos(golden_angle * j));
+        dirs[3 * j + 1] = (float)(rho * std::sin(golden_angle * j));
+        dirs[3 * j + 2] = (float)z;
+    }
+    // uploaded: records, directions, host receptors
+    Staging up;
+    const size_t o_items = up.take(sizeof(SurfaceItem) * k), o_dirs = up.put(dirs.data(), sizeof(float) * dirs.size());
+    std::vector<size_t> o_xyz(k), o_el(k), o_rad(k);
+    Carve zero, work;        // cleared; written before it is read
+    const size_t o_status = zero.take<int>(2 * (size_t)k);
+    std::vector<size_t> o_count(k), o_head(k), o_atoms(k), o_arad(k), o_key(k), o_next(k), o_order(k), o_kept(k), o_nkept(k),
+        o_off(k), o_offs(k);
+    int n_max = 0;
+    for (int j = 0; j < k; ++j) {
+        const SurfaceJob& J = jobs[j];
+        const size_t n = J.n;
+        n_max = std::max(n_max, J.n);
+        if (J.r->mem == PV_MEM_HOST) {
+            o_xyz[j] = up.put(J.r->xyz, sizeof(float) * 3 * n);
+            if (J.r->element && !J.radius) o_el[j] = up.put(J.r->element, n);
+            if (J.radius) o_rad[j] = up.put(J.radius, sizeof(float) * n);
+        }
+        o_count[j] = zero.take<int>(J.n_cells);
+        o_head[j] = zero.take<int>(J.n_cells);
+        o_atoms[j] = work.take<float4>(n);
+        o_arad[j] = work.take<float>(n);
+        o_key[j] = work.take<int>(n);
+        o_next[j] = work.take<int>(n);
+        o_order[j] = work.take<int>(n);
+        o_kept[j] = work.take<uint32_t>(32 * n);
+        o_nkept[j] = work.take<int>(n);
+        o_off[j] = work.take<int>(n + 1);
+        o_offs[j] = work.take<int>(n + 1);
+    }
+    Carve all;
+    const size_t a_up = all.take<char>(up.host.size()), a_zero = all.take<char>(zero.bytes), a_work = all.take<char>(work.bytes);
+    *stage = "allocation";
+    char* d = scratch.take<char>(all.bytes);
+    if (!d) return scratch.err;
+    char *d_up = d + a_up, *d_zero = d + a_zero, *d_work = d + a_work;
+    std::vector<SurfaceItem> items(k);
+    for (int j = 0; j < k; ++j) {
+        SurfaceJob& J = jobs[j];
+        const size_t n = J.n;
+        pv_surface* S = J.S = new (std::nothrow) pv_surface();
+        if (!S) return cudaErrorMemoryAllocation;
+        S->ctx = ctx;
+        S->device = dev;
+        S->pool.init(st, dev);
+        S->n_atoms = J.n;
+        S->n_sphere = ns;
+        S->G = J.G;
+        Carve c;
+        const size_t o_sorted = c.take<float4>(n), o_start = c.take<int>(J.n_cells + 1), o_srad = c.take<float>(n);
+        char* keep = S->pool.take<char>(c.bytes);
+        if (!keep) return S->pool.err;
+        S->sorted = (float4*)(keep + o_sorted);
+        S->cell_start = (int*)(keep + o_start);
+        SurfaceItem& g = items[j];
+        const bool host = J.r->mem == PV_MEM_HOST;
+        g.xyz = host ? (const float*)(d_up + o_xyz[j]) : J.r->xyz;
+        g.element = host ? (const uint8_t*)(d_up + o_el[j]) : J.r->element;
+        g.radius = !J.radius ? nullptr : host ? (const float*)(d_up + o_rad[j]) : J.radius;
+        g.n = J.n;
+        g.n_cells = (int)J.n_cells;
+        g.G = J.G;
+        g.reach_max = J.r_max + p->probe + 1e-3f;
+        g.atoms = (float4*)(d_work + o_atoms[j]);
+        g.arad = (float*)(d_work + o_arad[j]);
+        g.key = (int*)(d_work + o_key[j]);
+        g.count = (int*)(d_zero + o_count[j]);
+        g.head = (int*)(d_zero + o_head[j]);
+        g.next = (int*)(d_work + o_next[j]);
+        g.cell_start = S->cell_start;
+        g.sorted = S->sorted;
+        g.srad = (float*)(keep + o_srad);
+        g.order = (int*)(d_work + o_order[j]);
+        g.kept = (uint32_t*)(d_work + o_kept[j]);
+        g.n_kept = (int*)(d_work + o_nkept[j]);
+        g.offset = (int*)(d_work + o_off[j]);
+        g.offset_sorted = (int*)(d_work + o_offs[j]);
+        g.pts = nullptr;
+        g.src = nullptr;
+        g.perm = nullptr;
+        g.status = (int*)(d_zero + o_status) + 2 * j;
+    }
+    std::memcpy(up.host.data() + o_items, items.data(), sizeof(SurfaceItem) * k);
+    SurfaceItem* d_items = (SurfaceItem*)(d_up + o_items);
+    const float* d_dirs = (const float*)(d_up + o_dirs);
+    *stage = "receptor upload";
+    cudaError_t e = cudaMemcpyAsync(d_up, up.host.data(), up.host.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_zero, 0, zero.bytes, st);
+    if (e != cudaSuccess) return e;
+    *stage = "surface points";
+    const unsigned b256 = (n_max + 255) / 256, bw = (n_max + kSasWarps - 1) / kSasWarps;
+    for (int y0 = 0; y0 < k; y0 += kMaxGridY) {
+        const unsigned ny = std::min(kMaxGridY, k - y0);
+        const SurfaceItem* it = d_items + y0;
+        prep_atoms_kernel<<<dim3(b256, ny), 256, 0, st>>>(it, p->probe);
+        cell_scan_kernel<<<dim3(1, ny), 1024, 0, st>>>(it);
+        sort_atoms_kernel<<<dim3(b256, ny), 256, 0, st>>>(it);
+        sas_kernel<<<dim3(bw, ny), kSasWarps * 32, 0, st>>>(it, d_dirs, ns);
+        point_scan_kernel<<<dim3(2, ny), 1024, 0, st>>>(it);
+    }
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    // one readback of all error words and point counts
+    *stage = "readback";
+    std::vector<int> status(2 * (size_t)k, 0);
+    e = cudaMemcpyAsync(status.data(), d_zero + o_status, sizeof(int) * status.size(), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    for (int j = 0; j < k; ++j) *bad |= status[2 * j];
+    if (*bad) return cudaSuccess;
+    // the points, their sources and the order in which the feature kernel groups them
     *stage = "point allocation";
-    if (S->pool.err != cudaSuccess) return S->pool.err;
-    sas_write_kernel<<<(n + 3) / 4, 128, 0, st>>>(J.atoms, J.arad, J.d_dirs, n, ns, J.kept, J.offset, S->points, S->src);
-    // the point order of the feature kernel: atoms in cell order (slot_elem and key are free again)
-    sorted_counts_kernel<<<(n + 255) / 256, 256, 0, st>>>(J.order, J.n_kept, n, J.slot_elem);
-    scan_kernel<<<1, 1024, 0, st>>>(J.slot_elem, n, J.key);
-    perm_kernel<<<(n + 255) / 256, 256, 0, st>>>(J.order, J.n_kept, J.offset, J.key, n, S->perm);
+    for (int j = 0; j < k; ++j) {
+        pv_surface* S = jobs[j].S;
+        S->n_points = status[2 * j + 1];
+        const size_t m = S->n_points > 0 ? S->n_points : 1;
+        Carve c;
+        const size_t o_pts = c.take<float>(3 * m), o_src = c.take<int>(m), o_perm = c.take<int>(m);
+        char* keep = S->pool.take<char>(c.bytes);
+        if (!keep) return S->pool.err;
+        items[j].pts = S->points = (float*)(keep + o_pts);
+        items[j].src = S->src = (int*)(keep + o_src);
+        items[j].perm = S->perm = (int*)(keep + o_perm);
+    }
     *stage = "point order";
-    cudaError_t e = cudaGetLastError();
-    J.scratch.release();
+    e = cudaMemcpyAsync(d_items, items.data(), sizeof(SurfaceItem) * k, cudaMemcpyHostToDevice, st);
+    for (int y0 = 0; y0 < k && e == cudaSuccess; y0 += kMaxGridY) {
+        sas_write_kernel<<<dim3((n_max + 3) / 4, std::min(kMaxGridY, k - y0)), 128, 0, st>>>(d_items + y0, d_dirs, ns);
+        e = cudaGetLastError();
+    }
     return e;
 }
 
@@ -1077,45 +1270,25 @@ extern "C" pv_status pv_surface_create_many(pv_context* ctx, int32_t n_receptors
     for (int j = 0; j < n_receptors; ++j) {
         jobs[j].r = receptors + j;
         jobs[j].radius = radii ? radii[j] : nullptr;
-        const pv_status s = surface_prepare(ctx, st, jobs[j]);
-        if (s != PV_OK) return s;
     }
-    // lattice directions (spherical Fibonacci lattice, evaluated in double)
-    const int ns = p->n_sphere;
-    std::vector<float> dirs(3 * (size_t)ns);
-    const double golden_angle = kPi * (3.0 - std::sqrt(5.0));
-    for (int k = 0; k < ns; ++k) {
-        const double z = 1.0 - (2.0 * k + 1.0) / ns, rho = std::sqrt(std::max(0.0, 1.0 - z * z));
-        dirs[3 * k] = (float)(rho * std::cos(golden_angle * k));
-        dirs[3 * k + 1] = (float)(rho * std::sin(golden_angle * k));
-        dirs[3 * k + 2] = (float)z;
-    }
-    // every receptor's work up to its point count, then one readback of all error words and counts
-    Pool batch(st, dev);
-    int* status = batch.take<int>(2 * (size_t)n_receptors);
-    cudaError_t e = batch.err;
-    const char* stage = "allocation";
-    for (int j = 0; j < n_receptors && e == cudaSuccess; ++j) e = surface_issue(ctx, st, dev, p, dirs, jobs[j], status + 2 * j, &stage);
-    std::vector<int> h_status(2 * (size_t)n_receptors, 0);
-    if (e == cudaSuccess) {
-        stage = "readback";
-        e = cudaMemcpyAsync(h_status.data(), status, sizeof(int) * h_status.size(), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    }
+    const pv_status ps = surface_prepare(ctx, st, dev, jobs);
+    if (ps != PV_OK) return ps;
+    Pool scratch(st, dev);
     int bad = 0;
-    for (int j = 0; j < n_receptors && e == cudaSuccess; ++j) bad |= h_status[2 * j];
-    if (e == cudaSuccess && bad) {
-        release_jobs(jobs);
-        batch.release();
+    const char* stage = "allocation";
+    cudaError_t e = scratch.err;
+    if (e == cudaSuccess) e = surface_build(ctx, st, dev, p, jobs, scratch, &bad, &stage);
+    scratch.release();   // stream-ordered: after the kernels above
+    if (e != cudaSuccess || bad) {
+        for (SurfaceJob& J : jobs)
+            if (J.S) {
+                J.S->pool.release();
+                delete J.S;
+            }
+        if (e != cudaSuccess) return cuda_fail(ctx, e, (std::string("surface: ") + stage).c_str());
         return fail(ctx, PV_ERR_ARG, (bad & kErrElement) ? "receptor element must be 0..3"
                                      : (bad & kErrRadius) ? "atom radius must be in (0, 10] A"
                                                           : "receptor coordinates must be finite");
-    }
-    for (int j = 0; j < n_receptors && e == cudaSuccess; ++j) e = surface_finish(st, p, jobs[j], h_status[2 * j + 1], &stage);
-    batch.release();
-    if (e != cudaSuccess) {
-        release_jobs(jobs);
-        return cuda_fail(ctx, e, (std::string("surface: ") + stage).c_str());
     }
     for (int j = 0; j < n_receptors; ++j) out[j] = jobs[j].S;
     return PV_OK;
@@ -1234,98 +1407,101 @@ extern "C" void pv_surface_destroy(pv_surface* s) {
 
 namespace {
 
-// Steps 4-5 for one point set, issued on the stream; its error word and cluster count are copied
-// to status[0] and status[1] (device memory). C is allocated here (released by the caller on error).
-cudaError_t cluster_issue(pv_context* ctx, cudaStream_t st, int dev, int n, const float* dev_xyz,
-                          const float* dev_score, const pv_pocket_params* p, pv_clusters** Cout, int* status,
-                          const char** stage) {
-    pv_clusters* C = *Cout = new (std::nothrow) pv_clusters();
+// Steps 4-5 for all point sets, issued on the stream; status[2 j], status[2 j + 1] (host) receive the
+// error word and the cluster count of set j.
+cudaError_t cluster_build(pv_context* ctx, cudaStream_t st, int dev, int k, const int32_t* n_points,
+                          const float* const* dev_xyz, const float* const* dev_score, const pv_pocket_params* p,
+                          std::vector<pv_clusters*>& cs, Pool& scratch, std::vector<int>& status, const char** stage) {
     *stage = "allocation";
-    if (!C) return cudaErrorMemoryAllocation;
-    C->ctx = ctx;
-    C->device = dev;
-    C->pool.init(st, dev);
-    C->n = n;
-    const size_t m = n > 0 ? (size_t)n : 1;
-    C->cluster = C->pool.take<int>(m);
-    C->score = C->pool.take<float>(m);
-    C->center = C->pool.take<float>(3 * m);
-    C->size = C->pool.take<int>(m);
-    C->first = C->pool.take<int>(m);
-    if (C->pool.err != cudaSuccess) return C->pool.err;
-    if (n == 0) return cudaMemsetAsync(status, 0, 2 * sizeof(int), st);
-    uint32_t buckets = 1024;
-    while (2 * buckets < (uint32_t)n) buckets <<= 1;
-    Pool scratch(st, dev);
-    int* key = scratch.take<int>(m);
-    int* count = scratch.take<int>(buckets);
-    int* start = scratch.take<int>(buckets + 1);
-    int* cursor = scratch.take<int>(buckets);
-    int* slot_elem = scratch.take<int>(m);
-    int* order = scratch.take<int>(m);
-    int* parent = scratch.take<int>(m);
-    int* err = scratch.take<int>(1);
-    int* root = scratch.take<int>(m);
-    int* cid = scratch.take<int>(m);
-    int* n_clusters = scratch.take<int>(1);
-    float4* spts = scratch.take<float4>(m);
-    double* s2 = scratch.take<double>(m);
-    double* sx = scratch.take<double>(3 * m);
-    int* size = scratch.take<int>(m);
-    double* c_s2 = scratch.take<double>(m);
-    int* c_first = scratch.take<int>(m);
-    int* rank = scratch.take<int>(m);
-    cudaError_t e = scratch.err;
-    auto step = [&](cudaError_t x, const char* what) {
-        if (e == cudaSuccess && x != cudaSuccess) { e = x; *stage = what; }
-    };
-    if (e == cudaSuccess) {
-        step(cudaMemsetAsync(count, 0, sizeof(int) * buckets, st), "memset");
-        step(cudaMemsetAsync(err, 0, sizeof(int), st), "memset");
-        step(cudaMemsetAsync(s2, 0, sizeof(double) * m, st), "memset");
-        step(cudaMemsetAsync(sx, 0, sizeof(double) * 3 * m, st), "memset");
-        step(cudaMemsetAsync(size, 0, sizeof(int) * m, st), "memset");
-        step(cudaMemsetAsync(n_clusters, 0, sizeof(int), st), "memset");
-    }
-    if (e == cudaSuccess) {
-        ClusterArgs a;
-        a.pts = dev_xyz;
-        a.score = dev_score;
-        a.n = n;
-        a.theta = p->threshold;
-        a.link2 = p->link * p->link;
-        // cells a little wider than the link so that linked points always sit in adjacent cells
-        a.inv_cell = (float)(1.0 / ((double)p->link * (1.0 + 1e-5)));
-        a.hmask = buckets - 1;
-        a.key = key;
-        a.count = count;
-        a.parent = parent;
-        a.err = err;
-        const int b = (n + 255) / 256;
-        cl_init_kernel<<<b, 256, 0, st>>>(a);
-        step(cudaGetLastError(), "cluster set-up");
-        step(bin_keys(key, n, (int)buckets, count, start, cursor, slot_elem, order, st), "point binning");
-        cl_gather_kernel<<<b, 256, 0, st>>>(order, dev_xyz, start + buckets, spts);
-        const int bw = (n + 7) / 8;                     // a warp per point: 8 points per CTA of 256
-        for (int round = 0; round < kHookRounds; ++round) {
-            cl_hook_kernel<<<bw, 256, 0, st>>>(a, start, spts, (int)buckets);
-            cl_flatten_kernel<<<b, 256, 0, st>>>(a, start, spts, (int)buckets);
+    Carve zero, work;        // cleared; written before it is read
+    const size_t o_items = work.take<ClusterItem>(k), o_status = zero.take<int>(2 * (size_t)k);
+    std::vector<ClusterItem> items(k);
+    int n_max = 0;
+    // two passes over the same layout: offsets first, then addresses in the one allocation
+    char *d_zero = nullptr, *d_work = nullptr;
+    for (int pass = 0; pass < 2; ++pass) {
+        if (pass == 1) {
+            Carve all;
+            const size_t a_zero = all.take<char>(zero.bytes), a_work = all.take<char>(work.bytes);
+            char* d = scratch.take<char>(all.bytes);
+            if (!d) return scratch.err;
+            d_zero = d + a_zero;
+            d_work = d + a_work;
+            zero = Carve();
+            work = Carve();
+            work.take<ClusterItem>(k);
+            zero.take<int>(2 * (size_t)k);
         }
-        cl_union_kernel<<<bw, 256, 0, st>>>(a, start, spts, (int)buckets);
-        step(cudaGetLastError(), "single linkage");
-        StatsArgs sa{dev_xyz, dev_score, key, parent, n, root, cid, n_clusters, s2, sx, size};
-        cl_root_kernel<<<b, 256, 0, st>>>(sa);
-        cl_stats_kernel<<<b, 256, 0, st>>>(sa);
-        step(cudaGetLastError(), "cluster sums");
-        RankArgs ra{cid, n_clusters, s2, sx, size, n, c_s2, c_first, rank, C->score, C->center, C->size, C->first, root, C->cluster};
-        cl_compact_kernel<<<b, 256, 0, st>>>(ra);
-        cl_rank_kernel<<<b, 256, 0, st>>>(ra);
-        cl_output_kernel<<<b, 256, 0, st>>>(ra);
-        step(cudaGetLastError(), "cluster ranking");
-        step(cudaMemcpyAsync(status, err, sizeof(int), cudaMemcpyDeviceToDevice, st), "readback");
-        step(cudaMemcpyAsync(status + 1, n_clusters, sizeof(int), cudaMemcpyDeviceToDevice, st), "readback");
+        for (int j = 0; j < k; ++j) {
+            const size_t m = n_points[j] > 0 ? n_points[j] : 1;
+            uint32_t buckets = 1024;
+            while (2 * buckets < (uint32_t)n_points[j]) buckets <<= 1;
+            ClusterItem& g = items[j];
+            g.n = n_points[j];
+            g.n_buckets = (int)buckets;
+            g.hmask = buckets - 1;
+            n_max = std::max(n_max, g.n);
+            g.count = (int*)(d_zero + zero.take<int>(buckets));
+            g.s2 = (double*)(d_zero + zero.take<double>(m));
+            g.sx = (double*)(d_zero + zero.take<double>(3 * m));
+            g.size = (int*)(d_zero + zero.take<int>(m));
+            g.start = (int*)(d_work + work.take<int>(buckets + 1));
+            g.key = (int*)(d_work + work.take<int>(m));
+            g.spts = (float4*)(d_work + work.take<float4>(m));
+            g.parent = (int*)(d_work + work.take<int>(m));
+            g.root = (int*)(d_work + work.take<int>(m));
+            g.cid = (int*)(d_work + work.take<int>(m));
+            g.c_first = (int*)(d_work + work.take<int>(m));
+            g.rank = (int*)(d_work + work.take<int>(m));
+        }
     }
-    scratch.release();   // stream-ordered: after the kernels above
+    for (int j = 0; j < k; ++j) {
+        pv_clusters* C = cs[j] = new (std::nothrow) pv_clusters();
+        if (!C) return cudaErrorMemoryAllocation;
+        C->ctx = ctx;
+        C->device = dev;
+        C->pool.init(st, dev);
+        C->n = n_points[j];
+        C->data = C->pool.take<int>(7 * (size_t)(C->n > 0 ? C->n : 1));
+        if (!C->data) return C->pool.err;
+        ClusterItem& g = items[j];
+        g.pts = dev_xyz[j];
+        g.score = dev_score[j];
+        g.theta = p->threshold;
+        g.link2 = p->link * p->link;
+        // cells a little wider than the link so that linked points always sit in adjacent cells
+        g.inv_cell = (float)(1.0 / ((double)p->link * (1.0 + 1e-5)));
+        g.status = (int*)(d_zero + o_status) + 2 * j;
+        g.cluster = C->data;
+        g.out = (float*)(C->data + C->n);
+    }
+    *stage = "memset";
+    cudaError_t e = cudaMemcpyAsync(d_work + o_items, items.data(), sizeof(ClusterItem) * k, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_zero, 0, zero.bytes, st);
+    if (e != cudaSuccess) return e;
+    *stage = "single linkage";
+    const unsigned b = (n_max + 255) / 256, bw = (n_max + 7) / 8;   // bw: a warp per point, 8 points per CTA
+    for (int y0 = 0; y0 < k && n_max > 0; y0 += kMaxGridY) {
+        const unsigned ny = std::min(kMaxGridY, k - y0);
+        const ClusterItem* it = (const ClusterItem*)(d_work + o_items) + y0;
+        cl_init_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
+        cl_scan_kernel<<<dim3(1, ny), 1024, 0, st>>>(it);
+        cl_place_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
+        for (int round = 0; round < kHookRounds; ++round) {
+            cl_hook_kernel<<<dim3(bw, ny), 256, 0, st>>>(it);
+            cl_flatten_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
+        }
+        cl_union_kernel<<<dim3(bw, ny), 256, 0, st>>>(it);
+        cl_stats_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
+        cl_rank_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
+        cl_output_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    // one readback of all error words and cluster counts
+    *stage = "readback";
+    e = cudaMemcpyAsync(status.data(), d_zero + o_status, sizeof(int) * status.size(), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     return e;
 }
 
@@ -1354,20 +1530,13 @@ extern "C" pv_status pv_cluster_points_many(pv_context* ctx, int32_t n_sets, con
                 C = nullptr;
             }
     };
-    // every set's work, then one readback of all error words and cluster counts
-    Pool batch(st, dev);
-    int* status = batch.take<int>(2 * (size_t)n_sets);
-    cudaError_t e = batch.err;
-    const char* stage = "allocation";
-    for (int j = 0; j < n_sets && e == cudaSuccess; ++j)
-        e = cluster_issue(ctx, st, dev, n_points[j], dev_xyz[j], dev_score[j], p, &cs[j], status + 2 * j, &stage);
+    Pool scratch(st, dev);
     std::vector<int> h_status(2 * (size_t)n_sets, 0);
-    if (e == cudaSuccess) {
-        stage = "readback";
-        e = cudaMemcpyAsync(h_status.data(), status, sizeof(int) * h_status.size(), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    }
-    batch.release();
+    cudaError_t e = scratch.err;
+    const char* stage = "allocation";
+    if (e == cudaSuccess)
+        e = cluster_build(ctx, st, dev, n_sets, n_points, dev_xyz, dev_score, p, cs, scratch, h_status, &stage);
+    scratch.release();   // stream-ordered: after the kernels above
     if (e != cudaSuccess) {
         release_all();
         return cuda_fail(ctx, e, (std::string("clusters: ") + stage).c_str());
@@ -1412,16 +1581,25 @@ extern "C" pv_status pv_clusters_read(pv_context* ctx, const pv_clusters* c, int
     if (!c || c->magic != kClustersMagic || c->ctx != ctx) return fail(ctx, PV_ERR_STATE, "clusters of another context");
     if (mem != PV_MEM_HOST && mem != PV_MEM_DEVICE) return fail(ctx, PV_ERR_ARG, "mem kind");
     DeviceGuard guard(dev);
-    const cudaMemcpyKind kind = mem == PV_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+    const size_t n = (size_t)c->n, K = (size_t)c->K;
+    const struct { void* dst; size_t at, count; } parts[5] = {
+        {cluster, 0, n}, {score, n, K}, {center, n + K, 3 * K}, {size, n + 4 * K, K}, {first, n + 5 * K, K}};
+    if (mem == PV_MEM_HOST) {   // one copy of the lot, without the points when they are not asked for
+        const size_t from = cluster ? 0 : n;
+        std::vector<int> all(n + 6 * K);
+        cudaError_t e = all.size() == from ? cudaSuccess
+                                           : cudaMemcpyAsync(all.data() + from, c->data + from,
+                                                             sizeof(int) * (all.size() - from), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "clusters read");
+        for (const auto& q : parts)
+            if (q.dst && q.count) std::memcpy(q.dst, all.data() + q.at, sizeof(int) * q.count);
+        return PV_OK;
+    }
     cudaError_t e = cudaSuccess;
-    auto copy = [&](void* dst, const void* srcp, size_t bytes) {
-        if (e == cudaSuccess && dst && bytes) e = cudaMemcpyAsync(dst, srcp, bytes, kind, st);
-    };
-    copy(cluster, c->cluster, sizeof(int) * (size_t)c->n);
-    copy(score, c->score, sizeof(float) * (size_t)c->K);
-    copy(center, c->center, sizeof(float) * 3 * (size_t)c->K);
-    copy(size, c->size, sizeof(int) * (size_t)c->K);
-    copy(first, c->first, sizeof(int) * (size_t)c->K);
+    for (const auto& q : parts)
+        if (e == cudaSuccess && q.dst && q.count)
+            e = cudaMemcpyAsync(q.dst, c->data + q.at, sizeof(int) * q.count, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     return e == cudaSuccess ? PV_OK : cuda_fail(ctx, e, "clusters read");
 }

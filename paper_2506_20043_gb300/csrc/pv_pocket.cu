@@ -39,7 +39,7 @@ constexpr float kCell = 4.0f;            // atom binning cell edge, A
 constexpr int kMaxAtoms = 200000;
 constexpr int kNb = 128;                 // neighbour list capacity per warp (SAS kernel)
 constexpr int kSasWarps = 4;
-constexpr int kFeatSplit = 16;           // warps sharing one group of 32 points (feature kernel)
+constexpr int kFeatSplit = 12;           // warps sharing one group of 32 points (feature kernel)
 constexpr int kFeatRows = 256;           // cell rows listed at a time by the feature kernel
 constexpr int kPropChunk = 8;            // property columns per feature launch row (a multiple of 4)
 constexpr double kPi = 3.14159265358979323846;
@@ -448,19 +448,31 @@ struct FeatArgs {
     int n_pts;
     const float* props;      // [n_atoms][n_props], input atom order
     int n_props;
-    float inv_rf, rf2, rp2, reach;
+    float inv_rf, rf2, rp2, reach, reach_f;   // reach: of either radius, reach_f: of the features
     float* feat;             // [n_pts][n_props]
     int* prot;               // [n_pts] or null
 };
+
+// The smallest of a warp's values, through the integer reduction on an order-preserving image.
+__device__ __forceinline__ float warp_min(float v) {
+    int i = __float_as_int(v);
+    i = __reduce_min_sync(0xffffffffu, i ^ ((i >> 31) & 0x7fffffff));
+    return __int_as_float(i ^ ((i >> 31) & 0x7fffffff));
+}
 
 // One CTA per group of 32 points. The cell rows within reach of the group's bounding box (each
 // row's x range trimmed to the box swept by the reach) are listed with their atom counts, up to
 // kFeatRows at a time, and the concatenated atoms of the listed rows are cut into chunks of 32:
 // the CTA's kFeatSplit warps take the chunks in turn (balanced to within one chunk), each loading
-// its next chunk into registers while it works on the current one; the partial sums are added in
-// shared memory at the end.
-__global__ void __launch_bounds__(kFeatSplit * 32) feature_kernel(FeatArgs g) {
-    __shared__ float4 s_at[kFeatSplit][32];
+// its next chunk into registers while it works on the current one, keeping of a chunk the atoms within
+// reach of the box (about half), those within the feature radius of it first, and testing two atoms at a
+// time in packed arithmetic; the partial sums are added in shared memory at the end.
+//
+// Bound by the latency of its phases at the warps that fit (registers): 12 warps by 3 CTAs per SM
+// measured best, 36 us for 8,000 atoms with 7 columns and 63 us with 20 (event-timed), against 42 and 89 us
+// for 16 warps by the 2 CTAs that 59 registers allow, 40 and 69 us for 8 warps by 4.
+__global__ void __launch_bounds__(kFeatSplit * 32, 3) feature_kernel(FeatArgs g) {
+    __shared__ float s_at[kFeatSplit][3][32];                 // a chunk's atoms, read two at a time
     __shared__ float4 s_pr[kFeatSplit][32][kPropChunk / 4];   // an atom's chunk: two broadcast loads
     __shared__ float s_red[kFeatSplit][kPropChunk + 1][32];
     __shared__ int s_beg[kFeatRows];                          // first atom of a listed row
@@ -479,21 +491,19 @@ __global__ void __launch_bounds__(kFeatSplit * 32) feature_kernel(FeatArgs g) {
     }
     // the group's bounding box (non-finite points take no part); every warp computes the same one
     const bool fin = live && isfinite(px) && isfinite(py) && isfinite(pz);
-    float lo3[3] = {fin ? px : INFINITY, fin ? py : INFINITY, fin ? pz : INFINITY};
-    float hi3[3] = {fin ? px : -INFINITY, fin ? py : -INFINITY, fin ? pz : -INFINITY};
+    const float pos[3] = {px, py, pz};
+    float lo3[3], hi3[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            lo3[k] = fminf(lo3[k], __shfl_xor_sync(0xffffffffu, lo3[k], o));
-            hi3[k] = fmaxf(hi3[k], __shfl_xor_sync(0xffffffffu, hi3[k], o));
-        }
+    for (int k = 0; k < 3; ++k) {
+        lo3[k] = warp_min(fin ? pos[k] : INFINITY);
+        hi3[k] = -warp_min(fin ? -pos[k] : INFINITY);
+    }
     float acc[kPropChunk];
 #pragma unroll
     for (int q = 0; q < kPropChunk; ++q) acc[q] = 0.f;
     int count = 0;
     if (lo3[0] <= hi3[0]) {                             // at least one finite point (CTA-uniform)
-        const float reach2 = g.reach * g.reach;
+        const float reach2 = g.reach * g.reach, feat2 = g.reach_f * g.reach_f;
         const float cell = 1.0f / g.G.inv_cell;
         int c0[3], c1[3];
 #pragma unroll
@@ -542,8 +552,9 @@ __global__ void __launch_bounds__(kFeatSplit * 32) feature_kernel(FeatArgs g) {
             __syncthreads();
             const int total = s_off[nr], n_chunks = (total + 31) >> 5;
             // the atom at list position p: its row by binary search over the offsets
-            auto fetch = [&](int c, float4& B, float (&v)[kPropChunk]) {
+            auto fetch = [&](int c, float4& B, int& kind, float (&v)[kPropChunk]) {
                 const int p = c * 32 + lane;
+                kind = 0;
                 if (p < total) {
                     int lo = 0, hi = nr - 1;                // the last row with s_off[row] <= p
                     while (lo < hi) {
@@ -552,35 +563,64 @@ __global__ void __launch_bounds__(kFeatSplit * 32) feature_kernel(FeatArgs g) {
                         else hi = mid - 1;
                     }
                     B = g.sorted[s_beg[lo] + (p - s_off[lo])];
-                    const float* pr = g.props + (size_t)__float_as_int(B.w) * g.n_props + q0;
+                    const float ex = fmaxf(0.f, fmaxf(lo3[0] - B.x, B.x - hi3[0])), ey = fmaxf(0.f, fmaxf(lo3[1] - B.y, B.y - hi3[1])),
+                                ez = fmaxf(0.f, fmaxf(lo3[2] - B.z, B.z - hi3[2]));
+                    const float e2 = ex * ex + ey * ey + ez * ez;
+                    kind = e2 < feat2 ? 2 : (e2 < reach2 ? 1 : 0);
+                    if (kind == 2) {
+                        const float* pr = g.props + (size_t)__float_as_int(B.w) * g.n_props + q0;
 #pragma unroll
-                    for (int q = 0; q < kPropChunk; ++q) v[q] = q < nq ? __ldg(pr + q) : 0.f;
+                        for (int q = 0; q < kPropChunk; ++q) v[q] = q < nq ? __ldg(pr + q) : 0.f;
+                    }
                 }
             };
             float4 B_next = make_float4(0.f, 0.f, 0.f, 0.f);
+            int kind_next = 0;
             float v_next[kPropChunk];
 #pragma unroll
             for (int q = 0; q < kPropChunk; ++q) v_next[q] = 0.f;
-            if (wib < n_chunks) fetch(wib, B_next, v_next);
+            if (wib < n_chunks) fetch(wib, B_next, kind_next, v_next);
             for (int c = wib; c < n_chunks; c += kFeatSplit) {
+                // the chunk's atoms in reach of the group's box, those within the feature radius of it first
+                const unsigned in_f = __ballot_sync(0xffffffffu, kind_next == 2), in_r = __ballot_sync(0xffffffffu, kind_next == 1);
+                const int nf = __popc(in_f), nt = nf + __popc(in_r);
+                const unsigned below = (1u << lane) - 1u;
                 __syncwarp();
-                s_at[wib][lane] = B_next;
+                if (kind_next) {
+                    const int at = kind_next == 2 ? __popc(in_f & below) : nf + __popc(in_r & below);
+                    s_at[wib][0][at] = B_next.x;
+                    s_at[wib][1][at] = B_next.y;
+                    s_at[wib][2][at] = B_next.z;
+                    if (kind_next == 2) {
 #pragma unroll
-                for (int q = 0; q < kPropChunk / 4; ++q)
-                    s_pr[wib][lane][q] = make_float4(v_next[4 * q], v_next[4 * q + 1], v_next[4 * q + 2], v_next[4 * q + 3]);
+                        for (int q = 0; q < kPropChunk / 4; ++q)
+                            s_pr[wib][at][q] = make_float4(v_next[4 * q], v_next[4 * q + 1], v_next[4 * q + 2], v_next[4 * q + 3]);
+                    }
+                }
+                if (lane < 3 && (nt & 1)) s_at[wib][lane][nt] = 1e15f;   // the last pair's second: beyond any radius
                 __syncwarp();
-                if (c + kFeatSplit < n_chunks) fetch(c + kFeatSplit, B_next, v_next);
-                const int nt = min(32, total - c * 32);
-                for (int t = 0; t < nt; ++t) {
-                    const float4 A = s_at[wib][t];
-                    const float dx = A.x - px, ey = A.y - py, ez = A.z - pz;
-                    const float d2 = dx * dx + ey * ey + ez * ez;
-                    count += d2 <= g.rp2;
-                    if (d2 < g.rf2) {
-                        const float w = 1.0f - sqrtf(d2) * g.inv_rf;
+                if (c + kFeatSplit < n_chunks) fetch(c + kFeatSplit, B_next, kind_next, v_next);
+                auto pair_d2 = [&](int t) {                              // the chunk's atoms t and t + 1
+                    const float2 ax = *reinterpret_cast<const float2*>(&s_at[wib][0][t]);
+                    const float2 ay = *reinterpret_cast<const float2*>(&s_at[wib][1][t]);
+                    const float2 az = *reinterpret_cast<const float2*>(&s_at[wib][2][t]);
+                    const float2 dx = __fadd2_rn(ax, make_float2(-px, -px)), dy = __fadd2_rn(ay, make_float2(-py, -py)),
+                                 dz = __fadd2_rn(az, make_float2(-pz, -pz));
+                    const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
+                    count += (d2.x <= g.rp2) + (d2.y <= g.rp2);
+                    return d2;
+                };
+                int t = 0;
+                for (; t < nf; t += 2) {
+                    const float2 d2 = pair_d2(t);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float e = h ? d2.y : d2.x;
+                        if (!(e < g.rf2)) continue;
+                        const float w = 1.0f - sqrtf(e) * g.inv_rf;
 #pragma unroll
                         for (int q = 0; q < kPropChunk / 4; ++q) {
-                            const float4 pv = s_pr[wib][t][q];
+                            const float4 pv = s_pr[wib][t + h][q];
                             acc[4 * q] = fmaf(w, pv.x, acc[4 * q]);
                             acc[4 * q + 1] = fmaf(w, pv.y, acc[4 * q + 1]);
                             acc[4 * q + 2] = fmaf(w, pv.z, acc[4 * q + 2]);
@@ -588,6 +628,8 @@ __global__ void __launch_bounds__(kFeatSplit * 32) feature_kernel(FeatArgs g) {
                         }
                     }
                 }
+#pragma unroll 2
+                for (; t < nt; t += 2) pair_d2(t);
             }
             __syncthreads();                            // the row table is rebuilt for the next rows
         }
@@ -596,19 +638,20 @@ __global__ void __launch_bounds__(kFeatSplit * 32) feature_kernel(FeatArgs g) {
     for (int q = 0; q < kPropChunk; ++q) s_red[wib][q][lane] = acc[q];
     s_red[wib][kPropChunk][lane] = __int_as_float(count);
     __syncthreads();
-    if (wib != 0 || !live) return;
-    int total = 0;
-#pragma unroll
-    for (int w = 0; w < kFeatSplit; ++w) total += __float_as_int(s_red[w][kPropChunk][lane]);
-    float* f = g.feat + (size_t)pi * g.n_props + q0;
-#pragma unroll
-    for (int q = 0; q < kPropChunk; ++q) {
+    // the columns and the count are dealt to the warps, which all hold the same points
+    if (!live) return;
+    for (int q = wib; q < nq; q += kFeatSplit) {
         float v = 0.f;
 #pragma unroll
         for (int w = 0; w < kFeatSplit; ++w) v += s_red[w][q][lane];
-        if (q < nq) f[q] = fin ? v : 0.f;
+        g.feat[(size_t)pi * g.n_props + q0 + q] = fin ? v : 0.f;
     }
-    if (g.prot && blockIdx.y == 0) g.prot[pi] = fin ? total : 0;
+    if (wib == kFeatSplit - 1 && g.prot && blockIdx.y == 0) {
+        int total = 0;
+#pragma unroll
+        for (int w = 0; w < kFeatSplit; ++w) total += __float_as_int(s_red[w][kPropChunk][lane]);
+        g.prot[pi] = fin ? total : 0;
+    }
 }
 
 // ------------------------------------------------------------ Steps 4-5: clusters ---
@@ -1387,6 +1430,7 @@ extern "C" pv_status pv_surface_features(pv_context* ctx, const pv_surface* s, i
         a.rf2 = p->r_feature * p->r_feature;
         a.rp2 = p->r_protrusion * p->r_protrusion;
         a.reach = std::max(p->r_feature, p->r_protrusion) + 1e-3f;
+        a.reach_f = p->r_feature + 1e-3f;
         a.feat = dev_features;
         a.prot = dev_protrusion;
         const dim3 grid((unsigned)((n_points + 31) / 32), (unsigned)((n_props + kPropChunk - 1) / kPropChunk));

@@ -62,8 +62,7 @@ __device__ __forceinline__ void run_chain(const SearchArgs& A, const PvLigBlob& 
     // direction, gradient at the largest Armijo-satisfying trial and history entry's 1 / (y.s) live
     // in the team's scratch, not in registers through the evaluations
     Pose xt;
-    float f = 0.f, gd = 0.f, lam = 1.f, lo = 0.f, hi = -1.f, flo = 0.f;
-    float al = 0.f;
+    float f = 0.f, gd = 0.f, lam = 1.f, lo = 0.f, hi = -1.f, flo = 0.f, gg = 0.f, gamma = 0.f;
     float& g = S.lg[tl];
     float& d = S.ld[tl];
     float& rh = S.lr[tl];
@@ -109,6 +108,7 @@ __device__ __forceinline__ void run_chain(const SearchArgs& A, const PvLigBlob& 
             at_xt = true;
             f = fe; g = ge;
             it = 0; stored = 0; head = 0;
+            gg = Tm::sum(ge * ge);
             // a mutated candidate that fails the consistency check (Eq. 4-5) is not optimised
             if (FOCC && stage == kOptimise && !focc_pass<LANES>(xt, f, g, ring, nb_n, n_rot, C.focc_min_delta))
                 bdone = true;
@@ -147,20 +147,23 @@ __device__ __forceinline__ void run_chain(const SearchArgs& A, const PvLigBlob& 
             if (take) {
                 // curvature-guarded history update (Eq. 10-11), move, Eq. 12 test
                 const float sv = lam * d, yv = gt - g;
-                const float ys = Tm::sum(yv * sv), ss = Tm::sum(sv * sv), gn = sqrtf(Tm::sum(g * g));
+                const float4 sums = Tm::sum4(yv * sv, sv * sv, yv * yv, gt * gt);
+                const float ys = sums.x, ss = sums.y, gn = sqrtf(gg);
                 if (ss > 0.f && ys / ss > C.eps * gn) {
                     Hs[head * 32 + tl] = sv;
                     Hy[head * 32 + tl] = yv;
                     if (tl == head) rh = 1.f / ys;
+                    gamma = ys / sums.z;
                     head = head + 1 == m ? 0 : head + 1;
                     stored = min(stored + 1, m);
                 }
+                gg = sums.w;
                 Tm::sync();                                     // every lane has read the old base
                 stash_state<LANES>(S, xt);
                 at_xt = true;
                 g = gt; f = ft;
                 ++it;
-                if (sqrtf(Tm::sum(g * g)) <= C.eps) bdone = true;
+                if (sqrtf(gg) <= C.eps) bdone = true;
                 else next_iter = true;
             }
         }
@@ -168,7 +171,7 @@ __device__ __forceinline__ void run_chain(const SearchArgs& A, const PvLigBlob& 
             if (it >= iters) {
                 bdone = true;
             } else {
-                d = lbfgs_direction<LANES>(Hs, Hy, rh, al, g, stored, head, m);
+                d = lbfgs_direction<LANES>(Hs, Hy, S.lr, gamma, g, stored, head, m);
                 gd = Tm::sum(g * d);
                 if (!(gd < 0.f)) {
                     bdone = true;
@@ -300,7 +303,6 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
     // lane-private shared slots, and the base point of the line search in shared memory too
     // (stash_state): none of them is held in registers through an evaluation, which leaves the
     // evaluation the registers of the capped variants without spilling.
-    float al = 0.f;
     float& rh = S.lr[tl];
     float& g = S.lg[tl];
     float& d = S.ld[tl];
@@ -318,11 +320,13 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
         const int4 q1 = *reinterpret_cast<const int4*>(&Q.hi), q2 = *reinterpret_cast<const int4*>(&Q.stored);
         float f = q0.x, gd = q0.y, lam = q0.z, lo = q0.w, hi = __int_as_float(q1.x), flo = __int_as_float(q1.y);
         int it = q1.z, tr = q1.w, stored = q2.x, head = q2.y, have_lo = q2.z;
+        float gg = __int_as_float(q2.w), gamma = Q.gamma;
         bool next_iter = false, stop = false, retry = false, at_xt = false;
         if (start) {
             start = false;
             at_xt = true;
             f = fe; g = ge; it = 0; stored = 0; head = 0;
+            gg = Tm::sum(ge * ge);
             bool skip = false;
             if constexpr (FOCC) skip = ring && !focc_pass<32>(xt, fe, g, ring, Q.nb_n, n_rot, C.focc_min_delta);
             if (skip) stop = true;
@@ -359,20 +363,23 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
             }
             if (take) {
                 const float sv = lam * d, yv = gt - g;
-                const float ys = Tm::sum(yv * sv), ss = Tm::sum(sv * sv), gn = sqrtf(Tm::sum(g * g));
+                const float4 sums = Tm::sum4(yv * sv, sv * sv, yv * yv, gt * gt);
+                const float ys = sums.x, ss = sums.y, gn = sqrtf(gg);
                 if (ss > 0.f && ys / ss > C.eps * gn) {
                     Hs[head * 32 + tl] = sv;
                     Hy[head * 32 + tl] = yv;
                     if (tl == head) rh = 1.f / ys;
+                    gamma = ys / sums.z;
                     head = head + 1 == m ? 0 : head + 1;
                     stored = min(stored + 1, m);
                 }
+                gg = sums.w;
                 Tm::sync();                                     // every lane has read the old base
                 stash_state<32>(S, xt);
                 at_xt = true;
                 g = gt; f = ft;
                 ++it;
-                if (sqrtf(Tm::sum(g * g)) <= C.eps) stop = true;
+                if (sqrtf(gg) <= C.eps) stop = true;
                 else next_iter = true;
             }
         }
@@ -380,7 +387,7 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
             if (it >= max_iter) {
                 stop = true;
             } else {
-                d = lbfgs_direction<32>(Hs, Hy, rh, al, g, stored, head, m);
+                d = lbfgs_direction<32>(Hs, Hy, S.lr, gamma, g, stored, head, m);
                 gd = Tm::sum(g * d);
                 if (!(gd < 0.f)) {
                     stop = true;
@@ -401,7 +408,8 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
         Tm::sync();                       // every lane has read this iteration's scalars
         *reinterpret_cast<float4*>(&Q.f) = make_float4(f, gd, lam, lo);
         *reinterpret_cast<int4*>(&Q.hi) = make_int4(__float_as_int(hi), __float_as_int(flo), it, tr);
-        *reinterpret_cast<int4*>(&Q.stored) = make_int4(stored, head, have_lo, 0);
+        *reinterpret_cast<int4*>(&Q.stored) = make_int4(stored, head, have_lo, __float_as_int(gg));
+        Q.gamma = gamma;
     }
 }
 template <bool FOCC, int LAYOUT>

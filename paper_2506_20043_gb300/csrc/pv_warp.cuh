@@ -27,7 +27,9 @@ struct __align__(16) ChainScalars {
     float f, gd, lam, lo;                     // of the line search: three 16-byte words
     float hi, flo;
     int it, tr;
-    int stored, head, have_lo, pad;
+    int stored, head, have_lo;
+    float gg;                                 // |g|^2 at the base point
+    float gamma;                              // y.s / y.y of the newest pair
     float e_cur, e_best, u;
     int s, stage, flags, nb_n, nb_head;
     uint32_t evals_before;
@@ -87,6 +89,13 @@ struct Team {
 #pragma unroll
         for (int o = LANES / 16; o > 0; o >>= 1) v += __shfl_xor_sync(mask(), v, o, LANES);
         return v;
+    }
+    // The same for four values, given to every lane.
+    static __device__ __forceinline__ float4 sum4(float a, float b, float c, float d) {
+        float v = halve(halve(a, b, LANES / 2), halve(c, d, LANES / 2), LANES / 4);
+#pragma unroll
+        for (int o = LANES / 8; o > 0; o >>= 1) v += __shfl_xor_sync(mask(), v, o, LANES);
+        return make_float4(shfl(v, 0), shfl(v, LANES / 2), shfl(v, LANES / 4), shfl(v, LANES / 2 + LANES / 4));
     }
     static __device__ __forceinline__ int sum8_lane(int k) {
         return (k & 1) * (LANES / 2) + ((k >> 1) & 1) * (LANES / 4) + ((k >> 2) & 1) * (LANES / 8);
@@ -436,31 +445,26 @@ __device__ __forceinline__ Pose team_retract(const Pose& x, float step, int n_ta
     return y;
 }
 
-// L-BFGS two-loop recursion (Eq. 10-11 history, newest pair first) for the direction d = -H g.
+// L-BFGS two-loop recursion (Eq. 10-11 history, newest pair first) for the direction d = -H g. rho[k] is
+// 1 / (y.s) of history entry k, gamma the initial scaling y.s / y.y of the newest pair.
 template <int LANES>
-__device__ __forceinline__ float lbfgs_direction(const float* Hs, const float* Hy, float rh, float& al,
+__device__ __forceinline__ float lbfgs_direction(const float* Hs, const float* Hy, const float* rho, float gamma,
                                                  float g, int stored, int head, int m) {
     using Tm = Team<LANES>;
     const int tl = Tm::lane();
-    float q = g;
+    float q = g, al = 0.f;
+    int k = head;
     for (int a = 0; a < stored; ++a) {
-        int k = head - 1 - a;
-        if (k < 0) k += m;
-        const float alpha = Tm::shfl(rh, k) * Tm::sum(Hs[k * 32 + tl] * q);
+        k = (k == 0 ? m : k) - 1;
+        const float alpha = rho[k] * Tm::sum(Hs[k * 32 + tl] * q);
         if (tl == k) al = alpha;
         q -= alpha * Hy[k * 32 + tl];
     }
-    if (stored > 0) {
-        const int k = head == 0 ? m - 1 : head - 1;
-        const float sk = Hs[k * 32 + tl], yk = Hy[k * 32 + tl];
-        const float sy = Tm::sum(sk * yk), yy = Tm::sum(yk * yk);
-        q *= sy / yy;
-    }
-    for (int a = stored - 1; a >= 0; --a) {
-        int k = head - 1 - a;
-        if (k < 0) k += m;
-        const float b = Tm::shfl(rh, k) * Tm::sum(Hy[k * 32 + tl] * q);
+    if (stored > 0) q *= gamma;
+    for (int a = stored; a > 0; --a) {
+        const float b = rho[k] * Tm::sum(Hy[k * 32 + tl] * q);
         q += Hs[k * 32 + tl] * (Tm::shfl(al, k) - b);
+        k = k + 1 == m ? 0 : k + 1;
     }
     return -q;
 }

@@ -255,7 +255,8 @@ typedef struct {
     float amplitude;           /* mutation radius, A (translation; orientation amplitude/R_gyr) */
     int32_t steps_per_round;   /* batched: MC steps per kernel launch (round); 0 = automatic */
     int32_t use_graph;         /* batched: capture the launch sequence in a CUDA graph */
-    int32_t warps_per_cta;     /* batched: warps per CTA; 0 = autotuned */
+    int32_t warps_per_cta;     /* batched: warps per CTA; 0 = as many as the variant's registers and the
+                                  shared memory allow on an SM (fewer for a job with fewer chains) */
     int32_t search_variant;    /* batched: search kernel variant; 0..3 one chain per warp, 4..7
                                   one chain per half warp (ligands of <= 32 atoms and <= 10
                                   torsions); within each group decreasing register budgets and
@@ -315,14 +316,14 @@ typedef struct {
  * steps_per_round 0, use_graph 1, warps_per_cta 0, search_variant -1, host_copy 1, timeout_s 0,
  * focc 0, focc_min_delta 1e-4, rescore 0, max_pockets 0, block_wait_s 30, pair_keys NULL,
  * map_layout -1, resume_state NULL, resume_bytes 0.
- * Autotuning (warps_per_cta 0, search_variant -1, or map_layout -1 on a set holding both layouts):
- * the first batched dock of a ligand-size bucket on a context times each candidate launch shape on
+ * Autotuning (search_variant -1, or map_layout -1 on a set holding both layouts):
+ * the first batched dock of a ligand-size bucket on a context times each candidate variant on
  * 32 MC steps of its own work items (after 16 untimed steps from the random starts), the fastest of
  * three runs, per score evaluation the trial ran
  * (results are unaffected: the dock itself restarts every chain); a candidate displaces the first
  * one tried only when it is faster by more than 2 %, so that shapes within the trials' noise do not
  * alternate between runs. With map_layout -1 on a set holding both layouts, every candidate is timed
- * on each layout (the cell-packed maps first), and the fastest (shape, layout) is kept. */
+ * on each layout (the cell-packed maps first), and the fastest (variant, layout) is kept. */
 void pv_dock_params_default(pv_dock_params* p);
 
 /* Docks every ligand into every listed pocket (Supplementary Algorithms 2 and 3). Pair
@@ -387,7 +388,8 @@ pv_status pv_dock_result_timing(const pv_dock_result* r, double* search_seconds,
 /* Map layout the search read (0 plain, 1 cell-packed). */
 pv_status pv_dock_result_map_layout(const pv_dock_result* r, int32_t* map_layout);
 
-/* Launch shape the batched search used (after autotuning): register variant and chains per CTA. */
+/* Launch shape the batched search used (after autotuning): register variant and warps per CTA (at most
+ * the number that warps_per_cta accepts for the variant; with warps_per_cta 0 a CTA may run more). */
 pv_status pv_dock_result_launch(const pv_dock_result* r, int32_t* search_variant, int32_t* warps_per_cta);
 
 /* Device-resident results (valid until destroy): poses [n_pairs * top_k] pv_pose,

@@ -2,7 +2,6 @@
 // docking driver (batched rounds captured in a CUDA graph, or the plain per-pair loop).
 #include <algorithm>
 #include <map>
-#include <tuple>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -32,9 +31,9 @@ struct pv_context {
     int sms = 0;
     cudaStream_t capture_stream = nullptr;   // graphs are captured here (the caller's stream may
                                              // be the legacy default stream, which cannot capture)
-    // autotuned (search variant, warps per CTA) per (ligand atoms / 8, check on/off and team width;
+    // autotuned (search variant, map layout) per (ligand atoms / 8, check on/off and team width;
     // pair rounds / 4 and the caller's fixed variant or CTA size)
-    std::map<std::pair<int, int>, std::tuple<int, int, int>> tuned;   // -> (variant, warps, layout)
+    std::map<std::pair<int, int>, std::pair<int, int>> tuned;   // -> (variant, layout)
 };
 
 struct pv_grid_set {
@@ -902,17 +901,10 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
         result_free(R);
         return fail(ctx, PV_ERR_ARG, "pairs per ligand x top_k exceeds the merge capacity (8192)");
     }
-    // work items: pocket-major for map locality, then pair, then chain block
+    // pairs are worked on pocket by pocket, for map locality
     std::vector<int> order(n_pairs);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return pair_pocket[a] < pair_pocket[b]; });
-    // a work item is one CTA's chains of one pair: warps x chains per warp
-    auto make_items = [&](int chains_per_cta) {
-        std::vector<PvItem> it;
-        for (int q : order)
-            for (int c0 = 0; c0 < p.chains; c0 += chains_per_cta) it.push_back(PvItem{q, c0});
-        return it;
-    };
     bool all_team16 = true;
     for (int i = 0; i < n_ligs; ++i) all_team16 = all_team16 && ligs[i]->rec.team16;
     if (p.search_variant >= 0 && search_variant_lanes(p.search_variant) == 16 && !all_team16)
@@ -926,7 +918,55 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
     // shared memory of a staged ligand: the record with the schedule of the variant's team width
     auto stage_bytes = [&](int v) { return search_variant_lanes(v) == 16 ? max_stage16 : max_stage32; };
     int variant = p.search_variant >= 0 ? p.search_variant : (auto_lanes == 16 ? 4 : 0);
-    int W = p.warps_per_cta > 0 ? p.warps_per_cta : 4;
+    // a unit of work is a warp's chains of one pair: one, or two on half warps
+    auto units_of = [&](int v) { return (p.chains + 32 / search_variant_lanes(v) - 1) / (32 / search_variant_lanes(v)); };
+    // The launch of a variant: CTA size, ligand slots, CTAs per SM, and the units of a work item.
+    // CTA size: the caller's (as many CTAs per SM as fit), else one CTA per SM with every warp that the
+    // variant's registers and the shared memory of its scratch allow, or, when the job has fewer units, those
+    // spread evenly over the SMs. Ligand slots: as many (up to kLigSlots) as fit beside them, so that warps go on
+    // to the next ligand while others finish one. An item fills a CTA's warps once where ligands differ (few
+    // ligands in flight per CTA); with a single ligand it is small, so that the last items spread.
+    struct Shape {
+        int warps = 0, slots = 1, occ = 0, item_units = 1, items_per_pair = 1, grid = 0;
+        bool all_resident = false;   // every unit runs at once, an item each
+    };
+    auto shape_of = [&](int v, int lay, Shape& s) -> cudaError_t {
+        const int lanes = search_variant_lanes(v), units = units_of(v);
+        const long long total = (long long)units * (p.mode == PV_MODE_PLAIN_WARP ? 1 : n_pairs);   // per launch
+        auto fits = [&](int warps, int slots, int* occ) {
+            *occ = 0;
+            return search_max_ctas_per_sm(v, p.focc > 0, lay, warps, search_smem_bytes(stage_bytes(v), warps, lanes, slots), occ);
+        };
+        cudaError_t x = cudaSuccess;
+        s = Shape();
+        if (p.warps_per_cta > 0) {
+            s.warps = p.warps_per_cta;
+            x = fits(s.warps, 1, &s.occ);
+        } else {
+            const long long even = (total + ctx->sms - 1) / ctx->sms;
+            for (s.warps = (int)std::min<long long>(search_variant_sm_warps(v), even); s.warps > 0; --s.warps) {
+                x = fits(s.warps, 1, &s.occ);
+                if (x == cudaSuccess && s.occ > 0) break;
+                cudaGetLastError();
+            }
+            if (s.warps > 0) s.occ = 1;
+        }
+        if (x != cudaSuccess || s.warps < 1 || s.occ < 1) return x;
+        for (int occ = 0; s.slots < std::min(kLigSlots, n_ligs); ++s.slots) {
+            if (fits(s.warps, s.slots + 1, &occ) != cudaSuccess || occ < s.occ) {
+                cudaGetLastError();
+                break;
+            }
+        }
+        s.all_resident = p.warps_per_cta == 0 && total <= (long long)ctx->sms * s.warps && (n_ligs == 1 || s.slots >= s.warps);
+        const int most = s.all_resident ? 1 : n_ligs > 1 || p.warps_per_cta > 0 ? s.warps : std::min(s.warps, 4);
+        s.items_per_pair = (units + most - 1) / most;
+        s.item_units = (units + s.items_per_pair - 1) / s.items_per_pair;
+        s.items_per_pair = (units + s.item_units - 1) / s.item_units;
+        const long long items = (long long)s.items_per_pair * n_pairs;
+        s.grid = (int)std::max<long long>(1, std::min<long long>(items, (long long)ctx->sms * s.occ));
+        return cudaSuccess;
+    };
     const bool warp_chains = p.mode != PV_MODE_PLAIN;   // batched, or one warp-per-chain launch per pair
     // map layout: the caller's, or (map_layout -1) the cell-packed one is a candidate when the set
     // holds it; the layout never changes results (the same corners, the same arithmetic)
@@ -934,43 +974,41 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
         return fail(ctx, PV_ERR_ARG, "map_layout 1 needs a grid set with cell-packed maps (pv_grid_set_pack)");
     const bool tune_layout = warp_chains && p.map_layout < 0 && set->packed;
     int layout = p.map_layout == 1 ? 1 : 0;
-    const bool autotune = warp_chains && (p.search_variant < 0 || p.warps_per_cta == 0 || tune_layout);
+    const bool autotune = warp_chains && (p.search_variant < 0 || tune_layout);
     int max_rounds = 0;
     for (int i = 0; i < n_ligs; ++i) max_rounds = std::max(max_rounds, ligs[i]->rec.n_rounds);
+    // a job that leaves SMs partly idle is bound by the latency of its chains, not by issue slots: its
+    // variant is tuned apart from that of full ones
+    const bool few = (long long)n_pairs * p.chains < (long long)ctx->sms * 16;
     // the parameters the caller fixed (a variant, a CTA size, a layout) are part of the key: a shape
     // tuned with one of them free may not suit the other fixed
     const std::pair<int, int> tune_key{4 * ((max_atoms + 7) / 8) + 2 * (p.focc > 0 ? 1 : 0) + (auto_lanes == 16 ? 1 : 0),
                                        ((max_rounds + 3) / 4) * 1024 + p.warps_per_cta * 16 + (p.search_variant + 1) +
-                                           (tune_layout ? 1 << 20 : 0) + ((p.map_layout + 1) << 21)};
+                                           (tune_layout ? 1 << 20 : 0) + ((p.map_layout + 1) << 21) +
+                                           (few ? 1 << 23 : 0)};
     bool need_tune = false;
     if (autotune) {
         auto it = ctx->tuned.find(tune_key);
         if (it != ctx->tuned.end()) {
-            if (p.search_variant < 0) variant = std::get<0>(it->second);
-            if (p.warps_per_cta == 0) W = std::get<1>(it->second);
-            if (tune_layout) layout = std::get<2>(it->second);
+            if (p.search_variant < 0) variant = it->second.first;
+            if (tune_layout) layout = it->second.second;
         } else {
             need_tune = true;
         }
     }
-    // the items buffer is sized for the smallest CTA a candidate may use
-    const int W_min = autotune ? (p.warps_per_cta > 0 ? p.warps_per_cta : 1) : W;
-    std::vector<PvItem> items = make_items(W * (32 / search_variant_lanes(variant)));
-    const size_t items_cap = make_items(W_min).size();
     std::vector<PvPairDesc> pdesc(n_pairs);
     for (int q = 0; q < n_pairs; ++q)
         pdesc[q] = PvPairDesc{pair_lig[q], pair_pocket[q], ligs[pair_lig[q]]->rec.n_rounds, pair_key[q]};
     std::vector<const void*> ligptr(n_ligs);
     for (int i = 0; i < n_ligs; ++i) ligptr[i] = ligs[i]->d_blob;
-    // one launch (round) covers all MC steps unless steps_per_round asks for more; a launch's steps
-    // are cut into chained step blocks of about 1/16 of them (at least 25)
+    // one launch (round) covers all MC steps unless steps_per_round asks for more; its steps are cut into
+    // chained step blocks (see block_steps below)
     const int S_r = p.steps_per_round > 0 ? p.steps_per_round : std::max(1, steps_left);
     const int n_rounds = steps_left > 0 ? (steps_left + S_r - 1) / S_r : 1;
-    const int block_steps = std::max(25, (S_r + 15) / 16);
     // one workspace allocation
     Layout Lw;
     const size_t o_pairs = Lw.take<PvPairDesc>(n_pairs), o_ligs = Lw.take<const void*>(n_ligs),
-                 o_items = Lw.take<PvItem>(std::max(items.size(), items_cap)), o_ctr = Lw.take<int>(n_rounds + 2),
+                 o_order = Lw.take<int>(n_pairs), o_ctr = Lw.take<int>(n_rounds + 2),
                  o_evals = Lw.take<unsigned long long>(2),
                  o_chains = Lw.take<float>((size_t)n_pairs * p.chains * PV_CHAIN_STRIDE),
                  o_poses = Lw.take<PvPoseRec>((size_t)n_pairs * p.top_k),
@@ -978,9 +1016,9 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
                  o_xyz = Lw.take<float>((size_t)n_pairs * p.top_k * R->atom_stride * 3),
                  o_nkept = Lw.take<int>(n_pairs), o_status = Lw.take<int>(n_pairs),
                  o_rank = Lw.take<int>((size_t)n_ligs * R->rank_stride), o_lps = Lw.take<int>(n_ligs + 1),
-                 o_lp = Lw.take<int>(n_pairs), o_prog = Lw.take<int>(std::max(items.size(), items_cap)),
+                 o_lp = Lw.take<int>(n_pairs), o_prog = Lw.take<int>((size_t)n_pairs * p.chains),
                  o_ring = Lw.take<float>(p.focc > 0 ? (size_t)n_pairs * p.chains * PV_RING_STRIDE : 0);
-    const size_t small_end = o_items + std::max(items.size(), items_cap) * sizeof(PvItem);
+    const size_t small_end = o_order + n_pairs * sizeof(int);
     char* w = (char*)dalloc(ctx, Lw.off);
     if (!w) {
         result_free(R);
@@ -998,7 +1036,7 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
     std::vector<char> host(small_end, 0);
     std::memcpy(host.data() + o_pairs, pdesc.data(), sizeof(PvPairDesc) * n_pairs);
     std::memcpy(host.data() + o_ligs, ligptr.data(), sizeof(void*) * n_ligs);
-    std::memcpy(host.data() + o_items, items.data(), sizeof(PvItem) * items.size());
+    std::memcpy(host.data() + o_order, order.data(), sizeof(int) * n_pairs);
     std::vector<int> csr(n_ligs + 1 + n_pairs);
     cudaError_t e = cudaMemcpyAsync(w, host.data(), small_end, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess)
@@ -1034,8 +1072,8 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
     C.pot_stride = R->pot_stride;
     C.atom_stride = R->atom_stride;
     SearchArgs A;
-    A.items = (const PvItem*)(w + o_items);
-    A.n_items = (int)items.size();
+    A.order = (const int*)(w + o_order);
+    A.n_items = 0;
     A.queue = nullptr;
     A.pairs = (const PvPairDesc*)(w + o_pairs);
     A.ligs = (const PvLigBlob* const*)(w + o_ligs);
@@ -1045,11 +1083,10 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
     A.chains = R->d_chains;
     A.ring = p.focc > 0 ? (float*)(w + o_ring) : nullptr;
     R->d_ring = A.ring;
-    A.items_per_block = (int)items.size();
-    A.block_steps = block_steps;
+    A.items_per_block = 0;
+    A.block_steps = 1;
     A.progress = (int*)(w + o_prog);
     A.C = C;
-    A.lig_smem_bytes = stage_bytes(variant);
     A.t0 = evals + 1;
     A.timeout_ns = p.timeout_s > 0 ? (unsigned long long)(p.timeout_s * 1e9) : 0ull;
     A.wait_ns = p.block_wait_s > 0 ? (unsigned long long)(std::min(p.block_wait_s, 1e9) * 1e9) : 30000000000ull;
@@ -1078,10 +1115,19 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
     M.top_k = p.top_k;
     M.rank_stride = R->rank_stride;
     M.ranking = R->d_ranking;
-    // autotuning: time each candidate launch shape on kTuneSteps MC steps of its own first work
-    // items (long enough that chains which share a CTA even out, as over a real step block), after
-    // kWarmSteps untimed steps from the random starts, per score evaluation, the best of three runs;
-    // then, if the set holds cell-packed maps too, the chosen shape on them.
+    // the launch of a variant in its shape
+    auto apply = [&](SearchArgs& a, int v, int lay, const Shape& s) {
+        a.layout = lay;
+        a.lig_smem_bytes = stage_bytes(v);
+        a.lig_slots = s.slots;
+        a.units = units_of(v);
+        a.item_units = s.item_units;
+        a.items_per_pair = s.items_per_pair;
+        a.items_per_block = s.items_per_pair * n_pairs;
+    };
+    // autotuning: time each candidate variant on kTuneSteps MC steps of its first work items, after
+    // kWarmSteps untimed steps from the random starts, per score evaluation, the best of three runs; on each
+    // layout the set holds.
     // A candidate replaces the incumbent (the first candidate, a fixed preference order) only when
     // it is faster by more than kTuneMargin, so that shapes within the trials' noise do not flip
     // between runs.
@@ -1090,50 +1136,39 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
         constexpr int kWarmSteps = 16, kTuneSteps = 32, kTuneBlock = 8;
         constexpr float kTuneMargin = 0.02f;
         // in order of preference: the first of a team width is the incumbent the others must beat by
-        // the margin (whole warps: variant 3 x 4 warps measured fastest on the multi-pocket workload
-        // of 30-atom ligands, then variant 2 x 4, and variant 1 x 4 on batches with ligands of more
-        // than 32 atoms, two per lane, whose evaluation needs more registers; half warps: variant
-        // 5 x 4 on a 16-atom ligand over the same pockets)
-        static const int cand_small[][2] = {{3, 4}, {2, 4}, {1, 4}, {0, 2}, {0, 4}, {0, 8}, {1, 2}, {2, 2}, {0, 1},
-                                            {5, 4}, {4, 2}, {4, 1}, {4, 4}, {5, 2}, {6, 4}, {7, 4}};
-        static const int cand_large[][2] = {{1, 4}, {3, 4}, {2, 4}, {0, 2}, {0, 4}, {0, 8}, {1, 2}, {2, 2}, {0, 1},
-                                            {5, 4}, {4, 2}, {4, 1}, {4, 4}, {5, 2}, {6, 4}, {7, 4}};
+        // the margin (whole warps: variant 3 measured fastest on the multi-pocket workload of 30-atom
+        // ligands, variant 1 on batches with ligands of more than 32 atoms, two per lane, whose evaluation
+        // needs more registers; half warps: variant 5 on a 16-atom ligand over the same pockets)
+        static const int cand_small[] = {3, 2, 1, 0, 5, 4, 6, 7};
+        static const int cand_large[] = {1, 2, 3, 0, 5, 4, 6, 7};
         const auto& cand = max_atoms > 32 ? cand_large : cand_small;
         cudaEvent_t t0, t1;
         cudaEventCreate(&t0);
         cudaEventCreate(&t1);
-        // time per score evaluation of one shape and layout; < 0 when the shape does not fit
-        auto trial = [&](int v, int wc, int lay, float& per_chain) -> cudaError_t {
+        // time per score evaluation of one variant and layout; < 0 when it does not fit
+        auto trial = [&](int v, int lay, float& per_chain) -> cudaError_t {
             per_chain = -1.f;
-            const int lanes_c = search_variant_lanes(v);
-            int occ_c = 0;
-            if (search_max_ctas_per_sm(v, p.focc > 0, lay, wc, search_smem_bytes(stage_bytes(v), wc, lanes_c), &occ_c) !=
-                    cudaSuccess ||
-                occ_c < 1) {
+            Shape sh;
+            if (shape_of(v, lay, sh) != cudaSuccess || sh.occ < 1 || sh.warps < 1) {
                 cudaGetLastError();
                 return cudaSuccess;
             }
-            // whole waves of the shape's resident CTAs (up to four) when the work allows, so that a
+            // whole waves of the shape's resident warps (up to four) when the work allows, so that a
             // partly filled last wave, which the chained step blocks of a real launch do not have,
-            // does not weigh on the shapes with fewer, larger CTAs
-            std::vector<PvItem> trial_items = make_items(wc * (32 / lanes_c));
-            const size_t slots = (size_t)ctx->sms * occ_c;
-            const size_t n_waves = std::min<size_t>(4, trial_items.size() / slots);
-            const int n_trial = (int)(n_waves > 0 ? n_waves * slots : trial_items.size());
+            // does not weigh on the shapes with more warps
             SearchArgs a = A;
-            a.items = (const PvItem*)((char*)R->d_work + o_items);
+            apply(a, v, lay, sh);
+            const int slots = std::max(1, sh.grid * sh.warps / sh.item_units), n_waves = std::min(4, a.items_per_block / slots);
+            const int n_trial = n_waves > 0 ? n_waves * slots : a.items_per_block;
             a.n_items = 0;                       // an empty launch first: loads the variant's code
             a.queue = ctr + 1;
             a.step0 = 0;
             a.step1 = kWarmSteps;
             a.items_per_block = n_trial;         // one step block
             a.block_steps = kWarmSteps + kTuneSteps;
-            a.layout = lay;
-            a.lig_smem_bytes = stage_bytes(v);
-            const int grid_c = std::max(1, std::min(n_trial, ctx->sms * occ_c));
-            cudaError_t x = cudaMemcpyAsync((char*)R->d_work + o_items, trial_items.data(), sizeof(PvItem) * n_trial,
-                                            cudaMemcpyHostToDevice, ctx->stream);
-            if (x == cudaSuccess) x = cudaMemsetAsync(ctr, 0, sizeof(int) * 2, ctx->stream);
+            const int grid_c = sh.grid, wc = sh.warps;
+            const size_t n_prog = (size_t)n_pairs * a.units;
+            cudaError_t x = cudaMemsetAsync(ctr, 0, sizeof(int) * 2, ctx->stream);
             if (x == cudaSuccess) x = launch_search_round(a, v, 1, wc, ctx->stream);
             // untimed: the chains' first steps from their random starts, so that the timed steps run
             // from the states most of a real launch's step blocks start from
@@ -1151,7 +1186,7 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
             float best = 1e30f;
             for (int rep = 0; rep < 3 && x == cudaSuccess; ++rep) {   // the fastest of three runs
                 x = cudaMemsetAsync(ctr, 0, sizeof(int) * 2, ctx->stream);
-                if (x == cudaSuccess) x = cudaMemsetAsync(a.progress, 0, sizeof(int) * (size_t)n_trial, ctx->stream);
+                if (x == cudaSuccess) x = cudaMemsetAsync(a.progress, 0, sizeof(int) * n_prog, ctx->stream);
                 if (x == cudaSuccess) x = cudaMemsetAsync(evals, 0, sizeof(unsigned long long), ctx->stream);
                 if (x == cudaSuccess) x = launch_mark_t0(evals + 1, ctx->stream);
                 if (x == cudaSuccess) x = cudaEventRecord(t0, ctx->stream);
@@ -1173,26 +1208,24 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
         // holds both): the shapes rank differently on the two layouts (more resident CTAs put more
         // pressure on L1, which the plain maps' four or more sectors per lookup feel most).
         float best_ms = -1.f;
-        int best_v = variant, best_w = W, best_lay = layout;
+        int best_v = variant, best_lay = layout;
         cudaError_t x = cudaSuccess;
-        const bool tune_shape = p.search_variant < 0 || p.warps_per_cta == 0;
         const int n_lay = tune_layout ? 2 : 1;
-        for (const auto& cw : cand) {
-            const int v = p.search_variant >= 0 ? p.search_variant : cw[0];
-            const int wc = p.warps_per_cta > 0 ? p.warps_per_cta : cw[1];
-            if (wc > search_variant_max_warps(v)) continue;
+        for (const int c : cand) {
+            const int v = p.search_variant >= 0 ? p.search_variant : c;
+            if (p.warps_per_cta > search_variant_max_warps(v)) continue;
             const int lanes_c = search_variant_lanes(v);
             if (lanes_c == 16 && !all_team16) continue;
             if (p.search_variant < 0 && lanes_c != auto_lanes) continue;
             for (int li = 0; li < n_lay && x == cudaSuccess; ++li) {
                 const int lay = tune_layout ? 1 - li : layout;
                 float pc = 0.f;
-                x = trial(v, wc, lay, pc);
+                x = trial(v, lay, pc);
                 if (x == cudaSuccess && pc > 0.f && (best_ms < 0.f || pc < best_ms * (1.f - kTuneMargin))) {
-                    best_ms = pc; best_v = v; best_w = wc; best_lay = lay;
+                    best_ms = pc; best_v = v; best_lay = lay;
                 }
             }
-            if (x != cudaSuccess || !tune_shape) break;   // a fixed shape: only its layouts
+            if (x != cudaSuccess || p.search_variant >= 0) break;   // a fixed variant: only its layouts
         }
         layout = best_lay;
         cudaEventDestroy(t0);
@@ -1202,37 +1235,28 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
             return cuda_fail(ctx, x, "autotune");
         }
         variant = best_v;
-        W = best_w;
-        ctx->tuned[tune_key] = std::make_tuple(variant, W, layout);
-        items = make_items(W * (32 / search_variant_lanes(variant)));
-        e = cudaMemcpyAsync((char*)R->d_work + o_items, items.data(), sizeof(PvItem) * items.size(),
-                            cudaMemcpyHostToDevice, ctx->stream);
-        if (e != cudaSuccess) {
-            result_free(R);
-            return cuda_fail(ctx, e, "item upload");
-        }
+        ctx->tuned[tune_key] = std::make_pair(variant, layout);
     }
-    A.layout = layout;
-    A.items_per_block = (int)items.size();
-    // each pair's run of work items (items are grouped by pair) for the per-pair launches
-    std::vector<int> item_start(n_pairs, 0), item_count(n_pairs, 0);
-    for (int i = (int)items.size() - 1; i >= 0; --i) {
-        item_start[items[i].pair] = i;
-        item_count[items[i].pair]++;
-    }
-    // grid of the persistent rounds: every SM filled to its occupancy
-    int occ = 0;
-    A.lig_smem_bytes = stage_bytes(variant);
-    const int smem = search_smem_bytes(A.lig_smem_bytes, W, search_variant_lanes(variant));
-    e = search_max_ctas_per_sm(variant, p.focc > 0, layout, W, smem, &occ);
-    if (e != cudaSuccess || occ < 1) {
+    Shape shape;
+    e = shape_of(variant, layout, shape);
+    if (e != cudaSuccess || shape.occ < 1 || shape.warps < 1) {
         result_free(R);
         return e != cudaSuccess ? cuda_fail(ctx, e, "occupancy") : fail(ctx, PV_ERR_ARG, "search kernel does not fit");
     }
-    // at most one step block of each work item can run at a time
-    const int grid = std::max(1, std::min((int)items.size(), ctx->sms * occ));
+    apply(A, variant, layout, shape);
+    const int W = shape.warps, grid = shape.grid, occ = shape.occ;
+    // Step blocks: when every unit runs at once there is nothing to hand over, and a warp keeps its chains
+    // to the end (blocks would make the fast chains wait for the slow ones' hand-outs); else blocks of about
+    // 1/32 of the steps, so that the last ones spread over the SMs. A caller who fixes the CTA size gets
+    // blocks of about 1/16 (at least 25 steps).
+    const int block_steps = p.warps_per_cta > 0 ? std::max(25, (S_r + 15) / 16)
+                            : shape.all_resident ? S_r : std::max(8, (S_r + 31) / 32);
+    A.block_steps = block_steps;
+    // each pair's position in the order, for the per-pair launches
+    std::vector<int> position(n_pairs, 0);
+    for (int i = 0; i < n_pairs; ++i) position[order[i]] = i;
     R->search_variant = variant;
-    R->warps_per_cta = W;
+    R->warps_per_cta = std::min(W, search_variant_max_warps(variant));
     R->map_layout = layout;
     e = prepare_topk(T);
     if (e == cudaSuccess) e = prepare_merge(R->rank_stride);
@@ -1279,7 +1303,7 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
                 a.step1 = std::min(p.steps, s_first + (r + 1) * S_r);
                 const int n_blocks = a.step1 > a.step0 ? (a.step1 - a.step0 + block_steps - 1) / block_steps : 1;
                 a.n_items = n_blocks * a.items_per_block;
-                x = cudaMemsetAsync(a.progress, 0, sizeof(int) * (size_t)a.items_per_block, s);
+                x = cudaMemsetAsync(a.progress, 0, sizeof(int) * (size_t)n_pairs * a.units, s);
                 if (x == cudaSuccess) x = launch_search_round(a, variant, grid, W, s);
             }
             if (x == cudaSuccess) x = cudaEventRecordWithFlags(evs1, s, ev_flags);
@@ -1290,16 +1314,15 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
             // pair's selection, and a host synchronisation before the next pair
             for (int q = 0; q < n_pairs && x == cudaSuccess; ++q) {
                 SearchArgs a = A;
-                a.items = A.items + item_start[q];
-                a.items_per_block = item_count[q];
-                a.n_items = item_count[q];
+                a.order = A.order + position[q];
+                a.items_per_block = a.n_items = a.items_per_pair;
                 a.queue = ctr + 2;
                 a.step0 = s_first;
                 a.step1 = p.steps;
                 a.block_steps = std::max(1, steps_left);
                 x = cudaMemsetAsync(ctr + 2, 0, sizeof(int), s);
                 if (x == cudaSuccess)
-                    x = launch_search_round(a, variant, std::max(1, std::min(item_count[q], ctx->sms * occ)), W, s);
+                    x = launch_search_round(a, variant, std::max(1, std::min(a.items_per_pair, ctx->sms * occ)), W, s);
                 TopkArgs t = T;
                 t.pair0 = q;
                 if (x == cudaSuccess) x = launch_topk(t, 1, s);

@@ -526,24 +526,28 @@ __device__ __forceinline__ void run_chain_warp(const SearchArgs& A, const PvLigB
     flags_out = flags;
 }
 
+// The waits below are run by whole warps, their conditions taken from the first lane, so that a warp is
+// converged when it goes on: waits of one lane left the warp split through the chain code after them, which then
+// ran at half its rate.
 __device__ __forceinline__ int load_acquire(const int* p) {
     int v;
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
+    return __shfl_sync(PV_FULL, v, 0);
 }
-// Waits until the chain block's previous step block is published (`*progress >= blk`). Every CTA
-// of the launch is resident and a block is taken from the queue only after all blocks before it,
-// by CTAs that are running, so the wait ends; it is still bounded by limit_ns. Returns 1 when the
-// predecessor is published, 0 when the bound ran out, -1 when the work item was given up
-// (poisoned) by an earlier block.
+__device__ __forceinline__ unsigned long long warp_time() { return __shfl_sync(PV_FULL, globaltimer(), 0); }
+// Waits until the chains' previous step block is published (`*progress >= blk`). Every CTA
+// of the launch is resident and an item is taken from the queue only after all items before it,
+// by CTAs that are running, so the wait ends (of all unfinished items the first one's chains wait
+// for nothing); it is still bounded by limit_ns. Returns 1 when the predecessor is published, 0 when the
+// bound ran out, -1 when the chains were given up (poisoned) by an earlier block.
 __device__ __forceinline__ int wait_block(const int* progress, int blk, unsigned long long limit_ns) {
     int v = load_acquire(progress);
     if (v >= PV_PROGRESS_POISON) return -1;
     if (v >= blk) return 1;
-    const unsigned long long t0 = globaltimer();
+    const unsigned long long t0 = warp_time();
     unsigned ns = 64;
     for (;;) {
-        if (globaltimer() - t0 >= limit_ns) return 0;
+        if (warp_time() - t0 >= limit_ns) return 0;
         __nanosleep(ns);
         if (ns < 4096) ns <<= 1;
         v = load_acquire(progress);
@@ -552,91 +556,228 @@ __device__ __forceinline__ int wait_block(const int* progress, int blk, unsigned
     }
 }
 
+// What the warps of a CTA share: the item whose chains are being handed out, and the staged ligands.
+struct CtaWork {
+    int lock;                     // held by one lane for a handful of instructions
+    int done;                     // the queue is empty, or a wait ran out
+    int pending;                  // an item taken from the queue that no ligand slot was free for, -1 none
+    int blk, pos, pair, unit0;    // the current item: step block, its pair's position in the order, the pair, first unit
+    int next, count;              //                   units handed out, units in all
+    int slot;                     //                   ligand slot
+    int lig[kLigSlots];           // staged ligand, -1 none
+    int refs[kLigSlots];          // warps working on it
+    int ready[kLigSlots];         // staged in full
+};
+
+// A unit of work of one warp: one chain, or two on half warps, of a step block.
+struct WarpWork {
+    int status;                   // 0 none left, 1 taken, 2 taken and its ligand is to be staged by this warp
+    int blk, pos, pair, unit, slot;
+};
+
+// Takes the next unit for a warp. Chains of the CTA's current item are handed out one
+// by one; when it is used up the next item comes from the queue, into a ligand slot that holds its
+// ligand or that no warp works on. A warp holds no slot while it waits for one, and slots are given back when
+// their chains end, so the wait ends; a warp that waited kSlotWaitNs retires, and the warps whose chains hold
+// the slots take the waiting item when they are done.
+constexpr int kLockSpins = 1 << 22;                        // over 0.1 s
+constexpr unsigned long long kSlotWaitNs = 2000000000ull;
+constexpr unsigned long long kStageWaitNs = 1000000000ull; // a staging takes microseconds
+__device__ __forceinline__ WarpWork take_work(const SearchArgs& A, CtaWork& shared) {
+    volatile CtaWork& W = shared;
+    const bool first = (threadIdx.x & 31) == 0;
+    WarpWork w;
+    w.status = 0;
+    w.blk = w.pos = w.pair = w.unit = w.slot = 0;
+    unsigned long long t0 = 0ull;
+    for (;;) {
+        for (int spin = 0;; ++spin) {                       // the holder never waits
+            int busy = 0;
+            if (first) busy = atomicCAS(&shared.lock, 0, 1);
+            if (!__shfl_sync(PV_FULL, busy, 0)) break;
+            if (spin >= kLockSpins) {
+                if (first) atomicOr(A.err, PV_EBIT_WAIT);
+                return w;
+            }
+            __nanosleep(32);
+        }
+        __threadfence_block();
+        // every lane reads the state; the first writes it
+        int next = W.next, count = W.count, blk = W.blk, pos = W.pos, pair = W.pair, unit0 = W.unit0, slot = W.slot;
+        int t = W.pending;
+        const int done = W.done;
+        bool starved = false;
+        __syncwarp();
+        if (next >= count) {
+            if (t < 0 && !done) {
+                if (first) t = atomicAdd(A.queue, 1);
+                t = __shfl_sync(PV_FULL, t, 0);
+                if (t >= A.n_items) {
+                    if (first) W.done = 1;
+                    t = -1;
+                }
+            }
+            if (t >= 0) {
+                blk = t / A.items_per_block;
+                const int j = t - blk * A.items_per_block;
+                pos = j / A.items_per_pair;
+                unit0 = (j - pos * A.items_per_pair) * A.item_units;
+                pair = A.order[pos];
+                const int lig = A.pairs[pair].ligand;
+                int held = -1, open = -1;                   // a slot with this ligand; a slot nobody works on
+                for (int k = A.lig_slots - 1; k >= 0; --k) {
+                    if (W.lig[k] == lig) held = k;
+                    if (W.refs[k] == 0) open = k;
+                }
+                slot = held >= 0 ? held : open;
+                starved = slot < 0;
+                __syncwarp();
+                if (starved) {
+                    if (first) W.pending = t;
+                } else {
+                    next = 0;
+                    count = min(A.item_units, A.units - unit0);
+                    if (held < 0) w.status = 2;
+                    if (first) {
+                        if (held < 0) {
+                            W.lig[slot] = lig;
+                            W.ready[slot] = 0;
+                        }
+                        W.pending = -1;
+                        W.blk = blk;
+                        W.pos = pos;
+                        W.pair = pair;
+                        W.unit0 = unit0;
+                        W.count = count;
+                        W.slot = slot;
+                    }
+                }
+            }
+        }
+        if (!starved && next < count) {
+            if (w.status == 0) w.status = 1;
+            w.blk = blk;
+            w.pos = pos;
+            w.pair = pair;
+            w.slot = slot;
+            w.unit = unit0 + next;
+            if (first) {
+                W.next = next + 1;
+                atomicAdd(&shared.refs[slot], 1);
+            }
+        }
+        __threadfence_block();
+        __syncwarp();
+        if (first) atomicExch(&shared.lock, 0);
+        if (!starved) return w;
+        const unsigned long long now = warp_time();
+        if (t0 == 0ull) t0 = now;
+        if (now - t0 >= kSlotWaitNs) return w;              // the warps that hold the slots go on with it
+        __nanosleep(1000);
+    }
+}
+
 // One launch of the batched search: MC steps [step0, step1) of every chain of every pair, cut into
-// step blocks of block_steps; the queue hands out all work items (a pair's chain block) of block
-// 0, then of block 1, and so on, so no SM idles at a block boundary while the chains of the last
-// wave finish (the blocks of one chain block run in order through `progress`). Compiled for
-// several (threads per CTA, minimum CTAs per SM) bounds, i.e. register budgets, and team widths (a
-// chain per warp, or per half warp), and for both map layouts (plain, cell-packed); the runtime
-// picks one (search variant, layout).
-template <int THREADS, int MIN_CTAS, int LANES, bool FOCC, int LAYOUT>
-__global__ void __launch_bounds__(THREADS, MIN_CTAS) search_round_kernel(SearchArgs A) {
+// step blocks of block_steps; the queue hands out all work items (some chains of a pair) of block 0,
+// then of block 1, and so on, so no SM idles at a block boundary while the chains of the last
+// wave finish (the blocks of one chain run in order through `progress`). A CTA's warps are independent: each
+// takes a chain of the CTA's current item, runs its step block, publishes it and takes the next, without a
+// barrier. Chains differ in cost, so a barrier per item of a chain per warp kept the warps of 4-warp
+// CTAs waiting for 11 to 12 % of their time; and one CTA with all of an SM's warps stages a ligand once
+// where seven did (a 60-atom ligand's 28 KB held the 4-warp CTAs to 16 warps per SM, now 20). Ten pockets x
+// 1,000 chains x 100 steps, M evaluations/s: 568 -> 612 for a 30-atom ligand (variant 3), 228 -> 267 for 47 atoms,
+// 1,055 -> 1,140 for 16 atoms on half warps (variant 5), 527 -> 583 with the consistency check; 24 ligands of
+// 10-60 atoms x 5 pockets x 64 chains x 60 steps: 72.9 -> 60.8 ms (variant 1).
+// Compiled for several register budgets (threads per SM) and team widths (a chain per warp, or per half warp),
+// and for both map layouts (plain, cell-packed); the runtime picks one (search variant, layout).
+template <int THREADS, int LANES, bool FOCC, int LAYOUT>
+__global__ void __launch_bounds__(THREADS, 1) search_round_kernel(SearchArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
-    PvLigBlob& L = *reinterpret_cast<PvLigBlob*>(smem);
-    WarpScratch* scratch = reinterpret_cast<WarpScratch*>(smem + ((A.lig_smem_bytes + 127) & ~127));
-    __shared__ int s_item, s_lig, s_skip;
-    __shared__ __align__(16) PvPocket s_pocket;
+    __shared__ CtaWork s_work;
     constexpr int TPW = 32 / LANES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int team = warp * TPW + Team<LANES>::index();
-    init_scratch<LANES>(scratch[team]);
-    if (threadIdx.x == 0) s_lig = -1;
+    const int lig_bytes = (A.lig_smem_bytes + 127) & ~127;
+    PvPocket* pockets = reinterpret_cast<PvPocket*>(smem + A.lig_slots * lig_bytes);
+    WarpScratch* scratch = reinterpret_cast<WarpScratch*>(pockets + (blockDim.x >> 5));
+    WarpScratch& S = scratch[warp * TPW + Team<LANES>::index()];
+    PvPocket& P = pockets[warp];
+    init_scratch<LANES>(S);
+    if (threadIdx.x == 0) {
+        s_work.lock = 0;
+        s_work.done = 0;
+        s_work.pending = -1;
+        s_work.next = s_work.count = 0;
+        for (int k = 0; k < kLigSlots; ++k) {
+            s_work.lig[k] = -1;
+            s_work.refs[k] = 0;
+            s_work.ready[k] = 0;
+        }
+    }
+    __syncthreads();
     for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(A.queue, 1);
-        __syncthreads();
-        const int it = s_item;
-        if (it >= A.n_items) break;
-        // item `it` = step block `blk` of the work item `j` (a pair's chain block); the blocks of one
-        // chain block run in order, the first waiting, if need be, for its predecessor
-        const int blk = it / A.items_per_block, j = it - blk * A.items_per_block;
+        const WarpWork w = take_work(A, s_work);
+        if (w.status == 0) break;
+        const int blk = w.blk, pair = w.pair, slot = w.slot, at = w.pos * A.units + w.unit;
         const int step0 = A.step0 + blk * A.block_steps, step1 = min(A.step1, step0 + A.block_steps);
-        const PvItem item = A.items[j];
-        const PvPairDesc pd = A.pairs[item.pair];
-        const bool reload = pd.ligand != s_lig;
-        if (threadIdx.x < (int)(sizeof(PvPocket) / 4))
-            reinterpret_cast<int*>(&s_pocket)[threadIdx.x] =
-                reinterpret_cast<const int*>(A.pockets + pd.pocket)[threadIdx.x];
-        __syncthreads();
-        if (reload) {
-            stage_ligand<LANES>(&L, A.ligs[pd.ligand], A.slots_lo, A.slots_hi);
-            if (threadIdx.x == 0) s_lig = pd.ligand;
-        }
-        if (threadIdx.x == 0) {
-            // a block whose predecessor is not published within the bound is skipped, not run on
-            // chain records that are still being written; the work item's later blocks are
-            // skipped too (poisoned progress) and the launch reports PV_EBIT_WAIT
-            const int w = blk > 0 ? wait_block(A.progress + j, blk, A.wait_ns) : 1;
-            if (w == 0) {
-                atomicOr(A.err, PV_EBIT_WAIT);
-                atomicMax(A.progress + j, PV_PROGRESS_POISON);
-            }
-            s_skip = w != 1;
-        }
-        __syncthreads();
-        const int chain = item.chain0 + team;
-        if (s_skip) {
-            if (Team<LANES>::lane() == 0 && chain < A.C.chains) {
-                float* rec = A.chains + ((size_t)item.pair * A.C.chains + chain) * PV_CHAIN_STRIDE;
-                atomicOr(reinterpret_cast<int*>(rec + PV_CH_FLAGS), PV_EBIT_WAIT);
-            }
-            continue;
-        }
-        Site site;
-        site.maps = s_pocket.maps;
-        site.P = &s_pocket;
-        uint32_t evals = 0;
-        int flags = 0;
-        if constexpr (LANES == 32) {
-            if (chain < A.C.chains)
-                run_chain_warp<FOCC, LAYOUT>(A, L, scratch[team], site, item.pair, (uint32_t)pd.key, chain, step0,
-                                             step1, evals, flags);
+        const PvPairDesc pd = A.pairs[pair];
+        PvLigBlob& L = *reinterpret_cast<PvLigBlob*>(smem + slot * lig_bytes);
+        if (lane < (int)(sizeof(PvPocket) / 4))
+            reinterpret_cast<int*>(&P)[lane] = reinterpret_cast<const int*>(A.pockets + pd.pocket)[lane];
+        // a unit whose predecessor is not published within the bound is skipped, not run on
+        // chain records that are still being written; its later blocks are skipped too (poisoned
+        // progress) and the launch reports PV_EBIT_WAIT
+        int go = 1;
+        if (w.status == 2) {
+            stage_ligand_by<LANES>(&L, A.ligs[pd.ligand], A.slots_lo, A.slots_hi, lane, 32, [] { __syncwarp(); });
+            __threadfence_block();
+            __syncwarp();
+            if (lane == 0) atomicExch(&s_work.ready[slot], 1);
         } else {
-            run_chain<LANES, FOCC, LAYOUT>(A, L, scratch[team], site, item.pair, (uint32_t)pd.key, chain,
-                                           chain < A.C.chains, step0, step1, evals, flags);
+            volatile int* ready = &s_work.ready[slot];
+            if (!__shfl_sync(PV_FULL, *ready, 0)) {
+                const unsigned long long t0 = warp_time();
+                while (go && !__shfl_sync(PV_FULL, *ready, 0)) {
+                    if (warp_time() - t0 >= kStageWaitNs) go = 0;
+                    __nanosleep(64);
+                }
+            }
+            __threadfence_block();
         }
-        if (Team<LANES>::lane() == 0 && evals) {
-            atomicAdd(A.evals, (unsigned long long)evals);
-            if (flags) atomicOr(A.err, flags);
+        if (blk > 0 && go == 1) go = wait_block(A.progress + at, blk, A.wait_ns);
+        if (go == 0 && lane == 0) {
+            atomicOr(A.err, PV_EBIT_WAIT);
+            atomicMax(A.progress + at, PV_PROGRESS_POISON);
         }
         __syncwarp();
-        (void)lane;
-        // the chain records of this block are written: publish it to the next block's item (a
-        // maximum, so that a poisoned item stays poisoned)
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        const int chain = w.unit * TPW + Team<LANES>::index();
+        if (go != 1) {
+            if (Team<LANES>::lane() == 0 && chain < A.C.chains) {
+                float* rec = A.chains + ((size_t)pair * A.C.chains + chain) * PV_CHAIN_STRIDE;
+                atomicOr(reinterpret_cast<int*>(rec + PV_CH_FLAGS), PV_EBIT_WAIT);
+            }
+        } else {
+            Site site;
+            site.maps = P.maps;
+            site.P = &P;
+            uint32_t evals = 0;
+            int flags = 0;
+            if constexpr (LANES == 32)
+                run_chain_warp<FOCC, LAYOUT>(A, L, S, site, pair, (uint32_t)pd.key, chain, step0, step1, evals, flags);
+            else
+                run_chain<LANES, FOCC, LAYOUT>(A, L, S, site, pair, (uint32_t)pd.key, chain, chain < A.C.chains, step0,
+                                               step1, evals, flags);
+            if (Team<LANES>::lane() == 0 && evals) {
+                atomicAdd(A.evals, (unsigned long long)evals);
+                if (flags) atomicOr(A.err, flags);
+            }
+        }
+        __syncwarp();
+        // the unit's chain records are written: publish them to its next block (a maximum, so that
+        // poisoned progress stays poisoned), and give the ligand slot back
+        if (lane == 0) {
             __threadfence();
-            atomicMax(A.progress + j, blk + 1);
+            if (go == 1) atomicMax(A.progress + at, blk + 1);
+            atomicSub(&s_work.refs[slot], 1);
         }
     }
 }

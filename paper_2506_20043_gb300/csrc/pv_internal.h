@@ -74,9 +74,13 @@ cudaError_t launch_gather_probe(const PvPocket* pockets_dev, int n_pockets, int 
 
 // ---- search (pv_search.cu) ----
 struct SearchArgs {
-    const PvItem* items;
-    int n_items;
+    const int* order;              // pairs in the order they are worked on
+    int n_items;                   // step blocks x items_per_block
     int* queue;                    // work counter of this round (zeroed before the launch)
+    int items_per_pair;            // batched: an item is item_units warp loads of chains of one pair
+    int item_units;                //          (a warp load: one chain, or two on half warps)
+    int units;                     // batched: warp loads per pair
+    int lig_slots;                 // batched: ligand records a CTA stages at a time, 1 .. kLigSlots
     const PvPairDesc* pairs;
     const PvLigBlob* const* ligs;  // device pointer table
     const PvPocket* pockets;
@@ -85,9 +89,9 @@ struct SearchArgs {
     float* ring;                   // [n_pairs * chains][PV_RING_STRIDE] when C.focc > 0, else null
     PvSearchConst C;
     int step0, step1;              // the launch's MC steps
-    int items_per_block;           // batched: work items of one step block (the items array)
+    int items_per_block;           // batched: work items of one step block
     int block_steps;               // batched: MC steps per block; block b covers step0 + b * block_steps ..
-    int* progress;                 // batched: [items_per_block] step blocks finished per work item
+    int* progress;                 // batched: step blocks finished per warp load of chains
     int lig_smem_bytes;            // staging capacity for one ligand
     const unsigned long long* t0;  // start time of the dock (globaltimer)
     unsigned long long timeout_ns; // 0 = none
@@ -96,13 +100,14 @@ struct SearchArgs {
     unsigned long long* evals;
     int layout;                    // map layout the kernel reads: 0 plain, 1 cell-packed
 };
-int search_smem_bytes(int lig_bytes, int warps, int lanes);
+constexpr int kLigSlots = 4;
+int search_smem_bytes(int lig_bytes, int warps, int lanes, int lig_slots);
 // Variants of the round kernel: 0-3 run a chain per warp, 4-7 a chain per half warp (ligands of
-// at most 32 atoms and 10 torsions); within each group the launch bounds (max threads per CTA,
-// min CTAs per SM) are (512, 1), (128, 5), (128, 6), (128, 7) for a chain per warp and (512, 1),
-// (128, 5), (128, 6), (128, 8) for a chain per half warp, i.e. decreasing register budgets.
+// at most 32 atoms and 10 torsions); within each group the launch bounds are 512, 640, 768 and 896
+// (half warps: 1,024) threads per SM, i.e. decreasing register budgets.
 constexpr int kSearchVariants = 8;
-int search_variant_max_warps(int variant);
+int search_variant_max_warps(int variant);     // the warps_per_cta a caller may ask for
+int search_variant_sm_warps(int variant);      // warps per SM the register budget is for
 int search_variant_lanes(int variant);
 cudaError_t search_max_ctas_per_sm(int variant, bool focc, int layout, int warps, int smem, int* out);
 // The round kernel of a variant with the consistency check (Eq. 4-5) compiled in (pv_search_focc.cu),

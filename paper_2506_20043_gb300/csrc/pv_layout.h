@@ -110,12 +110,6 @@ enum { PV_RING_POT = 0, PV_RING_G = 160, PV_RING_F = 288, PV_RING_N = 292, PV_RI
 enum { PV_CH_CUR = 0, PV_CH_BEST = 40, PV_CH_ECUR = 76, PV_CH_EBEST = 77, PV_CH_EVALS = 78,
        PV_CH_FLAGS = 79 };
 
-// Work item of the batched search: one pair, a block of consecutive chains.
-struct PvItem {
-    int32_t pair;
-    int32_t chain0;
-};
-
 // Per-pair job description (device).
 struct PvPairDesc {
     int32_t ligand;        // index into the ligand pointer table

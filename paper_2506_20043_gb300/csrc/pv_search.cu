@@ -3,7 +3,7 @@
 //
 // Batched form: one persistent launch per round of MC steps covers every (ligand, pocket,
 // chain-block) work item; CTAs pull items from an atomic counter, stage the item's ligand tree
-// in shared memory and run one chain per warp or half warp (pv_chain.cuh; the variants with the
+// in shared memory, and their warps take its chains one by one (pv_chain.cuh; the variants with the
 // consistency check of Eq. 4-5 are compiled in pv_search_focc.cu). Plain form (comparison path, the paper's
 // organisation): one launch per pair, one thread per chain, see pv_thread.cuh.
 #include "pv_chain.cuh"
@@ -32,25 +32,26 @@ cudaError_t launch_mark_t0(unsigned long long* t0, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-int search_smem_bytes(int lig_bytes, int warps, int lanes) {
-    int lig = (lig_bytes + 127) & ~127;
-    return lig + warps * (32 / lanes) * (int)sizeof(WarpScratch);
+int search_smem_bytes(int lig_bytes, int warps, int lanes, int lig_slots) {
+    const int lig = (lig_bytes + 127) & ~127;
+    return lig_slots * lig + warps * ((int)sizeof(PvPocket) + (32 / lanes) * (int)sizeof(WarpScratch));
 }
 
 struct VariantEntry {
     const void* fn;
-    int max_threads;
+    int max_threads;       // per CTA when the caller fixes the CTA size
+    int sm_threads;        // per SM: the register budget
     int lanes;
 };
 static const VariantEntry kVariants[kSearchVariants] = {
-    {(const void*)search_round_kernel<512, 1, 32, false, 0>, 512, 32},   // widest register budget
-    {(const void*)search_round_kernel<128, 5, 32, false, 0>, 128, 32},
-    {(const void*)search_round_kernel<128, 6, 32, false, 0>, 128, 32},
-    {(const void*)search_round_kernel<128, 7, 32, false, 0>, 128, 32},   // 72 registers
-    {(const void*)search_round_kernel<512, 1, 16, false, 0>, 512, 16},   // two chains per warp
-    {(const void*)search_round_kernel<128, 5, 16, false, 0>, 128, 16},
-    {(const void*)search_round_kernel<128, 6, 16, false, 0>, 128, 16},
-    {(const void*)search_round_kernel<128, 8, 16, false, 0>, 128, 16},
+    {(const void*)search_round_kernel<512, 32, false, 0>, 512, 512, 32},   // widest register budget
+    {(const void*)search_round_kernel<640, 32, false, 0>, 128, 640, 32},
+    {(const void*)search_round_kernel<768, 32, false, 0>, 128, 768, 32},
+    {(const void*)search_round_kernel<896, 32, false, 0>, 128, 896, 32},   // 72 registers
+    {(const void*)search_round_kernel<512, 16, false, 0>, 512, 512, 16},   // two chains per warp
+    {(const void*)search_round_kernel<640, 16, false, 0>, 128, 640, 16},
+    {(const void*)search_round_kernel<768, 16, false, 0>, 128, 768, 16},
+    {(const void*)search_round_kernel<1024, 16, false, 0>, 128, 1024, 16},
 };
 static int g_variant_smem[4][kSearchVariants][64];
 
@@ -65,13 +66,18 @@ int search_variant_max_warps(int variant) {
     return kVariants[variant].max_threads / 32;
 }
 
+int search_variant_sm_warps(int variant) {
+    if (variant < 0 || variant >= kSearchVariants) return 0;
+    return kVariants[variant].sm_threads / 32;
+}
+
 int search_variant_lanes(int variant) {
     if (variant < 0 || variant >= kSearchVariants) return 0;
     return kVariants[variant].lanes;
 }
 
 cudaError_t search_max_ctas_per_sm(int variant, bool focc, int layout, int warps, int smem, int* out) {
-    if (variant < 0 || variant >= kSearchVariants || warps * 32 > kVariants[variant].max_threads ||
+    if (variant < 0 || variant >= kSearchVariants || warps * 32 > kVariants[variant].sm_threads ||
         (layout != 0 && layout != 1))
         return cudaErrorInvalidValue;
     const void* fn = variant_fn(variant, focc, layout);
@@ -81,12 +87,13 @@ cudaError_t search_max_ctas_per_sm(int variant, bool focc, int layout, int warps
 }
 
 cudaError_t launch_search_round(const SearchArgs& a, int variant, int grid, int warps, cudaStream_t s) {
-    if (variant < 0 || variant >= kSearchVariants || warps * 32 > kVariants[variant].max_threads)
+    if (variant < 0 || variant >= kSearchVariants || warps * 32 > kVariants[variant].sm_threads || a.lig_slots < 1 ||
+        a.lig_slots > kLigSlots)
         return cudaErrorInvalidValue;
     const bool focc = a.C.focc > 0;
     if ((focc && !a.ring) || (a.layout != 0 && a.layout != 1)) return cudaErrorInvalidValue;
     const void* fn = variant_fn(variant, focc, a.layout);
-    const int smem = search_smem_bytes(a.lig_smem_bytes, warps, kVariants[variant].lanes);
+    const int smem = search_smem_bytes(a.lig_smem_bytes, warps, kVariants[variant].lanes, a.lig_slots);
     cudaError_t e = ensure_smem(fn, smem, g_variant_smem[2 * a.layout + (focc ? 1 : 0)][variant]);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&a};

@@ -7,10 +7,10 @@ namespace pv {
 
 const void* search_focc_kernel(int variant) {
     static const void* const kFns[kSearchVariants] = {
-        (const void*)search_round_kernel<512, 1, 32, true, 0>, (const void*)search_round_kernel<128, 5, 32, true, 0>,
-        (const void*)search_round_kernel<128, 6, 32, true, 0>, (const void*)search_round_kernel<128, 7, 32, true, 0>,
-        (const void*)search_round_kernel<512, 1, 16, true, 0>, (const void*)search_round_kernel<128, 5, 16, true, 0>,
-        (const void*)search_round_kernel<128, 6, 16, true, 0>, (const void*)search_round_kernel<128, 8, 16, true, 0>,
+        (const void*)search_round_kernel<512, 32, true, 0>, (const void*)search_round_kernel<640, 32, true, 0>,
+        (const void*)search_round_kernel<768, 32, true, 0>, (const void*)search_round_kernel<896, 32, true, 0>,
+        (const void*)search_round_kernel<512, 16, true, 0>, (const void*)search_round_kernel<640, 16, true, 0>,
+        (const void*)search_round_kernel<768, 16, true, 0>, (const void*)search_round_kernel<1024, 16, true, 0>,
     };
     return variant >= 0 && variant < kSearchVariants ? kFns[variant] : nullptr;
 }

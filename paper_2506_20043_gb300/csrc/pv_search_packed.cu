@@ -7,10 +7,10 @@ namespace pv {
 
 const void* search_packed_kernel(int variant) {
     static const void* const kFns[kSearchVariants] = {
-        (const void*)search_round_kernel<512, 1, 32, false, 1>, (const void*)search_round_kernel<128, 5, 32, false, 1>,
-        (const void*)search_round_kernel<128, 6, 32, false, 1>, (const void*)search_round_kernel<128, 7, 32, false, 1>,
-        (const void*)search_round_kernel<512, 1, 16, false, 1>, (const void*)search_round_kernel<128, 5, 16, false, 1>,
-        (const void*)search_round_kernel<128, 6, 16, false, 1>, (const void*)search_round_kernel<128, 8, 16, false, 1>,
+        (const void*)search_round_kernel<512, 32, false, 1>, (const void*)search_round_kernel<640, 32, false, 1>,
+        (const void*)search_round_kernel<768, 32, false, 1>, (const void*)search_round_kernel<896, 32, false, 1>,
+        (const void*)search_round_kernel<512, 16, false, 1>, (const void*)search_round_kernel<640, 16, false, 1>,
+        (const void*)search_round_kernel<768, 16, false, 1>, (const void*)search_round_kernel<1024, 16, false, 1>,
     };
     return variant >= 0 && variant < kSearchVariants ? kFns[variant] : nullptr;
 }

@@ -27,20 +27,21 @@ __device__ __forceinline__ int staged_meta(int meta) {
 // Copies the fixed part and the pair schedule of a team of LANES lanes of `src` into `dst`
 // (16-byte words; the other width's schedule is left out, and a half-warp copy holds its schedule
 // at slot 0), the schedule in its staged form, then writes each atom's map slot into bits 16-23 of its
-// packed word. Ends with __syncthreads().
+// packed word. `threads` threads take part, this one being the tid-th; sync() is their barrier, called at
+// the end too.
 static_assert(PV_LIG_FIXED_BYTES % 16 == 0 && sizeof(PvPairSlot) == 16, "ligand record is staged in 16-byte words");
-template <int LANES = 32>
-__device__ __forceinline__ void stage_ligand(PvLigBlob* dst, const PvLigBlob* __restrict__ src,
-                                             uint64_t slots_lo, uint64_t slots_hi) {
+template <int LANES, typename Sync>
+__device__ __forceinline__ void stage_ligand_by(PvLigBlob* dst, const PvLigBlob* __restrict__ src, uint64_t slots_lo,
+                                                uint64_t slots_hi, int tid, int threads, Sync&& sync) {
     const int fixed = PV_LIG_FIXED_BYTES / 16;
     const int rounds = LANES == 32 ? src->h.n_rounds : src->h.n_rounds16;
     const int first = LANES == 32 ? 0 : src->h.pairs16_at;
     const int4* s = reinterpret_cast<const int4*>(src);
     int4* d = reinterpret_cast<int4*>(dst);
-    for (int i = threadIdx.x; i < fixed; i += blockDim.x) d[i] = __ldg(s + i);
+    for (int i = tid; i < fixed; i += threads) d[i] = __ldg(s + i);
     const int4* sp = reinterpret_cast<const int4*>(src->pairs + first);
     int4* dp = reinterpret_cast<int4*>(dst->pairs);
-    for (int i = threadIdx.x; i < ((rounds + 1) >> 1) * LANES; i += blockDim.x) {
+    for (int i = tid; i < ((rounds + 1) >> 1) * LANES; i += threads) {
         const int at = 2 * (i & ~(LANES - 1)) + (i & (LANES - 1));   // the lane's slot of round 2 q
         int4 a = __ldg(sp + at);
         a.x = staged_meta(a.x);
@@ -52,17 +53,24 @@ __device__ __forceinline__ void stage_ligand(PvLigBlob* dst, const PvLigBlob* __
             dp[at] = a;
         }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) dst->h.pairs16_at = 0;
+    sync();
+    if (tid == 0) dst->h.pairs16_at = 0;
     const int n = dst->h.n_atoms;
-    for (int a = threadIdx.x; a < n; a += blockDim.x) {
+    for (int a = tid; a < n; a += threads) {
         int w = __float_as_int(dst->atom[a].w);
         int xs = (w >> 8) & 255;
         int slot = slot_of(slots_lo, slots_hi, xs);
         w = (w & 0xffff) | ((slot & 255) << 16);
         dst->atom[a].w = __int_as_float(w);
     }
-    __syncthreads();
+    sync();
+}
+
+// By the whole CTA, ending with __syncthreads().
+template <int LANES = 32>
+__device__ __forceinline__ void stage_ligand(PvLigBlob* dst, const PvLigBlob* __restrict__ src, uint64_t slots_lo,
+                                             uint64_t slots_hi) {
+    stage_ligand_by<LANES>(dst, src, slots_lo, slots_hi, threadIdx.x, blockDim.x, [] { __syncthreads(); });
 }
 
 }  // namespace pv

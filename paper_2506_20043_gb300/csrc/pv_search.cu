@@ -154,35 +154,75 @@ __device__ void bitonic_sort(unsigned long long* keys, int n) {
     }
 }
 
+// Square distance of a point from a box, a little less than that of any point in it allows for rounding.
+__device__ __forceinline__ float box_distance2(const float3 lo, const float3 hi, const float4 p) {
+    const float ex = fmaxf(0.f, fmaxf(lo.x - p.x, p.x - hi.x)), ey = fmaxf(0.f, fmaxf(lo.y - p.y, p.y - hi.y)),
+                ez = fmaxf(0.f, fmaxf(lo.z - p.z, p.z - hi.z));
+    return 0.999f * (ex * ex + ey * ey + ez * ez);
+}
+
 // e_inter of the pose in S.x summed directly over the pocket's receptor atoms within the 8 A
-// cutoff (no grid, no box): the whole warp, lanes over ligand atoms, receptor atoms broadcast.
+// cutoff (no grid, no box): the whole warp, lanes over ligand atoms, receptor atoms broadcast in their
+// order. Receptor atoms are read 32 at a time, a lane each, and only those within the cutoff of the pose's
+// box (a few hundred of thousands) are broadcast: 120 pairs of 9 poses over 6,000 atoms took 2.0 of the
+// selection's 2.25 ms when every atom was, one load after another; it is 0.50 ms now.
 __device__ float direct_inter(const PvLigBlob& L, const WarpScratch& S, const PvPocket& P) {
     const int lane = threadIdx.x & 31, n = L.h.n_atoms;
     float4 xi[2];
     int ti[2];
+    float3 lo = make_float3(INFINITY, INFINITY, INFINITY), hi = make_float3(-INFINITY, -INFINITY, -INFINITY);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int a = lane + 32 * h;
         xi[h] = a < n ? S.x[a] : make_float4(1e30f, 1e30f, 1e30f, 0.f);
         ti[h] = a < n ? ((__float_as_int(L.atom[a].w) >> 8) & 255) : 0;
+        if (a < n) {
+            lo = make_float3(fminf(lo.x, xi[h].x), fminf(lo.y, xi[h].y), fminf(lo.z, xi[h].z));
+            hi = make_float3(fmaxf(hi.x, xi[h].x), fmaxf(hi.y, xi[h].y), fmaxf(hi.z, xi[h].z));
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = make_float3(fminf(lo.x, __shfl_xor_sync(PV_FULL, lo.x, o)), fminf(lo.y, __shfl_xor_sync(PV_FULL, lo.y, o)),
+                         fminf(lo.z, __shfl_xor_sync(PV_FULL, lo.z, o)));
+        hi = make_float3(fmaxf(hi.x, __shfl_xor_sync(PV_FULL, hi.x, o)), fmaxf(hi.y, __shfl_xor_sync(PV_FULL, hi.y, o)),
+                         fmaxf(hi.z, __shfl_xor_sync(PV_FULL, hi.z, o)));
     }
     float e = 0.f;
-    for (int j = 0; j < P.rec_n; ++j) {
-        const float4 r = __ldg(P.rec_atoms + j);
-        const int tj = __float_as_int(r.w);
+    const float4 far = make_float4(1e30f, 1e30f, 1e30f, 0.f);
+    float4 next = lane < P.rec_n ? __ldg(P.rec_atoms + lane) : far;
+    for (int j0 = 0; j0 < P.rec_n; j0 += 32) {
+        const float4 mine = next;
+        next = j0 + 32 + lane < P.rec_n ? __ldg(P.rec_atoms + j0 + 32 + lane) : far;
+        for (unsigned m = __ballot_sync(PV_FULL, box_distance2(lo, hi, mine) < kCutoff2); m; m &= m - 1) {
+            const int t = __ffs(m) - 1;
+            const float4 r = make_float4(__shfl_sync(PV_FULL, mine.x, t), __shfl_sync(PV_FULL, mine.y, t),
+                                         __shfl_sync(PV_FULL, mine.z, t), __shfl_sync(PV_FULL, mine.w, t));
+            const int tj = __float_as_int(r.w);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float dx = xi[h].x - r.x, dy = xi[h].y - r.y, dz = xi[h].z - r.z;
-            const float r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 < kCutoff2) {
-                const bool hyd = xs_hydrophobic(ti[h]) && xs_hydrophobic(tj);
-                const bool hb = (xs_donor(ti[h]) && xs_acceptor(tj)) || (xs_acceptor(ti[h]) && xs_donor(tj));
-                float c;
-                e += vina_pair_r2(r2, xi[h].w + xs_radius(tj), hyd, hb, c);
+            for (int h = 0; h < 2; ++h) {
+                const float dx = xi[h].x - r.x, dy = xi[h].y - r.y, dz = xi[h].z - r.z;
+                const float r2 = dx * dx + dy * dy + dz * dz;
+                if (r2 < kCutoff2) {
+                    const bool hyd = xs_hydrophobic(ti[h]) && xs_hydrophobic(tj);
+                    const bool hb = (xs_donor(ti[h]) && xs_acceptor(tj)) || (xs_acceptor(ti[h]) && xs_donor(tj));
+                    float c;
+                    e += vina_pair_r2(r2, xi[h].w + xs_radius(tj), hyd, hb, c);
+                }
             }
         }
     }
     return warp_sum(e);
+}
+
+// Sum over the ligand's atoms of the square distance between two posed copies (whole warp).
+__device__ __forceinline__ float square_distance(const float4* p, const float4* q, int n) {
+    float s2 = 0.f;
+    for (int a = threadIdx.x & 31; a < n; a += 32) {
+        const float4 x = p[a], y = q[a];
+        s2 += (x.x - y.x) * (x.x - y.x) + (x.y - y.y) * (x.y - y.y) + (x.z - y.z) * (x.z - y.z);
+    }
+    return warp_sum(s2);
 }
 
 __global__ void __launch_bounds__(kTopkThreads) topk_kernel(TopkArgs A) {
@@ -198,7 +238,7 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(TopkArgs A) {
     while (n_sort < C.chains) n_sort <<= 1;
     unsigned long long* keys = reinterpret_cast<unsigned long long*>(kept_xyz + kMaxTopK * 64);
     __shared__ int s_kept[kMaxTopK];
-    __shared__ int s_nkept, s_status;
+    __shared__ int s_nkept, s_status, s_ok[kTopkThreads / 32];
     __shared__ PvPocket s_pocket;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     init_scratch<32>(scratch[warp]);
@@ -223,38 +263,43 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(TopkArgs A) {
     bitonic_sort(keys, n_sort);
     const int n = L.h.n_atoms, n_rot = L.h.n_rot;
     const int k_max = min(C.top_k, kMaxTopK);
-    if (warp == 0) {
-        WarpScratch& S = scratch[0];
-        int kept = 0;
-        const float thr2 = C.rmsd_min * C.rmsd_min * (float)n;
-        for (int idx = 0; idx < C.chains && kept < k_max; ++idx) {
-            const unsigned long long key = keys[idx];
-            if ((key >> 32) == 0xffffffffull) break;   // NaN scores are never kept
-            const int ch = (int)(key & 0xffffffffu);
-            Pose x = load_pose<32>(chains + (size_t)ch * PV_CHAIN_STRIDE + PV_CH_BEST, n_rot);
-            float3 axw, xa;
-            warp_fk(L, S, x, axw, xa);
-            __syncwarp();
-            bool ok = true;
-            for (int b = 0; b < kept && ok; ++b) {
-                float s2 = 0.f;
-                for (int a = lane; a < n; a += 32) {
-                    float4 p = S.x[a], q = kept_xyz[b * 64 + a];
-                    s2 += (p.x - q.x) * (p.x - q.x) + (p.y - q.y) * (p.y - q.y) + (p.z - q.z) * (p.z - q.z);
-                }
-                s2 = warp_sum(s2);
-                if (s2 < thr2) ok = false;
-            }
-            if (ok) {
-                for (int a = lane; a < n; a += 32) kept_xyz[kept * 64 + a] = S.x[a];
-                if (lane == 0) s_kept[kept] = ch;
-                kept++;
-            }
-            __syncwarp();
-        }
-        if (lane == 0) s_nkept = kept;
-    }
+    // The greedy filter, W candidates at a time in order of SF: each warp poses one and compares it with the
+    // poses kept before the batch, then warp 0 takes those that pass, in order, unless one kept from the same
+    // batch is too near. One warp alone, candidate after candidate, took 0.57 ms for 10 pairs of 1,000 chains;
+    // 0.22 ms.
+    const float thr2 = C.rmsd_min * C.rmsd_min * (float)n;
+    if (threadIdx.x == 0) s_nkept = 0;
     __syncthreads();
+    for (int base = 0; base < C.chains; base += W) {
+        const int kept = s_nkept;
+        if (kept >= k_max || (keys[base] >> 32) == 0xffffffffull) break;    // NaN scores (last) are never kept
+        const int idx = base + warp;
+        const unsigned long long key = idx < C.chains ? keys[idx] : ~0ull;
+        bool ok = (key >> 32) != 0xffffffffull;
+        if (ok) {
+            const Pose x = load_pose<32>(chains + (size_t)(key & 0xffffffffu) * PV_CHAIN_STRIDE + PV_CH_BEST, n_rot);
+            float3 axw, xa;
+            warp_fk(L, scratch[warp], x, axw, xa);
+            __syncwarp();
+            for (int b = 0; b < kept && ok; ++b) ok = !(square_distance(scratch[warp].x, kept_xyz + b * 64, n) < thr2);
+        }
+        if (lane == 0) s_ok[warp] = ok;
+        __syncthreads();
+        if (warp == 0) {
+            int now = kept;
+            for (int c = 0; c < W && now < k_max; ++c) {
+                bool take = s_ok[c];
+                for (int b = kept; b < now && take; ++b) take = !(square_distance(scratch[c].x, kept_xyz + b * 64, n) < thr2);
+                if (!take) continue;
+                for (int a = lane; a < n; a += 32) kept_xyz[now * 64 + a] = scratch[c].x[a];
+                if (lane == 0) s_kept[now] = (int)(keys[base + c] & 0xffffffffu);
+                __syncwarp();
+                ++now;
+            }
+            if (lane == 0) s_nkept = now;
+        }
+        __syncthreads();
+    }
     const int kept = s_nkept;
     // the kept poses' SF parts from the grid, one warp each; with C.rescore also e_inter summed
     // directly over the receptor's atoms (Algorithm 2's rescoring of the selected poses)

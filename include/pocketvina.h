@@ -203,6 +203,11 @@ pv_status pv_score_backward(pv_context* ctx, const pv_grid_set* set, const pv_li
                             const float* dev_grad_energy, float* dev_grad_pose,
                             float* dev_grad_xyz);
 
+/* Both at once from one evaluation per pose: dev_energy[n] = SF and dev_grad_pose[n][7 + n_rot] =
+ * dSF/dPOT (pv_score_backward's with dE = 1). */
+pv_status pv_score_value_grad(pv_context* ctx, const pv_grid_set* set, const pv_ligand* lig, int32_t pocket,
+                              int32_t n_poses, const float* dev_pose, float* dev_energy, float* dev_grad_pose);
+
 /* SF (Eq. 3) of posed ligands given by their atom coordinates rather than POTs, for automatic
  * differentiation over ligand coordinates: dev_xyz [n][n_atoms][3] float32, input atom order.
  * e_inter is interpolated from the pocket's maps as in pv_score (same out-of-grid rule), e_intra

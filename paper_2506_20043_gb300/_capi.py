@@ -86,6 +86,7 @@ SIGNATURES = {
     "pv_ligand_xs_types": (i32, [vp, C.POINTER(C.c_uint8)]),
     "pv_score": (i32, [vp, vp, vp, i32, i32, vp, vp, vp, vp]),
     "pv_score_backward": (i32, [vp, vp, vp, i32, i32, vp, vp, vp, vp]),
+    "pv_score_value_grad": (i32, [vp, vp, vp, i32, i32, vp, vp, vp]),
     "pv_pose_coords": (i32, [vp, vp, i32, vp, vp]),
     "pv_score_xyz": (i32, [vp, vp, vp, i32, i32, vp, vp, vp, vp]),
     "pv_measure_gather": (i32, [vp, vp, i32, i64, i32, vp]),

@@ -339,6 +339,17 @@ class Context:
                                                gx.data_ptr() if gx is not None else None), "pv_score_backward")
         return gp, gx
 
+    def score_value_grad(self, grids: "GridSet", lig: "Ligand", pocket: int, poses):
+        """SF of poses [n, 7 + n_rot] and dSF/dPOT [n, 7 + n_rot] from one evaluation per pose."""
+        torch = self.torch
+        poses = poses.to(device=f"cuda:{self.device}", dtype=torch.float32).contiguous()
+        n = poses.shape[0]
+        e = torch.empty(n, device=poses.device, dtype=torch.float32)
+        g = torch.empty_like(poses)
+        self._check(self.lib.pv_score_value_grad(self.h, grids.h, lig.h, int(pocket), n, poses.data_ptr(), e.data_ptr(),
+                                                 g.data_ptr()), "pv_score_value_grad")
+        return e, g
+
     def score_xyz(self, grids: "GridSet", lig: "Ligand", pocket: int, xyz, grad: bool = True, grad_energy=None):
         """SF (Eq. 3) of posed atom coordinates xyz [n, n_atoms, 3] (input order, cuda float32).
         Returns (energy [n] or None when grad_energy is given, dSF/dxyz [n, n_atoms, 3] scaled by
@@ -612,10 +623,18 @@ class DockResult:
             self.h = None
 
 
+def _scaled(g, ge):
+    """Rows of g times the incoming gradient ge [n] (whatever shape the rows were given in), a constant to
+    further differentiation."""
+    return g * (ge.detach() if ge.requires_grad else ge).view((-1,) + (1,) * (g.dim() - 1))
+
+
 class PVScore:
     """torch.autograd.Function over pose parameters: energy = SF(pose) for one ligand in one
-    pocket; backward is the library's adjoint kernel (the gradient BFGS consumes), mapped to POT
-    coordinates (translation, raw quaternion, torsions)."""
+    pocket; the gradient is the library's adjoint (the gradient BFGS consumes), mapped to POT
+    coordinates (translation, raw quaternion, torsions). An evaluation with the gradient costs little more
+    than one without, so when the pose needs a gradient the forward pass keeps it and the backward
+    scales it, instead of evaluating every pose again."""
 
     _fn = None
 
@@ -627,17 +646,17 @@ class PVScore:
             class _F(torch.autograd.Function):
                 @staticmethod
                 def forward(fctx, pose_t, pv_ctx, grids_, lig_, pocket_):
-                    e, _, _ = pv_ctx.score(grids_, lig_, pocket_, pose_t.detach(), grad=False)
-                    fctx.save_for_backward(pose_t)
-                    fctx.pv = (pv_ctx, grids_, lig_, pocket_)
+                    if not fctx.needs_input_grad[0]:
+                        return pv_ctx.score(grids_, lig_, pocket_, pose_t.detach(), grad=False)[0]
+                    e, g = pv_ctx.score_value_grad(grids_, lig_, pocket_, pose_t.detach())
+                    fctx.save_for_backward(pose_t, g)
                     return e
 
                 @staticmethod
                 def backward(fctx, ge):
-                    (pose_t,) = fctx.saved_tensors
-                    pv_ctx, grids_, lig_, pocket_ = fctx.pv
-                    gp, _ = pv_ctx.score_backward(grids_, lig_, pocket_, pose_t.detach(), ge.contiguous())
-                    return gp.to(pose_t.dtype), None, None, None, None
+                    pose_t, g = fctx.saved_tensors
+                    g = _scaled(g, ge)
+                    return g if g.dtype == pose_t.dtype else g.to(pose_t.dtype), None, None, None, None
 
             cls._fn = _F
         return cls._fn.apply(pose, ctx, grids, lig, pocket)
@@ -645,8 +664,8 @@ class PVScore:
 
 class PVScoreXYZ:
     """torch.autograd.Function over ligand atom coordinates: energy = SF(xyz) for posed atoms
-    [n, n_atoms, 3] of one ligand in one pocket; backward is the library's coordinate gradient
-    (dSF/dx_i scaled by the incoming gradient in the kernel)."""
+    [n, n_atoms, 3] of one ligand in one pocket; the gradient is the library's coordinate gradient
+    dSF/dx_i, kept by the forward pass when it is needed and scaled by the incoming gradient."""
 
     _fn = None
 
@@ -658,17 +677,17 @@ class PVScoreXYZ:
             class _F(torch.autograd.Function):
                 @staticmethod
                 def forward(fctx, xyz_t, pv_ctx, grids_, lig_, pocket_):
-                    e, _ = pv_ctx.score_xyz(grids_, lig_, pocket_, xyz_t.detach(), grad=False)
-                    fctx.save_for_backward(xyz_t)
-                    fctx.pv = (pv_ctx, grids_, lig_, pocket_)
+                    need = fctx.needs_input_grad[0]
+                    e, g = pv_ctx.score_xyz(grids_, lig_, pocket_, xyz_t.detach(), grad=need)
+                    if need:
+                        fctx.save_for_backward(xyz_t, g)
                     return e
 
                 @staticmethod
                 def backward(fctx, ge):
-                    (xyz_t,) = fctx.saved_tensors
-                    pv_ctx, grids_, lig_, pocket_ = fctx.pv
-                    _, gx = pv_ctx.score_xyz(grids_, lig_, pocket_, xyz_t.detach(), grad_energy=ge.contiguous())
-                    return gx.to(xyz_t.dtype), None, None, None, None
+                    xyz_t, g = fctx.saved_tensors
+                    g = _scaled(g, ge)
+                    return g if g.dtype == xyz_t.dtype else g.to(xyz_t.dtype), None, None, None, None
 
             cls._fn = _F
         return cls._fn.apply(xyz, ctx, grids, lig, pocket)

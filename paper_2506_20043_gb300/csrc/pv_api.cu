@@ -665,6 +665,21 @@ extern "C" pv_status pv_score_backward(pv_context* ctx, const pv_grid_set* set, 
     return PV_OK;
 }
 
+extern "C" pv_status pv_score_value_grad(pv_context* ctx, const pv_grid_set* set, const pv_ligand* lig,
+                                         int32_t pocket, int32_t n_poses, const float* dev_pose, float* dev_energy,
+                                         float* dev_grad_pose) {
+    NvtxRange nvtx("pv_score_value_grad");
+    pv_status st = check_score_args(ctx, set, lig, pocket, n_poses);
+    if (st != PV_OK) return st;
+    if (n_poses == 0) return PV_OK;
+    if (!dev_pose || !dev_energy || !dev_grad_pose) return fail(ctx, PV_ERR_ARG, "pose, energy and grad_pose required");
+    DeviceGuard g(ctx->device);
+    PV_CU(ctx, launch_score((const PvLigBlob*)lig->d_blob, lig->rec.staged32, set->d_pockets + pocket,
+                            slots_of(set), n_poses, 7 + lig->rec.n_rot, dev_pose, dev_energy, nullptr, nullptr,
+                            nullptr, dev_grad_pose, nullptr, set->packed ? 1 : 0, ctx->stream));
+    return PV_OK;
+}
+
 extern "C" pv_status pv_score_xyz(pv_context* ctx, const pv_grid_set* set, const pv_ligand* lig, int32_t pocket,
                                   int32_t n_poses, const float* dev_xyz, const float* dev_grad_energy,
                                   float* dev_energy, float* dev_grad_xyz) {

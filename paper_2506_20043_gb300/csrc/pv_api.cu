@@ -2,6 +2,7 @@
 // docking driver (batched rounds captured in a CUDA graph, or the plain per-pair loop).
 #include <algorithm>
 #include <map>
+#include <memory>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -17,6 +18,8 @@
 using namespace pv;
 
 static constexpr int kCtxMagic = 0x50564358;   // "PVCX"
+static constexpr size_t kStagedCopy = 65536;    // bytes of a pageable copy that does not wait for the stream
+static constexpr size_t kTableInline = 64;      // pockets of a table kept beside the maps
 static constexpr float kCellEdge = 3.0f;        // receptor binning cell, A
 static constexpr double kRecCutoff = 8.0;       // receptor atoms beyond this never reach a node
 
@@ -42,7 +45,8 @@ struct pv_grid_set {
     int n_maps = 0;
     int type_mask = 0;
     std::vector<PvPocket> pockets;
-    PvPocket* d_pockets = nullptr;
+    PvPocket* d_pockets = nullptr;  // the pocket table: in the newest arena, or
+    void* table = nullptr;          // an allocation of its own
     std::vector<void*> arenas;
     int64_t bytes = 0;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> map_events;   // around each map-build launch
@@ -299,61 +303,67 @@ static pv_status add_receptor(pv_context* ctx, pv_grid_set* set, const pv_recept
     const long long n_cells = (long long)cd[0] * cd[1] * cd[2];
     if (n_cells > (1 << 24)) return fail(ctx, PV_ERR_ARG, "pocket boxes span too large a region");
     const int first = (int)set->pockets.size();
-    // maps arena, and the typed receptor kept for direct rescoring of poses
-    float* arena = (float*)dalloc(ctx, map_floats * sizeof(float));
-    if (!arena) return fail(ctx, PV_ERR_OOM, "map allocation failed");
-    set->arenas.push_back(arena);
-    set->bytes += (int64_t)(map_floats * sizeof(float));
-    float4* typed = (float4*)dalloc(ctx, sizeof(float4) * (size_t)n);
-    if (!typed) return fail(ctx, PV_ERR_OOM, "receptor allocation failed");
-    set->arenas.push_back(typed);
-    size_t off = 0;
+    // An allocation or a release calls the allocator of the framework around, 4 us each (a build of one small box
+    // 98 -> 88 us, with the copies below), so there is one allocation kept by the set: the maps, the typed receptor (for direct rescoring of poses), the cell-packed
+    // maps when the set keeps them too, and the table of all its pockets while that is small (a large one is
+    // replaced at every append, and given back).
+    size_t cells = 0;
+    if (set->packed)
+        for (int p = 0; p < n_pockets; ++p) cells += (size_t)pk[p].ncells * set->n_maps;
+    const size_t n_table = set->pockets.size() + n_pockets;
+    Layout K;
+    const size_t o_maps = K.take<float>(map_floats), o_typed = K.take<float4>(n), o_cells = K.take<float4>(2 * cells),
+                 o_table = K.take<PvPocket>(n_table <= kTableInline ? n_table : 0);
+    char* kept = (char*)dalloc(ctx, K.off);
+    if (!kept) return fail(ctx, PV_ERR_OOM, "map allocation failed");
+    set->arenas.push_back(kept);
+    set->bytes += (int64_t)(map_floats * sizeof(float) + cells * 2 * sizeof(float4));
+    float4* typed = (float4*)(kept + o_typed);
+    size_t off = 0, co = 0;
     for (int p = 0; p < n_pockets; ++p) {
-        pk[p].maps = arena + off;
+        pk[p].maps = (float*)(kept + o_maps) + off;
         off += (size_t)pk[p].nxyz * set->n_maps;
         pk[p].rec_atoms = typed;
         pk[p].rec_n = n;
-    }
-    if (set->packed) {   // the set keeps the cell-packed layout too: pack the new pockets as well
-        size_t cells = 0;
-        for (int p = 0; p < n_pockets; ++p) cells += (size_t)pk[p].ncells * set->n_maps;
-        float4* carena = (float4*)dalloc(ctx, cells * 2 * sizeof(float4));
-        if (!carena) return fail(ctx, PV_ERR_OOM, "packed map allocation failed");
-        set->arenas.push_back(carena);
-        set->bytes += (int64_t)(cells * 2 * sizeof(float4));
-        size_t co = 0;
-        for (int p = 0; p < n_pockets; ++p) {
-            pk[p].cells = carena + co;
+        if (set->packed) {
+            pk[p].cells = (float4*)(kept + o_cells) + co;
             co += (size_t)pk[p].ncells * set->n_maps * 2;
         }
     }
-    // pocket table (all pockets of the set)
     set->pockets.insert(set->pockets.end(), pk.begin(), pk.end());
-    PvPocket* d_p = (PvPocket*)dalloc(ctx, sizeof(PvPocket) * set->pockets.size());
-    if (!d_p) return fail(ctx, PV_ERR_OOM, "pocket table allocation failed");
-    PV_CU(ctx, cudaMemcpyAsync(d_p, set->pockets.data(), sizeof(PvPocket) * set->pockets.size(),
-                               cudaMemcpyHostToDevice, ctx->stream));
-    // scratch
+    void* table = nullptr;
+    if (n_table > kTableInline && !(table = dalloc(ctx, sizeof(PvPocket) * n_table)))
+        return fail(ctx, PV_ERR_OOM, "pocket table allocation failed");
+    PvPocket* d_p = table ? (PvPocket*)table : (PvPocket*)(kept + o_table);
+    // scratch: the receptor's arrays first (host arrays go up in one copy), head beside sorted (cleared together)
     Layout L;
     const size_t o_xyz = L.take<float>(3 * (size_t)n), o_el = L.take<uint8_t>(n), o_don = L.take<uint8_t>(n),
-                 o_acc = L.take<uint8_t>(n), o_sorted = L.take<float4>(n),
-                 o_cof = L.take<int>(n), o_next = L.take<int>(n), o_head = L.take<int>(n_cells),
-                 o_start = L.take<int>(n_cells + 1);
+                 o_acc = L.take<uint8_t>(n), up_bytes = L.off, o_head = L.take<int>(n_cells), o_sorted = L.take<float4>(n),
+                 o_cof = L.take<int>(n), o_next = L.take<int>(n), o_start = L.take<int>(n_cells + 1);
     char* w = (char*)dalloc(ctx, L.off);
-    if (!w) return fail(ctx, PV_ERR_OOM, "grid scratch allocation failed");
+    if (!w) {
+        dfree(ctx, table);
+        return fail(ctx, PV_ERR_OOM, "grid scratch allocation failed");
+    }
     const float* xyz = (const float*)r->xyz;
     const uint8_t *el = r->element, *don = r->donor, *acc = r->acceptor;
-    cudaError_t e = cudaSuccess;
     const char* stage = "receptor upload";
-    if (r->mem == PV_MEM_HOST) {
-        e = cudaMemcpyAsync(w + o_xyz, r->xyz, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(w + o_el, r->element, n, cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(w + o_don, r->donor, n, cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(w + o_acc, r->acceptor, n, cudaMemcpyHostToDevice, ctx->stream);
-        // copies from page-locked memory are still in flight on return (pageable sources have been
-        // staged): wait for them, so the caller may reuse its arrays once the call returns
-        if (e == cudaSuccess && host_pinned(r->xyz, r->element, r->donor, r->acceptor))
-            e = cudaStreamSynchronize(ctx->stream);
+    cudaError_t e = cudaMemcpyAsync(d_p, set->pockets.data(), sizeof(PvPocket) * n_table, cudaMemcpyHostToDevice, ctx->stream);
+    if (r->mem == PV_MEM_HOST && e == cudaSuccess) {
+        // through one pageable buffer: such a copy has been taken from it when the call returns, so the caller's
+        // arrays, page-locked or not, are its own again. One copy for four arrays and no wait for a page-locked
+        // receptor; in pieces, because a pageable copy of more than 64 KB waits for all the stream has queued
+        // (36 ms behind 36 ms of work; 20 us at 64 KB).
+        const std::unique_ptr<char[]> up(new (std::nothrow) char[up_bytes]());
+        if (up) {
+            std::memcpy(&up[o_xyz], r->xyz, sizeof(float) * 3 * (size_t)n);
+            std::memcpy(&up[o_el], r->element, n);
+            std::memcpy(&up[o_don], r->donor, n);
+            std::memcpy(&up[o_acc], r->acceptor, n);
+        }
+        else e = cudaErrorMemoryAllocation;
+        for (size_t at = 0; at < up_bytes && e == cudaSuccess; at += kStagedCopy)
+            e = cudaMemcpyAsync(w + at, &up[at], std::min(kStagedCopy, up_bytes - at), cudaMemcpyHostToDevice, ctx->stream);
         xyz = (const float*)(w + o_xyz);
         el = (const uint8_t*)(w + o_el);
         don = (const uint8_t*)(w + o_don);
@@ -383,12 +393,13 @@ static pv_status add_receptor(pv_context* ctx, pv_grid_set* set, const pv_recept
     }
     if (e != cudaSuccess) {
         dfree(ctx, w);
-        dfree(ctx, d_p);
+        dfree(ctx, table);
         return cuda_fail(ctx, e, (std::string("grid build: ") + stage).c_str());
     }
     // free scratch in stream order (caching allocators) or after the work (cudaFree syncs)
     dfree(ctx, w);
-    if (set->d_pockets) dfree(ctx, set->d_pockets);
+    dfree(ctx, set->table);
+    set->table = table;
     set->d_pockets = d_p;
     return PV_OK;
 }
@@ -442,7 +453,7 @@ extern "C" void pv_grid_set_destroy(pv_grid_set* set) {
     if (ctx && ctx->magic == kCtxMagic) {
         DeviceGuard g(ctx->device);
         for (void* a : set->arenas) dfree(ctx, a);
-        dfree(ctx, set->d_pockets);
+        dfree(ctx, set->table);
         for (auto& ev : set->map_events) {
             cudaEventDestroy(ev.first);
             cudaEventDestroy(ev.second);
@@ -475,29 +486,34 @@ extern "C" pv_status pv_grid_set_pack(pv_context* ctx, pv_grid_set* set) {
     const int np = (int)set->pockets.size();
     size_t cells = 0;
     for (const PvPocket& P : set->pockets) cells += (size_t)P.ncells * set->n_maps;
-    float4* carena = (float4*)dalloc(ctx, cells * 2 * sizeof(float4));
-    if (!carena) return fail(ctx, PV_ERR_OOM, "packed map allocation failed");
+    Layout K;
+    const size_t o_cells = K.take<float4>(2 * cells), o_table = K.take<PvPocket>((size_t)np <= kTableInline ? np : 0);
+    char* kept = (char*)dalloc(ctx, K.off);
+    if (!kept) return fail(ctx, PV_ERR_OOM, "packed map allocation failed");
+    float4* carena = (float4*)(kept + o_cells);
     std::vector<PvPocket> pk = set->pockets;
     size_t co = 0;
     for (PvPocket& P : pk) {
         P.cells = carena + co;
         co += (size_t)P.ncells * set->n_maps * 2;
     }
-    PvPocket* d_p = (PvPocket*)dalloc(ctx, sizeof(PvPocket) * np);
-    if (!d_p) {
-        dfree(ctx, carena);
+    void* table = nullptr;
+    if ((size_t)np > kTableInline && !(table = dalloc(ctx, sizeof(PvPocket) * np))) {
+        dfree(ctx, kept);
         return fail(ctx, PV_ERR_OOM, "pocket table allocation failed");
     }
+    PvPocket* d_p = table ? (PvPocket*)table : (PvPocket*)(kept + o_table);
     cudaError_t e = cudaMemcpyAsync(d_p, pk.data(), sizeof(PvPocket) * np, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = launch_pack_cells(d_p, pk.data(), 0, np, set->n_maps, ctx->stream);
     if (e != cudaSuccess) {
-        dfree(ctx, d_p);
-        dfree(ctx, carena);
+        dfree(ctx, table);
+        dfree(ctx, kept);
         return cuda_fail(ctx, e, "map packing");
     }
-    set->arenas.push_back(carena);
+    set->arenas.push_back(kept);
     set->bytes += (int64_t)(cells * 2 * sizeof(float4));
-    dfree(ctx, set->d_pockets);
+    dfree(ctx, set->table);
+    set->table = table;
     set->d_pockets = d_p;
     set->pockets = pk;
     set->packed = true;

@@ -184,8 +184,11 @@ cudaError_t launch_receptor_prep(const float* xyz, const uint8_t* el, const uint
     while (buckets < n) buckets <<= 1;
     int* polar_head = reinterpret_cast<int*>(sorted);
     int* polar_next = polar_head + buckets;
-    cudaError_t e = cudaMemsetAsync(head, 0, sizeof(int) * n_cells, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(polar_head, 0, sizeof(int) * buckets, s);
+    // cleared together when one follows the other (but for padding)
+    const ptrdiff_t gap = reinterpret_cast<char*>(polar_head) - reinterpret_cast<char*>(head + n_cells);
+    const bool joined = gap >= 0 && gap <= 256;
+    cudaError_t e = cudaMemsetAsync(head, 0, sizeof(int) * n_cells + (joined ? gap + sizeof(int) * buckets : 0), s);
+    if (e == cudaSuccess && !joined) e = cudaMemsetAsync(polar_head, 0, sizeof(int) * buckets, s);
     if (e != cudaSuccess) return e;
     int* cursor = cell_start + n_cells;
     receptor_link_kernel<<<(n + 127) / 128, 128, 0, s>>>(xyz, el, n, G, (unsigned)buckets - 1u, cell_of, head, next,

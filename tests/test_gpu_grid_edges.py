@@ -93,3 +93,36 @@ def test_packed_cells_of_ragged_boxes_hold_the_plain_corners(shift):
         x = torch.tensor(at, device="cuda")
         for a, b in zip(ctx.score(plain, lig, p, x)[:2], ctx.score(packed, lig, p, x)[:2]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n_atoms,packed", [(40, False), (4400, True), (9000, False)])
+def test_appended_pockets_past_an_inline_table(n_atoms, packed):
+    """Appends that take a set from 1 over 63, 64 and 65 to 67 pockets, where its pocket table moves out of
+    the maps' memory, with receptors that go up in one piece and in several: maps and lookups in the packed
+    cells have the bits of a set built from the appended boxes alone."""
+    import torch
+    ctx = G.context()
+    rec = _receptor(n_atoms, 0.3, 12)
+    lig = ctx.ligand(S.Ligand(np.zeros((1, 3)), np.zeros(1, np.uint8), np.zeros(1, np.uint8), np.zeros(1, np.uint8),
+                              np.zeros((0, 2), np.int32), np.zeros(0, np.uint8)))
+    boxes = [_box((0.4 * i - 12, 1, 0), (2.6, 3.0 + 0.1 * (i % 5), 2.2)) for i in range(67)]
+    parts = [(0, 1), (1, 63), (63, 64), (64, 65), (65, 67)]
+    gs = ctx.build_grids(rec, boxes[:1], [0, 9])
+    if packed:
+        gs.pack()
+    for lo, hi in parts[1:]:
+        assert gs.append(rec, boxes[lo:hi]) == lo
+    if not packed:
+        gs.pack()
+    at = np.zeros((500, 7), np.float32)
+    at[:, 3] = 1.0
+    rng = np.random.default_rng(13)
+    for lo, hi in parts:
+        alone = ctx.build_grids(rec, boxes[lo:hi], [0, 9]).pack()
+        for p in {lo, hi - 1}:
+            for t in (0, 9):
+                np.testing.assert_array_equal(gs.read_map(p, t), alone.read_map(p - lo, t))
+            at[:, :3] = np.asarray(boxes[p].center) + (rng.random((500, 3)) - 0.5) * 3
+            x = torch.tensor(at, device="cuda")
+            for a, b in zip(ctx.score(gs, lig, p, x)[:2], ctx.score(alone, lig, p - lo, x)[:2]):
+                assert torch.equal(a, b)

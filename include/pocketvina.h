@@ -394,7 +394,9 @@ pv_status pv_dock_result_timing(const pv_dock_result* r, double* search_seconds,
 pv_status pv_dock_result_map_layout(const pv_dock_result* r, int32_t* map_layout);
 
 /* Launch shape the batched search used (after autotuning): register variant and warps per CTA (at most
- * the number that warps_per_cta accepts for the variant; with warps_per_cta 0 a CTA may run more). */
+ * the number that warps_per_cta accepts for the variant; with warps_per_cta 0 a CTA may run more). A dock
+ * of few chains (up to two per SM, ligands on whole warps, shape left free) runs in a kernel of its own and is not
+ * autotuned: it reports variant 0, whose results are the same bits. */
 pv_status pv_dock_result_launch(const pv_dock_result* r, int32_t* search_variant, int32_t* warps_per_cta);
 
 /* Device-resident results (valid until destroy): poses [n_pairs * top_k] pv_pose,

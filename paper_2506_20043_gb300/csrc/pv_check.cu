@@ -46,7 +46,7 @@ struct WarpAnalytic {
     using State = float;
     int kind, n;
     float a;                       // the lane's coefficient (quadratic)
-    __device__ __forceinline__ float eval(const float& x, float& g) const {
+    __device__ __forceinline__ float eval(const float& x, float& g, bool) const {
         const int k = threadIdx.x & 31;
         const float xn = __shfl_down_sync(PV_FULL, x, 1), xp = __shfl_up_sync(PV_FULL, x, 1);
         return Team<32>::sum(analytic_term(kind, n, k, xp, x, xn, a, g));

@@ -116,6 +116,10 @@ cudaError_t search_max_ctas_per_sm(int variant, bool focc, int layout, int warps
 const void* search_focc_kernel(int variant);
 const void* search_packed_kernel(int variant);
 const void* search_focc_packed_kernel(int variant);
+constexpr int kSearchFew = kSearchVariants;    // index of the kernel for few chains beside the variants
+constexpr int kFewWarps = 8;                   // warps of one chain there
+bool search_few_fits(bool focc, int layout, int lig_bytes, int n, int sms);
+cudaError_t launch_search_few(const SearchArgs& a, int n, cudaStream_t s);
 cudaError_t launch_search_round(const SearchArgs& a, int variant, int grid, int warps, cudaStream_t s);
 cudaError_t launch_plain_search(const SearchArgs& a, int pair, const PvLigBlob* lig_dev,
                                 cudaStream_t s);

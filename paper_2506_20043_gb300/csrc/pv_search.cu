@@ -37,6 +37,8 @@ int search_smem_bytes(int lig_bytes, int warps, int lanes, int lig_slots) {
     return lig_slots * lig + warps * ((int)sizeof(PvPocket) + (32 / lanes) * (int)sizeof(WarpScratch));
 }
 
+static int search_few_smem(int lig_bytes) { return search_smem_bytes(lig_bytes, 0, 32, 1) + kFewWarps * (int)sizeof(WarpScratch); }
+
 struct VariantEntry {
     const void* fn;
     int max_threads;       // per CTA when the caller fixes the CTA size
@@ -53,12 +55,13 @@ static const VariantEntry kVariants[kSearchVariants] = {
     {(const void*)search_round_kernel<768, 16, false, 0>, 128, 768, 16},
     {(const void*)search_round_kernel<1024, 16, false, 0>, 128, 1024, 16},
 };
-static int g_variant_smem[4][kSearchVariants][64];
+static int g_variant_smem[4][kSearchVariants + 1][64];
 
 // The kernel of a variant, with or without the consistency check, for a map layout.
 static const void* variant_fn(int variant, bool focc, int layout) {
     if (layout == 1) return focc ? search_focc_packed_kernel(variant) : search_packed_kernel(variant);
-    return focc ? search_focc_kernel(variant) : kVariants[variant].fn;
+    if (focc) return search_focc_kernel(variant);
+    return variant == kSearchFew ? (const void*)search_few_kernel<false, 0> : kVariants[variant].fn;
 }
 
 int search_variant_max_warps(int variant) {
@@ -98,6 +101,26 @@ cudaError_t launch_search_round(const SearchArgs& a, int variant, int grid, int 
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&a};
     return cudaLaunchKernel(fn, dim3(grid), dim3(warps * 32), args, (size_t)smem, s);
+}
+
+// The launch of few chains: whether n of them run at once, and the launch of one round.
+bool search_few_fits(bool focc, int layout, int lig_bytes, int n, int sms) {
+    int occ = 0;
+    const void* fn = variant_fn(kSearchFew, focc, layout);
+    const int smem = search_few_smem(lig_bytes);
+    if (ensure_smem(fn, smem, g_variant_smem[2 * layout + (focc ? 1 : 0)][kSearchFew]) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 32 * kFewWarps, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n <= (long long)sms * occ;
+}
+cudaError_t launch_search_few(const SearchArgs& a, int n, cudaStream_t s) {
+    const bool focc = a.C.focc > 0;
+    if ((focc && !a.ring) || (a.layout != 0 && a.layout != 1)) return cudaErrorInvalidValue;
+    void* args[] = {(void*)&a};
+    return cudaLaunchKernel(variant_fn(kSearchFew, focc, a.layout), dim3(n), dim3(32 * kFewWarps), args,
+                            (size_t)search_few_smem(a.lig_smem_bytes), s);
 }
 
 // Plain form: the chains of one pair, one thread per chain, all steps in one launch.

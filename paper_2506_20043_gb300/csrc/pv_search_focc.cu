@@ -12,6 +12,7 @@ const void* search_focc_kernel(int variant) {
         (const void*)search_round_kernel<512, 16, true, 0>, (const void*)search_round_kernel<640, 16, true, 0>,
         (const void*)search_round_kernel<768, 16, true, 0>, (const void*)search_round_kernel<1024, 16, true, 0>,
     };
+    if (variant == kSearchFew) return (const void*)search_few_kernel<true, 0>;
     return variant >= 0 && variant < kSearchVariants ? kFns[variant] : nullptr;
 }
 

@@ -11,6 +11,7 @@ const void* search_focc_packed_kernel(int variant) {
         (const void*)search_round_kernel<512, 16, true, 1>, (const void*)search_round_kernel<640, 16, true, 1>,
         (const void*)search_round_kernel<768, 16, true, 1>, (const void*)search_round_kernel<1024, 16, true, 1>,
     };
+    if (variant == kSearchFew) return (const void*)search_few_kernel<true, 1>;
     return variant >= 0 && variant < kSearchVariants ? kFns[variant] : nullptr;
 }
 

@@ -12,6 +12,7 @@ const void* search_packed_kernel(int variant) {
         (const void*)search_round_kernel<512, 16, false, 1>, (const void*)search_round_kernel<640, 16, false, 1>,
         (const void*)search_round_kernel<768, 16, false, 1>, (const void*)search_round_kernel<1024, 16, false, 1>,
     };
+    if (variant == kSearchFew) return (const void*)search_few_kernel<false, 1>;
     return variant >= 0 && variant < kSearchVariants ? kFns[variant] : nullptr;
 }
 

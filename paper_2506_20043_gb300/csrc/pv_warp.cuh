@@ -419,7 +419,9 @@ __device__ __forceinline__ float team_eval(const PvLigBlob& L, WarpScratch& S, c
             for (int a = a0 + sub; a < a1; a += k) t = t + cross3(f3(S.x[a]) - xa_f, f3(S.g[a]));
         }
         for (int o = 1; o < k; o <<= 1) t = t + Tm::xor3(t, o);
-        const float gpsi = dot3(ax_f, t);
+        // written out: the compiler orders the three terms of dot3 in its own way here from kernel to kernel, and
+        // an evaluation has the same bits in all of them
+        const float gpsi = __fmaf_rn(ax_f.z, t.z, __fmaf_rn(ax_f.x, t.x, __fmul_rn(ax_f.y, t.y)));
         const int nt = 6 + L.h.n_rot;
         const int src = (tl >= 6 && tl < nt) ? L.tor_frag[tl - 6] * k : tl;
         float gp = Tm::shfl(gpsi, src);

@@ -175,7 +175,7 @@ def stored_grid_profile():
 def stored_profile():
     """Figures of the committed ncu summary of the search kernel, if it was taken on the current
     kernel sources (else {}): 'traffic' = DRAM bytes (read + write) of one launch of the bench's
-    shape (16 step blocks, each sweeping the pockets' maps once; captured at 400 steps, which
+    shape (32 step blocks, each sweeping the pockets' maps once; captured at 400 steps, which
     makes the same sweeps), 'inst' = warp instructions per evaluation."""
     p = os.path.join(ROOT, "profiles", "search_round_kernel_multipocket.md")
     if not os.path.exists(p):
@@ -364,9 +364,9 @@ def run_ours(args):
                               "frac": round(terms * GRID_FLOPS_PER_TERM / map_s / 1e12 / peak_tflops, 4),
                               "term_evals_per_s": round(terms / map_s, 1), "launch_ms": round(map_s * 1e3, 3),
                               "traffic": (round(stored_grid_profile()) if stored_grid_profile() else None)},
-            # per step: typing, 4 binning launches and the map build; one cell-packing launch per
-            # pocket; the start stamp, the search rounds, top-k and merge
-            "gpu_launches": args.steps * (6 + len(my_boxes) + 1 + n_rounds + 2),
+            # per step: three typing and binning launches, the map build and the cell packing; the start stamp,
+            # the search rounds, top-k and merge
+            "gpu_launches": args.steps * (5 + 1 + n_rounds + 2),
             "clocks": clocks,
         }
         if not args.no_plain:

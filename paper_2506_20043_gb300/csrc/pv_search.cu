@@ -4,7 +4,8 @@
 // Batched form: one persistent launch per round of MC steps covers every (ligand, pocket,
 // chain-block) work item; CTAs pull items from an atomic counter, stage the item's ligand tree
 // in shared memory, and their warps take its chains one by one (pv_chain.cuh; the variants with the
-// consistency check of Eq. 4-5 are compiled in pv_search_focc.cu). Plain form (comparison path, the paper's
+// consistency check of Eq. 4-5 are compiled in pv_search_focc.cu); a launch of few chains has a CTA for each
+// instead (search_few_kernel). Plain form (comparison path, the paper's
 // organisation): one launch per pair, one thread per chain, see pv_thread.cuh.
 #include "pv_chain.cuh"
 #include "pv_thread.cuh"

@@ -472,7 +472,7 @@ __device__ __forceinline__ float warp_min(float v) {
 // measured best, 36 us for 8,000 atoms with 7 columns and 63 us with 20 (event-timed), against 42 and 89 us
 // for 16 warps by the 2 CTAs that 59 registers allow, 40 and 69 us for 8 warps by 4.
 __global__ void __launch_bounds__(kFeatSplit * 32, 3) feature_kernel(FeatArgs g) {
-    __shared__ float s_at[kFeatSplit][3][32];                 // a chunk's atoms, read two at a time
+    __shared__ __align__(16) float s_at[kFeatSplit][3][32];   // a chunk's atoms, read two at a time
     __shared__ float4 s_pr[kFeatSplit][32][kPropChunk / 4];   // an atom's chunk: two broadcast loads
     __shared__ float s_red[kFeatSplit][kPropChunk + 1][32];
     __shared__ int s_beg[kFeatRows];                          // first atom of a listed row

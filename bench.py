@@ -114,7 +114,7 @@ def workload(seed: int):
 
 # Sources of what the multi-pocket bench launches (grid build, search, top-k, merge) and of the
 # host code that shapes those launches; the stored profiles are valid while these are unchanged.
-DOCK_SOURCES = ("pv_api.cu", "pv_chain.cuh", "pv_device.cuh", "pv_grid.cu", "pv_internal.h",
+DOCK_SOURCES = ("pv_api.cu", "pv_chain.cuh", "pv_device.cuh", "pv_grid.cu", "pv_handout.cuh", "pv_internal.h",
                 "pv_layout.h", "pv_ligand.cpp", "pv_ligand.h", "pv_search.cu", "pv_search_packed.cu",
                 "pv_stage.cuh", "pv_terms.h", "pv_thread.cuh", "pv_warp.cuh")
 

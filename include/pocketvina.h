@@ -293,7 +293,9 @@ typedef struct {
     double block_wait_s;       /* batched: bound on a step block's wait for the previous block of
                                   its chains (in practice it never waits); a block that runs out
                                   is skipped with the chains' later blocks, and the dock returns
-                                  PV_ERR_STATE. <= 0: 30 s */
+                                  PV_ERR_STATE. A warp that finds no room for its next ligand
+                                  beside those being worked on waits as long, then leaves its
+                                  work to the others (the results are the same). <= 0: 30 s */
     const int32_t* pair_keys;  /* NULL, or one host int32 per pair as the call lists them (pv_dock:
                                   ligand * n_pockets + position in pocket_ids; pv_dock_pairs: the
                                   position in its list; both before any max_pockets cut): the

@@ -1043,7 +1043,7 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
     std::vector<const void*> ligptr(n_ligs);
     for (int i = 0; i < n_ligs; ++i) ligptr[i] = ligs[i]->d_blob;
     // one launch (round) covers all MC steps unless steps_per_round asks for more; its steps are cut into
-    // chained step blocks (see block_steps below)
+    // chained step blocks (step_block)
     const int S_r = p.steps_per_round > 0 ? p.steps_per_round : std::max(1, steps_left);
     const int n_rounds = steps_left > 0 ? (steps_left + S_r - 1) / S_r : 1;
     // one workspace allocation
@@ -1286,12 +1286,7 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
     }
     apply(A, variant, layout, shape);
     const int W = shape.warps, grid = shape.grid, occ = shape.occ;
-    // Step blocks: when every unit runs at once there is nothing to hand over, and a warp keeps its chains
-    // to the end (blocks would make the fast chains wait for the slow ones' hand-outs); else blocks of about
-    // 1/32 of the steps, so that the last ones spread over the SMs. A caller who fixes the CTA size gets
-    // blocks of about 1/16 (at least 25 steps).
-    const int block_steps = p.warps_per_cta > 0 ? std::max(25, (S_r + 15) / 16)
-                            : shape.all_resident ? S_r : std::max(8, (S_r + 31) / 32);
+    const int block_steps = step_block(S_r, p.warps_per_cta > 0, shape.all_resident, A.items_per_block);
     A.block_steps = block_steps;
     // each pair's position in the order, for the per-pair launches
     std::vector<int> position(n_pairs, 0);

@@ -30,10 +30,10 @@ struct WarpWork {
 // Takes the next unit for a warp. Chains of the CTA's current item are handed out one
 // by one; when it is used up the next item comes from the queue, into a ligand slot that holds its
 // ligand or that no warp works on. A warp holds no slot while it waits for one, and slots are given back when
-// their chains end, so the wait ends; a warp that waited kSlotWaitNs retires, and the warps whose chains hold
-// the slots take the waiting item when they are done.
+// their chains end, so the wait ends. It is bounded by the launch's wait_ns all the same; a warp that waited that
+// long retires for the rest of the launch, and the warps whose chains hold the slots take the waiting item when
+// they are done. A shorter bound of its own (it was 2 s) took warps out of launches whose step blocks ran longer.
 constexpr int kLockSpins = 1 << 22;                        // over 0.1 s
-constexpr unsigned long long kSlotWaitNs = 2000000000ull;
 constexpr unsigned long long kStageWaitNs = 1000000000ull; // a staging takes microseconds
 __device__ __forceinline__ WarpWork take_work(const SearchArgs& A, CtaWork& shared) {
     volatile CtaWork& W = shared;
@@ -125,7 +125,7 @@ __device__ __forceinline__ WarpWork take_work(const SearchArgs& A, CtaWork& shar
         if (!starved) return w;
         const unsigned long long now = warp_time();
         if (t0 == 0ull) t0 = now;
-        if (now - t0 >= kSlotWaitNs) return w;              // the warps that hold the slots go on with it
+        if (now - t0 >= A.wait_ns) return w;                // the warps that hold the slots go on with it
         __nanosleep(1000);
     }
 }

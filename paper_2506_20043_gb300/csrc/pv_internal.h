@@ -95,12 +95,27 @@ struct SearchArgs {
     int lig_smem_bytes;            // staging capacity for one ligand
     const unsigned long long* t0;  // start time of the dock (globaltimer)
     unsigned long long timeout_ns; // 0 = none
-    unsigned long long wait_ns;    // batched: bound on a step block's wait for its predecessor
+    unsigned long long wait_ns;    // batched: bound on a step block's wait for its predecessor, and on a warp's for a
+                                   // ligand slot
     int* err;
     unsigned long long* evals;
     int layout;                    // map layout the kernel reads: 0 plain, 1 cell-packed
 };
 constexpr int kLigSlots = 4;
+// MC steps of a step block, of the `steps` of a launch. When every unit of work runs at once there is nothing to hand
+// over, and a warp keeps its chains to the end (blocks would make the fast chains wait for the slow ones'
+// hand-outs); else blocks of about 1/32 of the steps, so that the last ones spread over the SMs. A caller who fixes
+// the CTA size gets blocks of about 1/16 (at least 25 steps). No block that is handed over is longer than
+// kMaxBlockSteps (a second of a large ligand's chain on a full GPU): warps that wait for a chain's block, or for
+// a ligand slot that its warp holds, would wait as long. Longer again where the items would not fit an int.
+constexpr int kMaxBlockSteps = 512;
+inline int step_block(int steps, bool fixed_cta, bool all_resident, int items_per_block) {
+    if (all_resident && !fixed_cta) return steps;
+    const int part = fixed_cta ? (steps > 400 ? (steps - 1) / 16 + 1 : 25) : (steps > 256 ? (steps - 1) / 32 + 1 : 8);
+    const long long least = ((long long)steps * items_per_block >> 30) + 1;
+    const int block = part < kMaxBlockSteps ? part : kMaxBlockSteps;
+    return least > block ? (int)least : block;
+}
 int search_smem_bytes(int lig_bytes, int warps, int lanes, int lig_slots);
 // Variants of the round kernel: 0-3 run a chain per warp, 4-7 a chain per half warp (ligands of
 // at most 32 atoms and 10 torsions); within each group the launch bounds are 512, 640, 768 and 896

@@ -198,3 +198,41 @@ extern "C" void handout_job(int warps, int n_ligs, int blocks, int units, int it
     out[3] = wrong;
     out[4] = J.err;
 }
+
+// Warp 0 works for busy_ns (by the emulated clock) on the one ligand slot while warp 1 waits for it with another
+// ligand, of two units of two ligands. out = units that warp 1 took, units taken, error bits.
+extern "C" void handout_starved(unsigned long long busy_ns, unsigned long long wait_ns, int* out) {
+    Job J(2, 1, 1, 1, 1, wait_ns);
+    emu::clock_ns = 1000;
+    std::atomic<int> taken[2] = {{0}, {0}};
+    std::atomic<bool> held{false};
+    run_warps(2, [&](int warp, int lane) {
+        if (warp == 1 && lane == 0)
+            while (!held) std::this_thread::yield();
+        emu::warp->meet();
+        for (;;) {
+            const pv::WarpWork w = pv::take_work(J.A, J.W);
+            if (w.status == 0) return;
+            if (lane == 0) {
+                ++taken[warp];
+                if (warp == 0 && !held) {
+                    held = true;
+                    while (__atomic_load_n(&J.W.pending, __ATOMIC_SEQ_CST) < 0) std::this_thread::yield();
+                    for (int i = 0; i < 50; ++i) {         // the clock runs on while warp 1 looks at it
+                        emu::clock_ns += busy_ns / 50;
+                        std::this_thread::sleep_for(std::chrono::milliseconds(10));
+                    }
+                }
+                atomicSub(&J.W.refs[w.slot], 1);
+            }
+            emu::warp->meet();
+        }
+    });
+    out[0] = taken[1];
+    out[1] = taken[0] + taken[1];
+    out[2] = J.err;
+}
+
+extern "C" int handout_step_block(int steps, int fixed_cta, int all_resident, int items_per_block) {
+    return pv::step_block(steps, fixed_cta, all_resident, items_per_block);
+}

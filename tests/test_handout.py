@@ -20,6 +20,7 @@ def lib(tmp_path_factory):
     subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-pthread", "-w", "-I", CSRC, "-I", cuda_inc,
                            os.path.join(ROOT, "tests", "csrc", "handout.cpp"), "-ldl", "-o", out])
     L = C.CDLL(out)
+    L.handout_starved.argtypes = [C.c_ulonglong, C.c_ulonglong, C.c_void_p]
     return L
 
 
@@ -31,3 +32,27 @@ def test_units_are_handed_out_once_and_lanes_agree(lib, warps, n_ligs, blocks, u
     once, total, split, wrong, err = out.tolist()
     assert (split, wrong, err) == (0, 0, 0)
     assert once == total == blocks * n_ligs * units
+
+
+@pytest.mark.parametrize("busy_s, wait_s, by_the_waiting_warp", [(20, 30, 1), (1, 30, 1), (20, 5, 0)])
+def test_a_warp_waits_for_a_slot_as_long_as_the_launch_allows(lib, busy_s, wait_s, by_the_waiting_warp):
+    """A slot held for 20 s does not cost the CTA the warp that waits for it unless the launch's bound is shorter;
+    either way every unit is done."""
+    out = np.zeros(3, np.int32)
+    lib.handout_starved(busy_s * 10 ** 9, wait_s * 10 ** 9, out.ctypes.data_as(C.c_void_p))
+    assert out.tolist() == [by_the_waiting_warp, 2, 0]
+
+
+def test_step_blocks_are_short_and_few_enough(lib):
+    block = lib.handout_step_block
+    for steps in (1, 7, 8, 100, 256, 257, 1000, 2000, 16384):       # 1/32 of the steps, at least 8
+        assert block(steps, 0, 0, 1000) == max(8, -(-steps // 32))
+    for steps in (1, 25, 400, 401, 2000, 8192):                      # a fixed CTA: 1/16, at least 25
+        assert block(steps, 1, 0, 1000) == block(steps, 1, 1, 1000) == max(25, -(-steps // 16))
+    for steps in (20000, 1000000, 2 ** 31 - 1):                      # never longer than 512 where blocks are handed over
+        for items in (1, 64, 40000, 10 ** 6):
+            for fixed in (0, 1):
+                b = block(steps, fixed, 0, items)
+                assert 0 < -(-steps // b) * items < 2 ** 31 - 10 ** 6
+                assert b <= 512 or -(-steps // 512) * items > 2 ** 30 - items
+        assert block(steps, 0, 1, 64) == steps                       # every chain resident: one block

@@ -118,6 +118,8 @@ class Context:
         self.lib = A.load()
         self.device = int(device)
         self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
+        if not isinstance(self.stream, torch.cuda.Stream):     # anything else that holds a CUDA stream's handle
+            self.stream = torch.cuda.ExternalStream(self.stream.cuda_stream, self.device)
         h = C.c_void_p()
         st = self.lib.pv_context_create(self.device, C.c_void_p(self.stream.cuda_stream), C.byref(h))
         if st != A.PV_OK:
@@ -623,10 +625,33 @@ class DockResult:
             self.h = None
 
 
-def _scaled(g, ge):
+def _kept(ctx, g):
+    """A gradient that the context's stream writes, kept for the backward pass: it may be dropped before that stream
+    has got to it."""
+    if ctx.stream != ctx.torch.cuda.current_stream(ctx.device):
+        g.record_stream(ctx.stream)
+    return g
+
+
+def _scaled(ctx, g, ge, dtype):
     """Rows of g times the incoming gradient ge [n] (whatever shape the rows were given in), a constant to
-    further differentiation."""
-    return g * (ge.detach() if ge.requires_grad else ge).view((-1,) + (1,) * (g.dim() - 1))
+    further differentiation. On the context's stream, which wrote g and where the result is waited for by a caller
+    who waits for the context; where the backward pass runs on another stream, each waits for the other."""
+    def product():
+        out = g * (ge.detach() if ge.requires_grad else ge).view((-1,) + (1,) * (g.dim() - 1))
+        return out if out.dtype == dtype else out.to(dtype)
+
+    cuda = ctx.torch.cuda
+    here = cuda.current_stream(ctx.device)
+    if ctx.stream == here:
+        return product()
+    ctx.stream.wait_stream(here)
+    with cuda.stream(ctx.stream):
+        out = product()
+    ge.record_stream(ctx.stream)
+    out.record_stream(here)
+    here.wait_stream(ctx.stream)
+    return out
 
 
 class PVScore:
@@ -649,14 +674,14 @@ class PVScore:
                     if not fctx.needs_input_grad[0]:
                         return pv_ctx.score(grids_, lig_, pocket_, pose_t.detach(), grad=False)[0]
                     e, g = pv_ctx.score_value_grad(grids_, lig_, pocket_, pose_t.detach())
-                    fctx.save_for_backward(pose_t, g)
+                    fctx.save_for_backward(pose_t, _kept(pv_ctx, g))
+                    fctx.pv = pv_ctx
                     return e
 
                 @staticmethod
                 def backward(fctx, ge):
                     pose_t, g = fctx.saved_tensors
-                    g = _scaled(g, ge)
-                    return g if g.dtype == pose_t.dtype else g.to(pose_t.dtype), None, None, None, None
+                    return _scaled(fctx.pv, g, ge, pose_t.dtype), None, None, None, None
 
             cls._fn = _F
         return cls._fn.apply(pose, ctx, grids, lig, pocket)
@@ -680,14 +705,14 @@ class PVScoreXYZ:
                     need = fctx.needs_input_grad[0]
                     e, g = pv_ctx.score_xyz(grids_, lig_, pocket_, xyz_t.detach(), grad=need)
                     if need:
-                        fctx.save_for_backward(xyz_t, g)
+                        fctx.save_for_backward(xyz_t, _kept(pv_ctx, g))
+                        fctx.pv = pv_ctx
                     return e
 
                 @staticmethod
                 def backward(fctx, ge):
                     xyz_t, g = fctx.saved_tensors
-                    g = _scaled(g, ge)
-                    return g if g.dtype == xyz_t.dtype else g.to(xyz_t.dtype), None, None, None, None
+                    return _scaled(fctx.pv, g, ge, xyz_t.dtype), None, None, None, None
 
             cls._fn = _F
         return cls._fn.apply(xyz, ctx, grids, lig, pocket)

@@ -658,8 +658,8 @@ class PVScore:
     """torch.autograd.Function over pose parameters: energy = SF(pose) for one ligand in one
     pocket; the gradient is the library's adjoint (the gradient BFGS consumes), mapped to POT
     coordinates (translation, raw quaternion, torsions). An evaluation with the gradient costs little more
-    than one without, so when the pose needs a gradient the forward pass keeps it and the backward
-    scales it, instead of evaluating every pose again."""
+    than one without, so when the pose needs a gradient and the call is recorded the forward pass keeps it and the
+    backward scales it, instead of evaluating every pose again."""
 
     _fn = None
 
@@ -670,8 +670,8 @@ class PVScore:
 
             class _F(torch.autograd.Function):
                 @staticmethod
-                def forward(fctx, pose_t, pv_ctx, grids_, lig_, pocket_):
-                    if not fctx.needs_input_grad[0]:
+                def forward(fctx, pose_t, pv_ctx, grids_, lig_, pocket_, recorded):
+                    if not (recorded and fctx.needs_input_grad[0]):
                         return pv_ctx.score(grids_, lig_, pocket_, pose_t.detach(), grad=False)[0]
                     e, g = pv_ctx.score_value_grad(grids_, lig_, pocket_, pose_t.detach())
                     fctx.save_for_backward(pose_t, _kept(pv_ctx, g))
@@ -681,16 +681,17 @@ class PVScore:
                 @staticmethod
                 def backward(fctx, ge):
                     pose_t, g = fctx.saved_tensors
-                    return _scaled(fctx.pv, g, ge, pose_t.dtype), None, None, None, None
+                    return _scaled(fctx.pv, g, ge, pose_t.dtype), None, None, None, None, None
 
             cls._fn = _F
-        return cls._fn.apply(pose, ctx, grids, lig, pocket)
+        return cls._fn.apply(pose, ctx, grids, lig, pocket, ctx.torch.is_grad_enabled())
 
 
 class PVScoreXYZ:
     """torch.autograd.Function over ligand atom coordinates: energy = SF(xyz) for posed atoms
     [n, n_atoms, 3] of one ligand in one pocket; the gradient is the library's coordinate gradient
-    dSF/dx_i, kept by the forward pass when it is needed and scaled by the incoming gradient."""
+    dSF/dx_i, kept by the forward pass when it is needed and the call is recorded (inside forward, grad mode can no
+    longer be seen), and scaled by the incoming gradient."""
 
     _fn = None
 
@@ -701,8 +702,8 @@ class PVScoreXYZ:
 
             class _F(torch.autograd.Function):
                 @staticmethod
-                def forward(fctx, xyz_t, pv_ctx, grids_, lig_, pocket_):
-                    need = fctx.needs_input_grad[0]
+                def forward(fctx, xyz_t, pv_ctx, grids_, lig_, pocket_, recorded):
+                    need = recorded and fctx.needs_input_grad[0]
                     e, g = pv_ctx.score_xyz(grids_, lig_, pocket_, xyz_t.detach(), grad=need)
                     if need:
                         fctx.save_for_backward(xyz_t, _kept(pv_ctx, g))
@@ -712,10 +713,10 @@ class PVScoreXYZ:
                 @staticmethod
                 def backward(fctx, ge):
                     xyz_t, g = fctx.saved_tensors
-                    return _scaled(fctx.pv, g, ge, xyz_t.dtype), None, None, None, None
+                    return _scaled(fctx.pv, g, ge, xyz_t.dtype), None, None, None, None, None
 
             cls._fn = _F
-        return cls._fn.apply(xyz, ctx, grids, lig, pocket)
+        return cls._fn.apply(xyz, ctx, grids, lig, pocket, ctx.torch.is_grad_enabled())
 
 
 class Surface:

@@ -3,6 +3,7 @@
 #include <algorithm>
 
 #include "pv_internal.h"
+#include "pv_smem.h"
 #include "pv_stage.cuh"
 #include "pv_warp.cuh"
 
@@ -115,23 +116,16 @@ __global__ void __launch_bounds__(kScoreWarps * 32, 1) score_kernel(ScoreArgs A)
 struct ScoreShape {
     int warps, grid, smem;
 };
-static cudaError_t score_shape(int n, int lig_bytes, ScoreShape& s) {
-    static int sms[64], smem_max[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidValue;
-    if (!sms[dev]) {
-        int v = 0;
-        e = cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        if (e != cudaSuccess) return e;
-        smem_max[dev] = v;
-        e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        sms[dev] = v;
-    }
-    const int lig = (lig_bytes + 127) & ~127, n_sm = sms[dev];
-    const int most = std::min(kScoreWarps, (smem_max[dev] - 1024 - lig) / (int)sizeof(WarpScratch));
+static cudaError_t score_shape(int dev, int n, int lig_bytes, ScoreShape& s) {
+    static DevicePair properties;
+    int n_sm = 0, smem_max = 0;
+    const int e = properties.get(dev, n_sm, smem_max, [dev](int& sms, int& smem) {
+        const cudaError_t x = cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        return (int)(x != cudaSuccess ? x : cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    });
+    if (e) return (cudaError_t)e;
+    const int lig = (lig_bytes + 127) & ~127;
+    const int most = std::min(kScoreWarps, (smem_max - 1024 - lig) / (int)sizeof(WarpScratch));
     if (most < 1) return cudaErrorInvalidValue;
     const int rounds = (n + n_sm * most - 1) / (n_sm * most);
     s.warps = std::max(std::min(most, kScoreLeastWarps), (n + n_sm * rounds - 1) / (n_sm * rounds));
@@ -140,26 +134,26 @@ static cudaError_t score_shape(int n, int lig_bytes, ScoreShape& s) {
     return cudaSuccess;
 }
 
-// The kernel's shared-memory limit on the current device, raised when a launch needs more.
-static cudaError_t score_smem(const void* fn, int smem, int* configured) {
+// The shape of a launch on the current device, and the kernel's shared-memory limit raised to it.
+static cudaError_t score_setup(const void* fn, SmemLimit& limit, int n, int lig_bytes, ScoreShape& s) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (smem > configured[dev]) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) configured[dev] = smem;
-    }
-    return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidValue;
+    e = score_shape(dev, n, lig_bytes, s);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)limit.raise(dev, s.smem, [fn](int bytes) {
+        return (int)cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    });
 }
 
 static cudaError_t launch(const ScoreArgs& a, int layout, cudaStream_t s) {
     if (layout < 0 || layout > 1) return cudaErrorInvalidValue;
     if (a.n_poses < 1) return cudaSuccess;
-    static int configured[2][64];
+    static SmemLimit limit[2];
     const void* fn = layout == 1 ? (const void*)score_kernel<1> : (const void*)score_kernel<0>;
     ScoreShape sh;
-    cudaError_t e = score_shape(a.n_poses, a.lig_bytes, sh);
-    if (e == cudaSuccess) e = score_smem(fn, sh.smem, configured[layout]);
+    const cudaError_t e = score_setup(fn, limit[layout], a.n_poses, a.lig_bytes, sh);
     if (e != cudaSuccess) return e;
     if (layout == 1) score_kernel<1><<<sh.grid, sh.warps * 32, sh.smem, s>>>(a);
     else score_kernel<0><<<sh.grid, sh.warps * 32, sh.smem, s>>>(a);
@@ -253,11 +247,10 @@ cudaError_t launch_score_xyz(const PvLigBlob* lig, int lig_bytes, const PvPocket
     a.n_poses = n_poses; a.xyz = xyz; a.grad_energy = grad_energy; a.energy = energy; a.grad_xyz = grad_xyz;
     if (layout < 0 || layout > 1) return cudaErrorInvalidValue;
     if (n_poses < 1) return cudaSuccess;
-    static int configured[2][64];
+    static SmemLimit limit[2];
     const void* fn = layout == 1 ? (const void*)score_xyz_kernel<1> : (const void*)score_xyz_kernel<0>;
     ScoreShape sh;
-    cudaError_t e = score_shape(n_poses, lig_bytes, sh);
-    if (e == cudaSuccess) e = score_smem(fn, sh.smem, configured[layout]);
+    const cudaError_t e = score_setup(fn, limit[layout], n_poses, lig_bytes, sh);
     if (e != cudaSuccess) return e;
     if (layout == 1) score_xyz_kernel<1><<<sh.grid, sh.warps * 32, sh.smem, s>>>(a);
     else score_xyz_kernel<0><<<sh.grid, sh.warps * 32, sh.smem, s>>>(a);

@@ -8,6 +8,7 @@
 // instead (search_few_kernel). Plain form (comparison path, the paper's
 // organisation): one launch per pair, one thread per chain, see pv_thread.cuh.
 #include "pv_chain.cuh"
+#include "pv_smem.h"
 #include "pv_thread.cuh"
 
 namespace pv {
@@ -16,17 +17,16 @@ __global__ void mark_t0_kernel(unsigned long long* t0) { *t0 = globaltimer(); }
 
 // Dynamic shared memory opt-in per kernel and device, raised only when a launch needs more;
 // callers raise it before stream capture so no attribute call happens while capturing.
-static cudaError_t ensure_smem(const void* fn, int smem, int* cache) {
+static cudaError_t ensure_smem(const void* fn, int smem, SmemLimit& limit) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (smem <= cache[dev]) return cudaSuccess;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) cache[dev] = smem;
-    return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    return (cudaError_t)limit.raise(dev, smem, [fn](int bytes) {
+        return (int)cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    });
 }
-static int g_topk_smem[64], g_merge_smem[64];
+static SmemLimit g_topk_smem, g_merge_smem;
 
 cudaError_t launch_mark_t0(unsigned long long* t0, cudaStream_t s) {
     mark_t0_kernel<<<1, 1, 0, s>>>(t0);
@@ -56,7 +56,7 @@ static const VariantEntry kVariants[kSearchVariants] = {
     {(const void*)search_round_kernel<768, 16, false, 0>, 128, 768, 16},
     {(const void*)search_round_kernel<1024, 16, false, 0>, 128, 1024, 16},
 };
-static int g_variant_smem[4][kSearchVariants + 1][64];
+static SmemLimit g_variant_smem[4][kSearchVariants + 1];
 
 // The kernel of a variant, with or without the consistency check, for a map layout.
 static const void* variant_fn(int variant, bool focc, int layout) {

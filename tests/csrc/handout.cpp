@@ -205,14 +205,17 @@ extern "C" void handout_starved(unsigned long long busy_ns, unsigned long long w
     Job J(2, 1, 1, 1, 1, wait_ns);
     emu::clock_ns = 1000;
     std::atomic<int> taken[2] = {{0}, {0}};
-    std::atomic<bool> held{false};
+    std::atomic<bool> held{false}, gone{false};
     run_warps(2, [&](int warp, int lane) {
         if (warp == 1 && lane == 0)
             while (!held) std::this_thread::yield();
         emu::warp->meet();
         for (;;) {
             const pv::WarpWork w = pv::take_work(J.A, J.W);
-            if (w.status == 0) return;
+            if (w.status == 0) {
+                if (warp == 1) gone = true;
+                return;
+            }
             if (lane == 0) {
                 ++taken[warp];
                 if (warp == 0 && !held) {
@@ -224,6 +227,7 @@ extern "C" void handout_starved(unsigned long long busy_ns, unsigned long long w
                     }
                 }
                 atomicSub(&J.W.refs[w.slot], 1);
+                while (warp == 0 && !taken[1] && !gone) std::this_thread::yield();   // warp 1 chooses first
             }
             emu::warp->meet();
         }

@@ -277,7 +277,7 @@ def run_ours(args):
             ev, _, st = r.stats()
             assert (st == 0).all(), st
             s_s, n_l, _ = r.timing()
-            shape = r.launch_shape()
+            variant, launched = r.launch_shape()[0], r.launched()
             layout = r.map_layout()
             search_s += s_s
             launches += n_l
@@ -330,8 +330,7 @@ def run_ours(args):
                                        f"{world} GPUs: {world} ligands x 10 pockets split into equal pocket-major "
                                        "runs of pairs (job-wide pair keys), ranked poses gathered and merged on "
                                        "rank 0 inside the timed step"),
-                       "search_launch": {"variant": shape[0], "warps_per_cta": shape[1], "chains_per_warp": 2 if shape[0] >= 4 else 1,
-                                         "map_layout": "cell-packed" if layout == 1 else "plain"},
+                       "search_launch": search_launch(variant, launched, layout),
                        "focc": args.focc},
             "best_sf_per_pocket": {"mean": round(float(best_sf.mean()), 4), "min": round(float(best_sf.min()), 4)},
             "top_pose": {str(l): list(v[0]) for l, v in sorted(merged.items())} if merged else None,
@@ -370,7 +369,7 @@ def run_ours(args):
             "clocks": clocks,
         }
         if not args.no_plain:
-            out["plain"] = run_plain(ctx, api, gs, lig, list(range(len(my_boxes))), (shape[0], shape[1], layout))
+            out["plain"] = run_plain(ctx, api, gs, lig, list(range(len(my_boxes))), variant, params.warps_per_cta, layout)
             out["batched_vs_plain"] = round(value / world / out["plain"]["thread_per_chain"]["value"], 2)
             out["batched_vs_plain_warp"] = round(value / world / out["plain"]["warp_per_chain"]["value"], 2)
         if not args.no_micro:
@@ -387,16 +386,25 @@ def run_ours(args):
     return out
 
 
-def run_plain(ctx, api, gs, lig, pockets, shape):
+def search_launch(variant, launched, layout):
+    """The search launch that ran, for the config of a bench line."""
+    kernel, warps, ctas = launched
+    return {"kernel": kernel, "variant": variant, "warps_per_cta": warps, "ctas": ctas,
+            "chains_per_warp": 2 if kernel == "search_round_kernel" and variant >= 4 else 1,
+            "map_layout": "cell-packed" if layout == 1 else "plain"}
+
+
+def run_plain(ctx, api, gs, lig, pockets, variant, warps_per_cta, layout):
     """The paper's organisation, one launch per pair and a host loop, on one pocket of the
     workload at its full length (1,000 chains x 2,000 MC steps, not extrapolated), in two forms:
     thread per chain (as in the paper's engine) and warp per chain (the batched path's own chain
-    kernel and launch shape, one launch per pair with all steps in one block, no queue across pairs,
-    no graph), so that the second ratio isolates what batching itself adds."""
+    kernel and variant, its CTAs sized by the same rule for a pair's chains, one launch per pair with all
+    steps in one block, no queue across pairs, no graph), so that the second ratio isolates what
+    batching itself adds."""
     out = {"sample": f"1 pocket x {CHAINS} chains x {STEPS} MC steps, one launch per pair, timed in full"}
     for name, kw in (("thread_per_chain", dict(mode="plain")),
-                     ("warp_per_chain", dict(mode="plain_warp", search_variant=shape[0], warps_per_cta=shape[1],
-                                             map_layout=shape[2]))):
+                     ("warp_per_chain", dict(mode="plain_warp", search_variant=variant, warps_per_cta=warps_per_cta,
+                                             map_layout=layout))):
         r = ctx.dock(gs, [lig], [pockets[0]], chains=CHAINS, steps=STEPS, seed=0, host_copy=False, **kw)
         ev, _, st = r.stats()
         assert (st == 0).all(), st
@@ -647,7 +655,7 @@ def run_batch_workload(args):
             s_s, _, _ = r.timing()
             evals += ev
             search_s += s_s
-            shape = r.launch_shape()
+            variant, launched = r.launch_shape()[0], r.launched()
             layout = r.map_layout()
             map_bytes = gs.bytes
     total_t = float(np.sum(times))
@@ -672,8 +680,7 @@ def run_batch_workload(args):
                        "map_bytes": int(map_bytes), "chains": w.chains, "mc_steps": w.steps,
                        "l2": f"flushed between timed steps ({L2_FLUSH_BYTES >> 20} MiB write)",
                        "inputs": "receptors and ligands resident in HBM; grids rebuilt every step",
-                       "search_launch": {"variant": shape[0], "warps_per_cta": shape[1],
-                                         "map_layout": "cell-packed" if layout == 1 else "plain"},
+                       "search_launch": search_launch(variant, launched, layout),
                        "host_generation_s": round(t_gen, 1)},
             "evals_per_s": round(evals / total_t, 1), "search_s_per_step": round(search_s / args.steps, 3),
             "roofline": {"kernel": "search_round_kernel", "bound": "alu", "achieved": round(achieved, 3),
@@ -922,7 +929,7 @@ def run_small_case(args):
     torch.cuda.synchronize()
     s_s, _, _ = r.timing()
     return {"case": "small", "evals": int(ev), "seconds": round(sec, 4), "search_seconds": round(s_s, 5),
-            "evals_per_s": round(ev / s_s, 1), "launch": r.launch_shape(), "layout": r.map_layout(),
+            "evals_per_s": round(ev / s_s, 1), "launch": r.launched(), "layout": r.map_layout(),
             "status_ok": bool((st == 0).all())}
 
 

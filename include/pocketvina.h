@@ -395,11 +395,19 @@ pv_status pv_dock_result_timing(const pv_dock_result* r, double* search_seconds,
 /* Map layout the search read (0 plain, 1 cell-packed). */
 pv_status pv_dock_result_map_layout(const pv_dock_result* r, int32_t* map_layout);
 
-/* Launch shape the batched search used (after autotuning): register variant and warps per CTA (at most
- * the number that warps_per_cta accepts for the variant; with warps_per_cta 0 a CTA may run more). A dock
- * of few chains (up to two per SM, ligands on whole warps, shape left free) runs in a kernel of its own and is not
- * autotuned: it reports variant 0, whose results are the same bits. */
+/* Register variant the search ran (after autotuning) and a warps_per_cta that another dock accepts with it: the
+ * caller's, or the variant's largest where it was left free (the launch itself may have run other CTAs then,
+ * pv_dock_result_kernel). A dock of few chains (up to two per SM, ligands on whole warps, shape left free) runs in a
+ * kernel of its own and is not autotuned: it reports variant 0, whose results are the same bits. */
 pv_status pv_dock_result_launch(const pv_dock_result* r, int32_t* search_variant, int32_t* warps_per_cta);
+
+/* The launch that ran: the kernel, its warps per CTA and its CTAs (per launch; any pointer may be null). */
+typedef enum {
+    PV_KERNEL_THREAD = 0,      /* a thread per chain (PV_MODE_PLAIN) */
+    PV_KERNEL_ROUND = 1,       /* a chain per warp or half warp, handed out by a queue */
+    PV_KERNEL_FEW = 2          /* few chains: a CTA per chain */
+} pv_search_kernel;
+pv_status pv_dock_result_kernel(const pv_dock_result* r, int32_t* kernel, int32_t* warps_per_cta, int32_t* ctas);
 
 /* Device-resident results (valid until destroy): poses [n_pairs * top_k] pv_pose,
  * n_kept [n_pairs], ranking [n_ligs][max_pairs_per_ligand * top_k] (-1 padded). */

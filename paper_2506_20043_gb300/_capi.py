@@ -102,6 +102,7 @@ SIGNATURES = {
     "pv_dock_result_stats": (i32, [vp, C.POINTER(u64), C.POINTER(C.c_double), pi32]),
     "pv_dock_result_timing": (i32, [vp, C.POINTER(C.c_double), pi32, C.POINTER(C.c_double)]),
     "pv_dock_result_launch": (i32, [vp, pi32, pi32]),
+    "pv_dock_result_kernel": (i32, [vp, pi32, pi32, pi32]),
     "pv_dock_result_map_layout": (i32, [vp, pi32]),
     "pv_dock_result_device": (i32, [vp, C.POINTER(vp), C.POINTER(vp), C.POINTER(vp)]),
     "pv_dock_result_chains": (i32, [vp, C.POINTER(vp), pi32, pi32, pi32, pi32]),

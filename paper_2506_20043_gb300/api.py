@@ -594,10 +594,17 @@ class DockResult:
         return v.value
 
     def launch_shape(self):
-        """(search kernel variant, warps per CTA) used by the batched search."""
+        """(search kernel variant, a warps_per_cta that another dock accepts with it); `launched` says what ran."""
         v, w = C.c_int32(), C.c_int32()
         self.ctx._check(self.ctx.lib.pv_dock_result_launch(self.h, C.byref(v), C.byref(w)), "pv_dock_result_launch")
         return v.value, w.value
+
+    def launched(self):
+        """The launch that ran: (kernel name, warps per CTA, CTAs)."""
+        k, w, n = C.c_int32(), C.c_int32(), C.c_int32()
+        self.ctx._check(self.ctx.lib.pv_dock_result_kernel(self.h, C.byref(k), C.byref(w), C.byref(n)),
+                        "pv_dock_result_kernel")
+        return ("plain_search_kernel", "search_round_kernel", "search_few_kernel")[k.value], w.value, n.value
 
     def chain_records(self):
         """Chain states after the search, copied to the host: (best POT [n_pairs, chains,

@@ -80,7 +80,8 @@ struct pv_dock_result {
     double seconds = 0.0;
     double search_seconds = 0.0;    // the search kernel launches alone (events around them)
     int search_launches = 0;
-    int search_variant = 0, warps_per_cta = 0;   // launch shape used (batched)
+    int search_variant = 0, warps_per_cta = 0;   // a launch shape to ask for, of the variant used
+    int kernel = PV_KERNEL_ROUND, kernel_warps = 0, kernel_ctas = 0;   // the launch that ran
     int map_layout = 0;                          // map layout the search read
     int mode = PV_MODE_BATCHED;
     int steps_done = 0, focc = 0;                // checkpoint: MC steps the chains have run
@@ -1285,7 +1286,8 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
         return e != cudaSuccess ? cuda_fail(ctx, e, "occupancy") : fail(ctx, PV_ERR_ARG, "search kernel does not fit");
     }
     apply(A, variant, layout, shape);
-    const int W = shape.warps, grid = shape.grid, occ = shape.occ;
+    const int W = shape.warps, grid = shape.grid;
+    const int grid_pair = std::max(1, std::min(A.items_per_pair, ctx->sms * shape.occ));   // of a pair's own launch
     const int block_steps = step_block(S_r, p.warps_per_cta > 0, shape.all_resident, A.items_per_block);
     A.block_steps = block_steps;
     // each pair's position in the order, for the per-pair launches
@@ -1293,6 +1295,10 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
     for (int i = 0; i < n_pairs; ++i) position[order[i]] = i;
     R->search_variant = variant;
     R->warps_per_cta = std::min(W, search_variant_max_warps(variant));
+    R->kernel = few_chains ? PV_KERNEL_FEW : warp_chains ? PV_KERNEL_ROUND : PV_KERNEL_THREAD;
+    R->kernel_warps = few_chains ? kFewWarps : warp_chains ? W : kPlainWarps;
+    R->kernel_ctas = few_chains ? (int)n_chains : p.mode == PV_MODE_BATCHED ? grid : p.mode == PV_MODE_PLAIN_WARP ? grid_pair
+                                                : (p.chains + 32 * kPlainWarps - 1) / (32 * kPlainWarps);
     R->map_layout = layout;
     e = prepare_topk(T);
     if (e == cudaSuccess) e = prepare_merge(R->rank_stride);
@@ -1359,7 +1365,7 @@ static pv_status dock_impl(pv_context* ctx, const pv_grid_set* set, pv_ligand* c
                 a.block_steps = std::max(1, steps_left);
                 x = cudaMemsetAsync(ctr + 2, 0, sizeof(int), s);
                 if (x == cudaSuccess)
-                    x = launch_search_round(a, variant, std::max(1, std::min(a.items_per_pair, ctx->sms * occ)), W, s);
+                    x = launch_search_round(a, variant, grid_pair, W, s);
                 TopkArgs t = T;
                 t.pair0 = q;
                 if (x == cudaSuccess) x = launch_topk(t, 1, s);
@@ -1663,5 +1669,13 @@ extern "C" pv_status pv_dock_result_launch(const pv_dock_result* r, int32_t* sea
     if (!r) return PV_ERR_ARG;
     if (search_variant) *search_variant = r->search_variant;
     if (warps_per_cta) *warps_per_cta = r->warps_per_cta;
+    return PV_OK;
+}
+
+extern "C" pv_status pv_dock_result_kernel(const pv_dock_result* r, int32_t* kernel, int32_t* warps_per_cta, int32_t* ctas) {
+    if (!r) return PV_ERR_ARG;
+    if (kernel) *kernel = r->kernel;
+    if (warps_per_cta) *warps_per_cta = r->kernel_warps;
+    if (ctas) *ctas = r->kernel_ctas;
     return PV_OK;
 }

@@ -136,6 +136,7 @@ constexpr int kFewWarps = 8;                   // warps of one chain there
 bool search_few_fits(bool focc, int layout, int lig_bytes, int n, int sms);
 cudaError_t launch_search_few(const SearchArgs& a, int n, cudaStream_t s);
 cudaError_t launch_search_round(const SearchArgs& a, int variant, int grid, int warps, cudaStream_t s);
+constexpr int kPlainWarps = 4;                 // warps per CTA of the thread-per-chain form
 cudaError_t launch_plain_search(const SearchArgs& a, int pair, const PvLigBlob* lig_dev,
                                 cudaStream_t s);
 cudaError_t launch_mark_t0(unsigned long long* t0, cudaStream_t s);

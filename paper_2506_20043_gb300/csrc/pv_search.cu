@@ -125,7 +125,7 @@ cudaError_t launch_search_few(const SearchArgs& a, int n, cudaStream_t s) {
 }
 
 // Plain form: the chains of one pair, one thread per chain, all steps in one launch.
-__global__ void __launch_bounds__(128) plain_search_kernel(SearchArgs A, int pair,
+__global__ void __launch_bounds__(32 * kPlainWarps) plain_search_kernel(SearchArgs A, int pair,
                                                            const PvLigBlob* __restrict__ L) {
     const int chain = blockIdx.x * blockDim.x + threadIdx.x;
     if (chain >= A.C.chains) return;
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(128) plain_search_kernel(SearchArgs A, int pai
 
 cudaError_t launch_plain_search(const SearchArgs& a, int pair, const PvLigBlob* lig_dev,
                                 cudaStream_t s) {
-    const int threads = 128;
+    const int threads = 32 * kPlainWarps;
     const int grid = (a.C.chains + threads - 1) / threads;
     plain_search_kernel<<<grid, threads, 0, s>>>(a, pair, lig_dev);
     return cudaGetLastError();

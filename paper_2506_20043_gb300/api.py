@@ -120,6 +120,8 @@ class Context:
         self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
         if not isinstance(self.stream, torch.cuda.Stream):     # anything else that holds a CUDA stream's handle
             self.stream = torch.cuda.ExternalStream(self.stream.cuda_stream, self.device)
+        self._raw_stream = self.stream.cuda_stream
+        self._current_raw = torch._C._cuda_getCurrentRawStream
         h = C.c_void_p()
         st = self.lib.pv_context_create(self.device, C.c_void_p(self.stream.cuda_stream), C.byref(h))
         if st != A.PV_OK:
@@ -632,32 +634,32 @@ class DockResult:
             self.h = None
 
 
-def _kept(ctx, g):
-    """A gradient that the context's stream writes, kept for the backward pass: it may be dropped before that stream
-    has got to it."""
-    if ctx.stream != ctx.torch.cuda.current_stream(ctx.device):
-        g.record_stream(ctx.stream)
-    return g
+def _side_stream(ctx):
+    """ctx, if its stream, which has just been given the evaluation of a forward pass, is not torch's current one, else
+    None. The current stream then waits for it: hooks on saved tensors read the gradient there, and its memory goes
+    back there. By handle: making and comparing stream objects costs an autograd call 14 us."""
+    if ctx._current_raw(ctx.device) == ctx._raw_stream:
+        return None
+    ctx.torch.cuda.current_stream(ctx.device).wait_stream(ctx.stream)
+    return ctx
 
 
-def _scaled(ctx, g, ge, dtype):
+def _scaled(side, g, ge, dtype):
     """Rows of g times the incoming gradient ge [n] (whatever shape the rows were given in), a constant to
-    further differentiation. On the context's stream, which wrote g and where the result is waited for by a caller
-    who waits for the context; where the backward pass runs on another stream, each waits for the other."""
-    def product():
-        out = g * (ge.detach() if ge.requires_grad else ge).view((-1,) + (1,) * (g.dim() - 1))
+    further differentiation. Where the context's stream is not the current one (side; the backward pass of a node runs
+    on the stream of its forward pass), on the context's, since a caller who waits for the context waits for the
+    gradient too, and each stream waits for the other."""
+    ge = (ge.detach() if ge.requires_grad else ge).view((-1,) + (1,) * (g.dim() - 1))
+    if side is None:
+        out = g * ge
         return out if out.dtype == dtype else out.to(dtype)
-
-    cuda = ctx.torch.cuda
-    here = cuda.current_stream(ctx.device)
-    if ctx.stream == here:
-        return product()
-    ctx.stream.wait_stream(here)
-    with cuda.stream(ctx.stream):
-        out = product()
-    ge.record_stream(ctx.stream)
+    cuda = side.torch.cuda
+    here = cuda.current_stream(side.device)
+    side.stream.wait_stream(here)
+    with cuda.stream(side.stream):
+        out = (g * ge).to(dtype)
     out.record_stream(here)
-    here.wait_stream(ctx.stream)
+    here.wait_stream(side.stream)
     return out
 
 
@@ -681,14 +683,14 @@ class PVScore:
                     if not (recorded and fctx.needs_input_grad[0]):
                         return pv_ctx.score(grids_, lig_, pocket_, pose_t.detach(), grad=False)[0]
                     e, g = pv_ctx.score_value_grad(grids_, lig_, pocket_, pose_t.detach())
-                    fctx.save_for_backward(pose_t, _kept(pv_ctx, g))
-                    fctx.pv = pv_ctx
+                    fctx.save_for_backward(pose_t, g)
+                    fctx.side = _side_stream(pv_ctx)
                     return e
 
                 @staticmethod
                 def backward(fctx, ge):
                     pose_t, g = fctx.saved_tensors
-                    return _scaled(fctx.pv, g, ge, pose_t.dtype), None, None, None, None, None
+                    return _scaled(fctx.side, g, ge, pose_t.dtype), None, None, None, None, None
 
             cls._fn = _F
         return cls._fn.apply(pose, ctx, grids, lig, pocket, ctx.torch.is_grad_enabled())
@@ -713,14 +715,14 @@ class PVScoreXYZ:
                     need = recorded and fctx.needs_input_grad[0]
                     e, g = pv_ctx.score_xyz(grids_, lig_, pocket_, xyz_t.detach(), grad=need)
                     if need:
-                        fctx.save_for_backward(xyz_t, _kept(pv_ctx, g))
-                        fctx.pv = pv_ctx
+                        fctx.save_for_backward(xyz_t, g)
+                        fctx.side = _side_stream(pv_ctx)
                     return e
 
                 @staticmethod
                 def backward(fctx, ge):
                     xyz_t, g = fctx.saved_tensors
-                    return _scaled(fctx.pv, g, ge, xyz_t.dtype), None, None, None, None, None
+                    return _scaled(fctx.side, g, ge, xyz_t.dtype), None, None, None, None, None
 
             cls._fn = _F
         return cls._fn.apply(xyz, ctx, grids, lig, pocket, ctx.torch.is_grad_enabled())

@@ -30,7 +30,7 @@ def site():
 
 
 @pytest.mark.parametrize("which", [0, 1])
-@pytest.mark.parametrize("wait", ["context", "current"])
+@pytest.mark.parametrize("wait", ["context", "current", "saved on the host"])
 def test_gradients_of_a_context_on_a_side_stream(site, which, wait):
     import torch
     from paper_2506_20043_gb300 import api
@@ -45,6 +45,10 @@ def test_gradients_of_a_context_on_a_side_stream(site, which, wait):
     if wait == "context":
         g, = torch.autograd.grad(fn.apply(x, ctx, gs, lig, 0), x, weight)
         side.synchronize()
+    elif wait == "saved on the host":                               # hooks copy the gradient as soon as it is saved
+        with torch.autograd.graph.save_on_cpu():
+            e = fn.apply(x, ctx, gs, lig, 0)
+        g, = torch.autograd.grad(e, x, weight)
     else:
         fn.apply(x * 1.0, ctx, gs, lig, 0).backward(weight)         # a node after it, on the current stream
         g = x.grad

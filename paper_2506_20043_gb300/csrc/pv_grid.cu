@@ -4,6 +4,7 @@
 // stages the receptor atoms of the cells within the cutoff of the tile into shared memory, and
 // every thread accumulates, for two nodes, the Vina energy of each requested ligand XS type.
 #include "pv_internal.h"
+#include "pv_runs.h"
 #include "pv_device.cuh"
 
 namespace pv {
@@ -499,22 +500,15 @@ __global__ void __launch_bounds__(128) pack_cells_kernel(const PvPocket* __restr
 
 cudaError_t launch_pack_cells(const PvPocket* pockets_dev, const PvPocket* pockets_host, int first, int n,
                               int n_maps, cudaStream_t s) {
-    // blockIdx: columns of a map, (map slot, chunk of z), pocket; sized for the largest pocket of the
-    // launch, at most 65,535 pockets each
-    for (int p0 = first; p0 < first + n; p0 += 65535) {
-        const int np = first + n - p0 < 65535 ? first + n - p0 : 65535;
-        int cols = 0, chunks = 0;
-        for (int p = p0; p < p0 + np; ++p) {
-            const int* d = pockets_host[p].dims;
-            const int c = (d[0] - 1) * (d[1] - 1), z = (d[2] - 1 + kPackZ - 1) / kPackZ;
-            cols = c > cols ? c : cols;
-            chunks = z > chunks ? z : chunks;
-        }
-        pack_cells_kernel<<<dim3((cols + 127) / 128, chunks * n_maps, np), 128, 0, s>>>(pockets_dev + p0, chunks);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    // blockIdx: columns of a map, (map slot, chunk of z), pocket
+    auto extent = [&](int p) {
+        const int* d = pockets_host[p].dims;
+        return RunExtent{((d[0] - 1) * (d[1] - 1) + 127) / 128, (long long)((d[2] - 1 + kPackZ - 1) / kPackZ) * n_maps};
+    };
+    return launch_runs(first, n, extent, [&](int p0, int np, RunExtent most) {
+        pack_cells_kernel<<<dim3((unsigned)most.x, (unsigned)most.y, np), 128, 0, s>>>(pockets_dev + p0, (int)most.y / n_maps);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_grid_maps(const float4* sorted, const int* cell_start, const float lo[3], float cell,
@@ -536,21 +530,16 @@ cudaError_t launch_grid_maps(const float4* sorted, const int* cell_start, const 
     const int classes = ((type_mask & 0x400) ? 1 : 0) | ((type_mask & 0x3) ? 2 : 0) | ((type_mask & 0x3c) ? 4 : 0) |
                         ((type_mask & 0x3c0) ? 8 : 0);
     if (!classes) return cudaErrorInvalidValue;
-    // blockIdx.y is the pocket, blockIdx.x its tile; at most 65,535 pockets per launch
-    for (int p0 = 0; p0 < n_pockets; p0 += 65535) {
-        const int np = n_pockets - p0 < 65535 ? n_pockets - p0 : 65535;
-        int most = 0;
-        for (int p = p0; p < p0 + np; ++p) {
-            const int* d = pockets_host[p].dims;
-            const int t = ((d[0] + kTile - 1) / kTile) * ((d[1] + kTile - 1) / kTile) * ((d[2] + kTileZ - 1) / kTileZ);
-            most = t > most ? t : most;
-        }
+    // blockIdx.y is the pocket, blockIdx.x its tile
+    auto extent = [&](int p) {
+        const int* d = pockets_host[p].dims;
+        return RunExtent{(long long)((d[0] + kTile - 1) / kTile) * ((d[1] + kTile - 1) / kTile) * ((d[2] + kTileZ - 1) / kTileZ), 1};
+    };
+    return launch_runs(0, n_pockets, extent, [&](int p0, int np, RunExtent most) {
         a.pockets = pockets_dev + p0;
-        kernels[classes]<<<dim3(most, np), kGridThreads, 0, s>>>(a);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+        kernels[classes]<<<dim3((unsigned)most.x, np), kGridThreads, 0, s>>>(a);
+        return cudaGetLastError();
+    });
 }
 
 }  // namespace pv

@@ -30,8 +30,12 @@
 
 #include "pocketvina.h"
 #include "pv_internal.h"
+#include "pv_runs.h"
 
 namespace {
+
+using pv::launch_runs;
+using pv::RunExtent;
 
 constexpr int kSurfaceMagic = 0x53524631;
 constexpr int kClustersMagic = 0x434c5331;
@@ -1048,8 +1052,6 @@ struct Carve {
     }
 };
 
-constexpr int kMaxGridY = 65535;   // items per launch
-
 // One receptor of a surface call on the host.
 struct SurfaceJob {
     const pv_receptor* r = nullptr;
@@ -1173,11 +1175,9 @@ cudaError_t surface_build(pv_context* ctx, cudaStream_t st, int dev, const pv_po
     const size_t o_status = zero.take<int>(2 * (size_t)k);
     std::vector<size_t> o_count(k), o_head(k), o_atoms(k), o_arad(k), o_key(k), o_next(k), o_order(k), o_kept(k), o_nkept(k),
         o_off(k), o_offs(k);
-    int n_max = 0;
     for (int j = 0; j < k; ++j) {
         const SurfaceJob& J = jobs[j];
         const size_t n = J.n;
-        n_max = std::max(n_max, J.n);
         if (J.r->mem == PV_MEM_HOST) {
             o_xyz[j] = up.put(J.r->xyz, sizeof(float) * 3 * n);
             if (J.r->element && !J.radius) o_el[j] = up.put(J.r->element, n);
@@ -1255,17 +1255,17 @@ cudaError_t surface_build(pv_context* ctx, cudaStream_t st, int dev, const pv_po
     if (e == cudaSuccess) e = cudaMemsetAsync(d_zero, 0, zero.bytes, st);
     if (e != cudaSuccess) return e;
     *stage = "surface points";
-    const unsigned b256 = (n_max + 255) / 256, bw = (n_max + kSasWarps - 1) / kSasWarps;
-    for (int y0 = 0; y0 < k; y0 += kMaxGridY) {
-        const unsigned ny = std::min(kMaxGridY, k - y0);
+    auto extent = [&](int j) { return RunExtent{(jobs[j].n + kSasWarps - 1) / kSasWarps, 1}; };   // a warp per atom
+    e = launch_runs(0, k, extent, [&](int y0, int ny, RunExtent most) {
+        const unsigned bw = (unsigned)most.x, b256 = (bw * kSasWarps + 255) / 256;
         const SurfaceItem* it = d_items + y0;
         prep_atoms_kernel<<<dim3(b256, ny), 256, 0, st>>>(it, p->probe);
         cell_scan_kernel<<<dim3(1, ny), 1024, 0, st>>>(it);
         sort_atoms_kernel<<<dim3(b256, ny), 256, 0, st>>>(it);
         sas_kernel<<<dim3(bw, ny), kSasWarps * 32, 0, st>>>(it, d_dirs, ns);
         point_scan_kernel<<<dim3(2, ny), 1024, 0, st>>>(it);
-    }
-    e = cudaGetLastError();
+        return cudaGetLastError();
+    });
     if (e != cudaSuccess) return e;
     // one readback of all error words and point counts
     *stage = "readback";
@@ -1291,10 +1291,12 @@ cudaError_t surface_build(pv_context* ctx, cudaStream_t st, int dev, const pv_po
     }
     *stage = "point order";
     e = cudaMemcpyAsync(d_items, items.data(), sizeof(SurfaceItem) * k, cudaMemcpyHostToDevice, st);
-    for (int y0 = 0; y0 < k && e == cudaSuccess; y0 += kMaxGridY) {
-        sas_write_kernel<<<dim3((n_max + 3) / 4, std::min(kMaxGridY, k - y0)), 128, 0, st>>>(d_items + y0, d_dirs, ns);
-        e = cudaGetLastError();
-    }
+    if (e != cudaSuccess) return e;
+    e = launch_runs(0, k, extent, [&](int y0, int ny, RunExtent most) {
+        static_assert(kSasWarps == 4, "sas_write_kernel takes four atoms per block");
+        sas_write_kernel<<<dim3((unsigned)most.x, ny), 128, 0, st>>>(d_items + y0, d_dirs, ns);
+        return cudaGetLastError();
+    });
     return e;
 }
 
@@ -1460,7 +1462,6 @@ cudaError_t cluster_build(pv_context* ctx, cudaStream_t st, int dev, int k, cons
     Carve zero, work;        // cleared; written before it is read
     const size_t o_items = work.take<ClusterItem>(k), o_status = zero.take<int>(2 * (size_t)k);
     std::vector<ClusterItem> items(k);
-    int n_max = 0;
     // two passes over the same layout: offsets first, then addresses in the one allocation
     char *d_zero = nullptr, *d_work = nullptr;
     for (int pass = 0; pass < 2; ++pass) {
@@ -1484,7 +1485,6 @@ cudaError_t cluster_build(pv_context* ctx, cudaStream_t st, int dev, int k, cons
             g.n = n_points[j];
             g.n_buckets = (int)buckets;
             g.hmask = buckets - 1;
-            n_max = std::max(n_max, g.n);
             g.count = (int*)(d_zero + zero.take<int>(buckets));
             g.s2 = (double*)(d_zero + zero.take<double>(m));
             g.sx = (double*)(d_zero + zero.take<double>(3 * m));
@@ -1524,9 +1524,9 @@ cudaError_t cluster_build(pv_context* ctx, cudaStream_t st, int dev, int k, cons
     if (e == cudaSuccess) e = cudaMemsetAsync(d_zero, 0, zero.bytes, st);
     if (e != cudaSuccess) return e;
     *stage = "single linkage";
-    const unsigned b = (n_max + 255) / 256, bw = (n_max + 7) / 8;   // bw: a warp per point, 8 points per CTA
-    for (int y0 = 0; y0 < k && n_max > 0; y0 += kMaxGridY) {
-        const unsigned ny = std::min(kMaxGridY, k - y0);
+    // a warp per point in most kernels, 8 points per block
+    e = launch_runs(0, k, [&](int j) { return RunExtent{((long long)n_points[j] + 7) / 8, 1}; }, [&](int y0, int ny, RunExtent most) {
+        const unsigned bw = (unsigned)most.x, b = (bw * 8 + 255) / 256;
         const ClusterItem* it = (const ClusterItem*)(d_work + o_items) + y0;
         cl_init_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
         cl_scan_kernel<<<dim3(1, ny), 1024, 0, st>>>(it);
@@ -1539,9 +1539,9 @@ cudaError_t cluster_build(pv_context* ctx, cudaStream_t st, int dev, int k, cons
         cl_stats_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
         cl_rank_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
         cl_output_kernel<<<dim3(b, ny), 256, 0, st>>>(it);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
+        return cudaGetLastError();
+    });
+    if (e != cudaSuccess) return e;
     // one readback of all error words and cluster counts
     *stage = "readback";
     e = cudaMemcpyAsync(status.data(), d_zero + o_status, sizeof(int) * status.size(), cudaMemcpyDeviceToHost, st);

@@ -503,7 +503,8 @@ pv_status pv_pocket_params_default(pv_pocket_params* p);
 pv_status pv_surface_create(pv_context* ctx, const pv_receptor* receptor, const float* radius,
                             const pv_pocket_params* p, pv_surface** out);
 /* Step 1 for n_receptors receptors at once: the same results as one pv_surface_create per
- * receptor, with one host synchronisation for all of them. radii: NULL, or n_receptors pointers
+ * receptor, with one host synchronisation for all of them, two when some are in device memory (their
+ * bounding boxes are read back first). radii: NULL, or n_receptors pointers
  * (each NULL or per-atom radii in that receptor's memory kind). out receives n_receptors handles,
  * each destroyed on its own; on any error none is returned. */
 pv_status pv_surface_create_many(pv_context* ctx, int32_t n_receptors, const pv_receptor* receptors,

@@ -1,8 +1,9 @@
 // pv_grid.cu -- the grid cache ("Kernel 1", Methods "Accelerated Docking"; Supplementary
 // Algorithm 2, Grid_cache(P)): receptor XS typing, binning of receptor atoms into cubic cells
-// (CSR, deterministic order), and the map build. Each CTA owns a tile of 8 x 8 x 8 grid nodes,
-// stages the receptor atoms of the cells within the cutoff of the tile into shared memory, and
-// every thread accumulates, for two nodes, the Vina energy of each requested ligand XS type.
+// (CSR, deterministic order), and the map build. Each CTA owns a tile of 8 x 8 x 4 grid nodes and
+// stages the receptor atoms within the cutoff of the tile's box (position, radius, flags) in shared memory;
+// each of its warps walks those within the cutoff of its 4 x 4 x 4 nodes, and every lane accumulates, for two
+// nodes, the Vina energy of each requested ligand XS type. Then the cell-packed copies of the maps.
 #include "pv_internal.h"
 #include "pv_runs.h"
 #include "pv_device.cuh"
